@@ -235,7 +235,7 @@ still_status still_compact_layer_beta(still_ctx* ctx, int32_t layer, const void*
  *   out    [nq][Hq][d] bf16
  *   scale  logit scale; 0 means 1 / sqrt(d)
  * d in {64, 128, 256}, t + S >= 1, nq * Hq / H <= 64; tensor pointers 16-byte aligned.
- * Keys are processed in chunks of 128 whose partial results are merged in a fixed order; the
+ * Keys are processed in slots whose partial results are merged in a fixed order; the
  * context's workspace holds the partials (grown on demand), so calls that share a context (this
  * one and the compaction calls) must be ordered on one stream or otherwise serialised. */
 still_status still_attend_biased(still_ctx* ctx, const void* q, int32_t nq, int32_t Hq,

@@ -70,8 +70,12 @@ struct DecodeStack {
   DecodeArgs layer[kDecodeMaxLayers];
   int32_t n = 0;
 };
-size_t decode_workspace_bytes(int64_t rows, int64_t entries, int d, int layers = 1);
-cudaError_t launch_decode_biased(const DecodeStack& st, void* ws, int num_sms, cudaStream_t s);
+// Slots that the entries of a KV-head are split into (each slot's partial is merged in order).
+int decode_slots(int64_t entries, int H, int num_sms);
+size_t decode_workspace_bytes(int64_t rows, int nslots, int d, int layers);
+// Entry pitches of both parts are equal (a.cst = a.fst). launches: kernels launched.
+cudaError_t launch_decode_biased(const DecodeStack& st, void* ws, int num_sms, cudaStream_t s,
+                                 int* launches);
 
 // Converts n bf16 values to fp16 in place (exact within the fp16 range; values below it
 // become fp16 subnormals, absolute error <= 2^-25).

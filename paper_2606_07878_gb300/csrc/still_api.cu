@@ -1613,12 +1613,14 @@ still_status attend_biased_impl(still_ctx* ctx, int32_t n_layers, const void* co
     a.scale = scale > 0.f ? scale : 1.f / std::sqrt((float)d);
   }
   CK(cudaSetDevice(ctx->device));
-  TRY(ensure_ws(ctx, decode_workspace_bytes((int64_t)nq * Hq, t + S, d, n_layers)));
+  TRY(ensure_ws(ctx, decode_workspace_bytes((int64_t)nq * Hq, decode_slots(t + S, H, ctx->nsm), d,
+                                            n_layers)));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   ctx->prof.begin(STILL_K_DECODE, s);
-  cudaError_t r = launch_decode_biased(st, ctx->ws, ctx->nsm, s);
+  int launches = 0;
+  cudaError_t r = launch_decode_biased(st, ctx->ws, ctx->nsm, s, &launches);
   ctx->prof.end(STILL_K_DECODE, s);
-  ctx->prof.launches[STILL_K_DECODE] += 1;  // the merge kernel (begin counted the first)
+  ctx->prof.launches[STILL_K_DECODE] += launches - 1;  // begin counted the first
   if (r != cudaSuccess) return STILL_ERR_CUDA;
   return STILL_OK;
 }
