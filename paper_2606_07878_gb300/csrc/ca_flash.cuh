@@ -637,26 +637,8 @@ inline cudaError_t launch_ca_flash(const Operand2D& Q, const Operand2D& K, const
   auto kern = ca_flash_kernel<D2, EX>;
   static thread_local int clusters = 0;  // resident CTA pairs (per instantiation)
   if (clusters == 0) {
-    cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kBytes);
+    const cudaError_t e = resident_pairs(kern, kFlashThreads, S::kBytes, num_sms, &clusters);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t q = {};
-    q.gridDim = dim3(2 * std::max(1, num_sms / 2), 1, 1);
-    q.blockDim = dim3(kFlashThreads, 1, 1);
-    q.dynamicSmemBytes = S::kBytes;
-    cudaLaunchAttribute qa[1];
-    qa[0].id = cudaLaunchAttributeClusterDimension;
-    qa[0].val.clusterDim.x = 2;
-    qa[0].val.clusterDim.y = 1;
-    qa[0].val.clusterDim.z = 1;
-    q.attrs = qa;
-    q.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kern, &q) != cudaSuccess || n < 1) {
-      cudaGetLastError();
-      n = num_sms / 2;
-    }
-    clusters = std::max(1, std::min(n, num_sms / 2));
   }
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(kFlashThreads, 1, 1);

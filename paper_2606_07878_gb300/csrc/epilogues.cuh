@@ -56,6 +56,17 @@ __device__ __forceinline__ void split_pack_f16(float a, float b, uint32_t& hi, u
   lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
+// The same of a packed fp32 pair, in fp16 or bf16.
+template <bool F16>
+__device__ __forceinline__ void split2(uint64_t v, uint32_t& hi, uint32_t& lo) {
+  float a, b;
+  unpack2(v, a, b);
+  if constexpr (F16)
+    split_pack_f16(a, b, hi, lo);
+  else
+    split_pack(a, b, hi, lo);
+}
+
 // 32 floats -> 32 bf16 packed in 4 x uint4
 __device__ __forceinline__ void pack_bf16x32(const float (&v)[32], uint4 (&o)[4]) {
 #pragma unroll
@@ -111,7 +122,6 @@ __device__ __forceinline__ void pack_f32x16(const float* v, uint4 (&o)[4]) {
 struct EpiAffine {
   static constexpr int kWarps = 8;  // two per lane quarter: alternating 32-column chunks
   static constexpr int kStages = 0;  // default pipeline depth
-  static constexpr int kStoreBufs = 1;
   int32_t kind = OUT_F32;
   void* out = nullptr;
   int64_t lo_off = 0;  // OUT_HILO: lo element offset from hi
@@ -347,18 +357,7 @@ __device__ __forceinline__ double seg_position(const PosSegs& s, int64_t idx) {
   return s.start[k] + (double)(idx - s.begin[k]) * s.step[k];
 }
 
-// Key projection epilogue (cross-attention keys):
-//   k~ = acc + b_K;  sumsq(token, head) += |k~|^2;  k = RoPE_c(k~, p_n)  -> hi/lo bf16.
-// Columns are in "pair-chunk" order: within each 256-column tile, columns [0,128) hold the
-// first elements of 128 RoPE pairs and [128,256) their partners, so a tile owns whole pairs.
-// The angle p_n * omega_m is split as G_g * omega_m + i * omega_m + f * omega_m with
-// delta = p_n - G_g in [0, kPosGrain), i = floor(delta) and f = delta - i: the first two
-// rotations come from tables built per call in fp64 (coarse[g], fine[i]), the third (only for
-// fractional positions, |f * omega_m| < 1) from Taylor series; the three are combined by the
-// angle-addition formulas. Every rotation is thus accurate to fp32 rounding; forming
-// delta * omega_m in fp32 instead would leave angle errors near 2e-6 rad at delta ~ 31. The
-// per-token (g, delta) come from a table formed once per call in fp64 (gd[n] = (g, delta)), so
-// the epilogue itself does no fp64 arithmetic.
+// Positions between two rows of the coarse compactor-RoPE table (see keyproj.cuh).
 constexpr int kPosGrain = 32;
 
 // sin and cos of |x| <= 1 from their Taylor series about 0, through x^11 and x^12 (the first
@@ -381,156 +380,6 @@ __device__ __forceinline__ void sincos_taylor(float x, float* s, float* c) {
   *c = fmaf(pc, -x2, 1.f);
 }
 
-// kFrac: some key positions are fractional (the sub-unit rotation is compiled in only then,
-// so the integer-position kernel keeps its registers).
-template <bool kFrac>
-struct EpiRopeCT {
-  // Element-wise heavy and MMA-light (K = 3d): four warps per lane quarter, each owning 32 of
-  // the tile's 128 pairs, processed 16 at a time; a short pipeline suffices.
-  static constexpr int kWarps = 16;
-  static constexpr int kParts = kWarps / 4;
-  static constexpr int kPairsPerPart = 128 / kParts;  // RoPE pairs of a tile per warp
-  static constexpr int kStages = 3;
-  static constexpr int kStoreBufs = 1;  // 4 KB TMA-store staging buffers per warp
-  __nv_bfloat16* out = nullptr;  // [H][n][N][2D]: hi at [0, D), lo at [D, 2D) (via the TMA view)
-  float* sumsq = nullptr;        // [H][n][kParts * D / 256][N] partial sums of |k~|^2 (part-major)
-  const float* bias = nullptr;   // [n*D], pair-chunk order
-  const float2* coarse = nullptr;  // [G][D/2]: (cos, sin)(G_g * omega_m)
-  // [D/2][kPosGrain]: (cos, sin)(i * omega_m), i fastest: the 32 consecutive tokens of a warp
-  // read 32 neighbouring entries of one pair's row (one 256-byte span per load)
-  const float2* fine = nullptr;
-  const float* omega = nullptr;    // [D/2] fp32
-  const float2* gd = nullptr;      // [Ntok]: (coarse index g as float, delta)
-  int32_t fp16 = 0;                // hi / lo as fp16 (about 22 bits) instead of bf16
-  int32_t D = 0, nheads = 0, ncoarse = 0;
-  int64_t Ntok = 0;
-  int32_t tile_cols_ = 256;  // must be 256: a tile holds 128 whole RoPE pairs
-
-  __device__ void prefetch(const GemmParams&, const TileCoord&, int, int) const {}
-
-  __device__ void operator()(const GemmParams& p, const TileCoord& tc, int row, uint32_t taddr,
-                             int half, uint4* stage, const CUtensorMap* tmc) const {
-    const int r = tc.tm * kBM + row;
-    const bool rvalid = r < p.M;
-    const int lane = threadIdx.x & 31;
-    const int row0 = tc.tm * kBM + row - lane;  // first token row of this warp
-    const int c_tile = tc.tn * 256;
-    const int head = c_tile / D;
-    const int f_tile = c_tile % D;       // column of this tile inside the head (pair-chunk order)
-    const int m_base = (f_tile / 256) * 128;  // first pair index of this tile
-    const float2 gdr = rvalid ? gd[r] : make_float2(0.f, 0.f);
-    const int g = max(0, min((int)gdr.x, ncoarse - 1));
-    const int di = max(0, min((int)gdr.y, kPosGrain - 1));
-    const float frac = gdr.y - (float)di;  // exact; 0 for integer positions
-    const bool any_frac = kFrac && __any_sync(0xffffffffu, frac != 0.f);
-    float ss = 0.f;
-    // Part p owns pairs [p, p + 1) * kPairsPerPart of the tile, 16 at a time. With kStoreBufs = 2 the
-    // staging area holds two 4 KB buffers used alternately, so one iteration's TMA stores can
-    // still be reading while the next fills the other buffer.
-    for (int it = 0; it < kPairsPerPart / 16; ++it) {
-      const int u = kPairsPerPart * half + 16 * it;
-      // tables first: their latency overlaps the TMEM loads
-      const float4* crow = reinterpret_cast<const float4*>(coarse + (int64_t)g * (D / 2) + m_base + u);
-      const float2* fcol = fine + (int64_t)(m_base + u) * kPosGrain + di;
-      const float4* om4 = reinterpret_cast<const float4*>(omega + m_base + u);
-      const float4* ba4 = reinterpret_cast<const float4*>(bias + c_tile + u);
-      const float4* bb4 = reinterpret_cast<const float4*>(bias + c_tile + 128 + u);
-      float4 w[4], xa[4], xb[4], cs[8];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        w[q] = any_frac ? om4[q] : make_float4(0.f, 0.f, 0.f, 0.f);
-        xa[q] = ba4[q];
-        xb[q] = bb4[q];
-        cs[2 * q] = crow[2 * q];
-        cs[2 * q + 1] = crow[2 * q + 1];
-      }
-      float a[16], bb[16];
-      tmem_ld16x2(taddr + (uint32_t)u, taddr + (uint32_t)(128 + u), a, bb);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float ws[4] = {w[q].x, w[q].y, w[q].z, w[q].w};
-        const float bas[4] = {xa[q].x, xa[q].y, xa[q].z, xa[q].w};
-        const float bbs[4] = {xb[q].x, xb[q].y, xb[q].z, xb[q].w};
-        const float cc[4] = {cs[2 * q].x, cs[2 * q].z, cs[2 * q + 1].x, cs[2 * q + 1].z};
-        const float sc[4] = {cs[2 * q].y, cs[2 * q].w, cs[2 * q + 1].y, cs[2 * q + 1].w};
-        float cf[4], sf[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float2 f = fcol[(4 * q + k) * kPosGrain];  // small table: L1-resident
-          cf[k] = f.x;
-          sf[k] = f.y;
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int e = 4 * q + k;
-          const float x = a[e] + bas[k];
-          const float y = bb[e] + bbs[k];
-          ss += x * x + y * y;
-          float cw = cc[k] * cf[k] - sc[k] * sf[k];  // cos(G w + i w)
-          float sw = sc[k] * cf[k] + cc[k] * sf[k];  // sin(G w + i w)
-          if (any_frac) {  // + f w, |f w| < 1
-            float s3, c3;
-            sincos_taylor(frac * ws[k], &s3, &c3);
-            const float c2 = cw * c3 - sw * s3;
-            sw = sw * c3 + cw * s3;
-            cw = c2;
-          }
-          a[e] = x * cw - y * sw;
-          bb[e] = x * sw + y * cw;
-        }
-      }
-      // Four boxes of 32 rows x 16 bf16 (hi a, lo a, hi b, lo b), 1 KB each, stored by TMA;
-      // rows past N are clipped by the copy engine.
-      uint4* box = stage + (kStoreBufs == 2 ? (it & 1) * 256 : 0);
-      if (lane == 0) {
-        if (kStoreBufs == 2)
-          bulk_wait_read1();
-        else
-          bulk_wait_read();
-      }
-      __syncwarp();
-      uint4* bl = box + lane * 2;
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        uint32_t h[4], l[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          if (fp16)
-            split_pack_f16(a[8 * q + 2 * k], a[8 * q + 2 * k + 1], h[k], l[k]);
-          else
-            split_pack(a[8 * q + 2 * k], a[8 * q + 2 * k + 1], h[k], l[k]);
-        }
-        bl[q] = make_uint4(h[0], h[1], h[2], h[3]);
-        bl[64 + q] = make_uint4(l[0], l[1], l[2], l[3]);
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (fp16)
-            split_pack_f16(bb[8 * q + 2 * k], bb[8 * q + 2 * k + 1], h[k], l[k]);
-          else
-            split_pack(bb[8 * q + 2 * k], bb[8 * q + 2 * k + 1], h[k], l[k]);
-        bl[128 + q] = make_uint4(h[0], h[1], h[2], h[3]);
-        bl[192 + q] = make_uint4(l[0], l[1], l[2], l[3]);
-      }
-      fence_proxy_async_smem();
-      __syncwarp();
-      if (lane == 0) {
-        const int z = tc.b * nheads + head;
-        const int x = f_tile + u;
-        tma_store_3d(tmc, box, x, row0, z);
-        tma_store_3d(tmc, box + 64, D + x, row0, z);
-        tma_store_3d(tmc, box + 128, x + 128, row0, z);
-        tma_store_3d(tmc, box + 192, D + x + 128, row0, z);
-        bulk_commit();
-      }
-    }
-    if (rvalid) {
-      const int parts = kParts * (D / 256);
-      sumsq[((int64_t)(tc.b * nheads + head) * parts + (f_tile / 256) * kParts + half) * Ntok + r] =
-          ss;
-    }
-  }
-};
-
 // Output heads: columns [0, d) = Z_out W_key, re-rotated by the base RoPE at the output
 // position of latent j; columns [d, 2d) = Z_out W_val. Rows r = h * t + j. bf16 stores into
 // the caller's C_k / C_v with element strides (st, sh). rot[j][m] = (cos, sin)(p_j * omega_m),
@@ -542,7 +391,6 @@ struct EpiRopeCT {
 struct EpiQuad {
   static constexpr int kWarps = 8;   // two per lane quarter: alternating 32-column chunks
   static constexpr int kStages = 0;
-  static constexpr int kStoreBufs = 1;
   float* part = nullptr;
   const __nv_bfloat16* xt = nullptr;  // x~ rows [hi | lo], pitch 2 Kp, of the group's first KV-head
   int64_t Ntok = 0;
@@ -586,7 +434,6 @@ struct EpiQuad {
 struct EpiHeads {
   static constexpr int kWarps = 8;
   static constexpr int kStages = 0;
-  static constexpr int kStoreBufs = 1;
   __nv_bfloat16* ck = nullptr;
   __nv_bfloat16* cv = nullptr;
   int64_t st = 0, sh = 0;  // element strides of [t, H, d]; d is contiguous, rows 16-B aligned

@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(256) strip_kernel(KVSource src, int64_t N, int
                                                     int rope_fix, int vec, int x16, int Kp,
                                                     __nv_bfloat16* __restrict__ X,
                                                     __half* __restrict__ XT, int64_t Np,
-                                                    float2* __restrict__ gd, double pmin, int G) {
+                                                    float2* __restrict__ gd, double origin, int G) {
   extern __shared__ __align__(16) uint8_t sm[];
   __shared__ double tpos[kStripTok];
   const int half = d / 2;
@@ -69,12 +69,12 @@ __global__ void __launch_bounds__(256) strip_kernel(KVSource src, int64_t N, int
   if (threadIdx.x < kStripTok) {
     // token position (fp64) once per token; also the compactor-RoPE coarse index and residual
     const int64_t n = n0 + threadIdx.x;
-    const double pos = n < N ? seg_position(segs, n) : pmin;
+    const double pos = n < N ? seg_position(segs, n) : origin;
     tpos[threadIdx.x] = pos;
     if (n < N) {
-      int g = (int)floor((pos - pmin) / (double)kPosGrain);
+      int g = (int)floor((pos - origin) / (double)kPosGrain);
       g = max(0, min(g, G - 1));
-      gd[n] = make_float2((float)g, (float)(pos - (pmin + (double)g * kPosGrain)));
+      gd[n] = make_float2((float)g, (float)(pos - (origin + (double)g * kPosGrain)));
     }
   }
   __syncthreads();
@@ -218,22 +218,26 @@ __global__ void __launch_bounds__(256) strip_kernel(KVSource src, int64_t N, int
   }
 }
 
-// Rows [0, G): coarse[g][m] = (cos, sin)((pmin + g * kPosGrain) * w_m); then, in the next
-// kPosGrain * D/2 entries, fine[m][i] = (cos, sin)(i * w_m). Angles formed and reduced in fp64.
-__global__ void rope_tables_kernel(float2* coarse, float* omega, int G, int D, double pmin,
+// Compactor-RoPE tables of (cos, cos, sin, sin) of two neighbouring pairs 2 q and 2 q + 1: rows
+// [0, G) hold coarse[g][q] at (origin + g * kPosGrain) * w_m, then, in the next kPosGrain * D/4
+// entries, fine[q][i] at i * w_m. Angles formed and reduced in fp64.
+__global__ void rope_tables_kernel(float4* coarse, float* omega, int G, int D, double origin,
                                    const double* __restrict__ omega_c) {
-  const int half = D / 2;
+  const int quarter = D / 4;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (int64_t)(G + kPosGrain) * half) return;
-  const int g = (int)(idx / half);
-  const int64_t f = idx - (int64_t)G * half;  // index into the fine table when >= 0
-  const int m = g < G ? (int)(idx % half) : (int)(f / kPosGrain);
-  const double w = omega_c[m];
-  float s, c;
-  const double ang = g < G ? (pmin + (double)g * kPosGrain) * w : (double)(f % kPosGrain) * w;
-  sincos_reduced(ang, &s, &c);
-  coarse[idx] = make_float2(c, s);
-  if (g == 0) omega[m] = (float)w;
+  if (idx >= (int64_t)(G + kPosGrain) * quarter) return;
+  const int g = (int)(idx / quarter);
+  const int64_t f = idx - (int64_t)G * quarter;  // index into the fine table when >= 0
+  const int q = g < G ? (int)(idx % quarter) : (int)(f / kPosGrain);
+  float s[2], c[2];
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const double w = omega_c[2 * q + e];
+    const double ang = g < G ? (origin + (double)g * kPosGrain) * w : (double)(f % kPosGrain) * w;
+    sincos_reduced(ang, &s[e], &c[e]);
+    if (g == 0) omega[2 * q + e] = (float)w;
+  }
+  coarse[idx] = make_float4(c[0], c[1], s[0], s[1]);
 }
 
 // rot[j][m] = (cos, sin)(p_j * omega[m]), p_j = pstart + j * pstep, angle reduced in fp64;
@@ -570,13 +574,15 @@ __global__ void inv_norms_kernel(const float* __restrict__ parts, int64_t nvec, 
 }
 
 __global__ void transpose_kernel(const __nv_bfloat16* __restrict__ in, int64_t R, int64_t C,
-                                 __nv_bfloat16* __restrict__ out, int perm_D) {
+                                 __nv_bfloat16* __restrict__ out, int perm_D,
+                                 int key_rows) {
   __shared__ __nv_bfloat16 tile[32][33];
   const int64_t c0 = (int64_t)blockIdx.x * 32, r0 = (int64_t)blockIdx.y * 32;
   for (int k = threadIdx.y; k < 32; k += blockDim.y) {
     const int64_t r = r0 + k, c = c0 + threadIdx.x;
     if (r < R && c < C) {
-      const int64_t src = perm_D > 0 ? pair_chunk_src((int)c, perm_D) : c;
+      const int pos = key_rows ? key_row_source((int)c) : (int)c;
+      const int64_t src = perm_D > 0 ? pair_chunk_src(pos, perm_D) : c;
       tile[k][threadIdx.x] = in[r * C + src];
     }
   }
@@ -706,29 +712,6 @@ __device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// Packed fp32 pairs (each half rounds as the scalar operation does).
-__device__ __forceinline__ uint64_t pack2(float x, float y) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-  return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& x, float& y) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-// The two bf16 of a word as an fp32 pair (exact).
-__device__ __forceinline__ uint64_t bf16_pair(uint32_t w) {
-  return pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-}
 // Read-once data: past L1, first to leave L2.
 __device__ __forceinline__ uint4 ld_stream(const __nv_bfloat16* p) {
   return __ldcs(reinterpret_cast<const uint4*>(p));
@@ -1081,7 +1064,7 @@ cudaError_t launch_beta(const __nv_bfloat16* Z, int t, int H, int D, const float
 
 cudaError_t launch_strip(const KVSource& src, int64_t N, int H, int d, const PosSegs& segs,
                          const double* omega, int rope_fix, __nv_bfloat16* X, __half* XT,
-                         int64_t Np, float2* gd, double pmin, int G, int x16, int Kp,
+                         int64_t Np, float2* gd, double origin, int G, int x16, int Kp,
                          cudaStream_t s) {
   if (d % 16 != 0 || Np % kStripTok != 0 || (Kp != 0 && (Kp % 64 != 0 || Kp < 2 * d + 1)))
     return cudaErrorInvalidValue;
@@ -1098,7 +1081,7 @@ cudaError_t launch_strip(const KVSource& src, int64_t N, int H, int d, const Pos
     attr = true;
   }
   strip_kernel<<<(unsigned)(Np / kStripTok), 256, smem, s>>>(src, N, H, d, segs, omega, rope_fix,
-                                                             vec, x16, Kp, X, XT, Np, gd, pmin, G);
+                                                             vec, x16, Kp, X, XT, Np, gd, origin, G);
   return cudaGetLastError();
 }
 
@@ -1109,10 +1092,10 @@ cudaError_t launch_heads_rot(float2* rot, int t, int hd, double pstart, double p
   return cudaGetLastError();
 }
 
-cudaError_t launch_rope_tables(float2* coarse, float* omega, int G, int D, double pmin,
+cudaError_t launch_rope_tables(float4* coarse, float* omega, int G, int D, double origin,
                                const double* omega_c, cudaStream_t s) {
-  const int64_t n = (int64_t)(G + kPosGrain) * (D / 2);
-  rope_tables_kernel<<<blocks_for(n, 256), 256, 0, s>>>(coarse, omega, G, D, pmin, omega_c);
+  const int64_t n = (int64_t)(G + kPosGrain) * (D / 4);
+  rope_tables_kernel<<<blocks_for(n, 256), 256, 0, s>>>(coarse, omega, G, D, origin, omega_c);
   return cudaGetLastError();
 }
 
@@ -1215,9 +1198,9 @@ cudaError_t launch_inv_norms(const float* parts, int64_t nvec, int nparts, int64
 }
 
 cudaError_t launch_transpose(const __nv_bfloat16* in, int64_t R, int64_t C, __nv_bfloat16* out,
-                             int perm_D, cudaStream_t s) {
+                             int perm_D, cudaStream_t s, int key_rows) {
   dim3 grid(blocks_for(C, 32), blocks_for(R, 32));
-  transpose_kernel<<<grid, dim3(32, 8), 0, s>>>(in, R, C, out, perm_D);
+  transpose_kernel<<<grid, dim3(32, 8), 0, s>>>(in, R, C, out, perm_D, key_rows);
   return cudaGetLastError();
 }
 

@@ -24,14 +24,14 @@ struct KVSource {
 //   XT[h]    = X[h]^T as fp16 hi / lo, token-contiguous, tokens padded with zeros to Np.
 // X:  [H*N][3d] bf16.  XT: [H*2d][2*Np] fp16 (hi at [0, Np), lo at [Np, 2Np); lo rows of
 // the value half are not written). omega: [d/2] fp64 base-model frequencies theta^(-2m/d).
-// Also gd[n] = (g, p_n - (pmin + g * kPosGrain)) with g = floor((p_n - pmin) / kPosGrain)
+// Also gd[n] = (g, p_n - (origin + g * kPosGrain)) with g = floor((p_n - origin) / kPosGrain)
 // clamped to [0, G): the compactor-RoPE coarse index and residual of token n (n < N).
 // x16: X in fp16 (hi | key lo as fp16 hi / lo, values as fp16) instead of bf16.
 // Kp > 0: X rows of 2 Kp elements, [x~ hi | x~ lo] with x~ = [unRoPE(K) | V | 1 | 0 ...]
 // (the folded key path; Kp a multiple of 64, >= 2d + 1).
 cudaError_t launch_strip(const KVSource& src, int64_t N, int H, int d, const PosSegs& segs,
                          const double* omega, int rope_fix, __nv_bfloat16* X, __half* XT,
-                         int64_t Np, float2* gd, double pmin, int G, int x16, int Kp,
+                         int64_t Np, float2* gd, double origin, int G, int x16, int Kp,
                          cudaStream_t s);
 
 // Folded key projection (no compactor RoPE): Wt [n][Kp][D] bf16, rows of W~_i = [W_K,i; b_K,i]
@@ -86,10 +86,11 @@ cudaError_t launch_bf16_to_f16(void* p, int64_t n, cudaStream_t s);
 cudaError_t launch_heads_rot(float2* rot, int t, int hd, double pstart, double pstep,
                              const double* omega, int use_rope, cudaStream_t s);
 
-// Compactor-RoPE tables: coarse[g][m] = (cos, sin)((pmin + g * kPosGrain) * w_m) for g < G,
-// then fine[m][i] = (cos, sin)(i * w_m) for i < kPosGrain at coarse + G * D/2; omega[m] = w_m
-// (fp32), w_m = omega_c[m] = theta_c^(-2m/D) (fp64 table), angles reduced in fp64.
-cudaError_t launch_rope_tables(float2* coarse, float* omega, int G, int D, double pmin,
+// Compactor-RoPE tables: coarse[g][q] = (cos, cos, sin, sin) of pairs m = 2 q and 2 q + 1 at
+// (origin + g * kPosGrain) * w_m for g < G, then fine[q][i] at i * w_m for i < kPosGrain, at
+// coarse + G * D/4; omega[m] = w_m (fp32), w_m = omega_c[m] = theta_c^(-2m/D) (fp64 table),
+// angles reduced in fp64.
+cudaError_t launch_rope_tables(float4* coarse, float* omega, int G, int D, double origin,
                                const double* omega_c, cudaStream_t s);
 
 // Per-call cross-attention queries: q = RoPE_c(q^, p_j) for latents j < t, batches
@@ -136,14 +137,22 @@ cudaError_t launch_rmsnorm(const void* in, int in_bf16, int64_t rows, int D, int
 cudaError_t launch_scale_rows(float* x, const float* inv, int64_t rows, int D, cudaStream_t s);
 
 // out[c][r] = in[r][src(c)] (bf16), in is [R][C] row-major; src(c) maps pair-chunk order
-// back to natural order inside blocks of D columns when perm_D > 0.
+// back to natural order inside blocks of D columns when perm_D > 0; with key_rows, row c holds
+// pair-chunk column key_row_source(c) (the key projection's row order).
 cudaError_t launch_transpose(const __nv_bfloat16* in, int64_t R, int64_t C, __nv_bfloat16* out,
-                             int perm_D, cudaStream_t s);
+                             int perm_D, cudaStream_t s, int key_rows = 0);
 
 // out[c] = float(in[src(c)]) (bf16 -> fp32 with the same optional permutation); in2 (optional)
 // is appended after in ([in | in2]), each of length C.
 cudaError_t launch_bias(const __nv_bfloat16* in, const __nv_bfloat16* in2, int64_t C,
                         float* out, int perm_D, cudaStream_t s);
+
+// The pair-chunk column that row c of the key projection's W (accumulator column c) holds: within
+// every 32, row 8 j + 2 l + b holds column 8 l + 2 j + b (j, l < 4, b < 2).
+__host__ __device__ inline int key_row_source(int c) {
+  const int u = c & 31;
+  return (c & ~31) | (((u >> 1) & 3) << 3) | (((u >> 3) & 3) << 1) | (u & 1);
+}
 
 // Natural column index of pair-chunk column c inside a block of D columns.
 __host__ __device__ inline int pair_chunk_src(int c, int D) {

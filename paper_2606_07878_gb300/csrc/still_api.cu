@@ -26,6 +26,7 @@
 #include "gemm_host.cuh"
 #include "kernels.cuh"
 #include "ca_flash.cuh"
+#include "keyproj.cuh"
 
 using namespace still;
 
@@ -36,7 +37,7 @@ using bf16 = __nv_bfloat16;
 // One compactor block's weights in the library's layouts (App. A, "Compactor blocks").
 struct BlockW {
   bool has_ca = false;   // cross-attention in this block
-  bf16* WkT = nullptr;   // [nD][2d]  pair-chunk order
+  bf16* WkT = nullptr;   // [nD][2d]  rows in key_row_source order (pair-chunk when folded)
   float* bk = nullptr;   // [nD]      pair-chunk order
   bf16* WqT = nullptr;   // [nD][D] pair-chunk order (queries formed per call only)
   float* bq = nullptr;   // [nD]    pair-chunk order (queries formed per call only)
@@ -275,20 +276,6 @@ still_status run_gemm256(still_ctx* ctx, const Operand2D& A, const Operand2D& B,
   return run_gemm_bn<CLS, 256>(ctx, A, B, p, e, ab_fmt, s, view);
 }
 
-// The same on CTA pairs (2-SM MMAs, 256 x 256 tiles): for the key projection, whose 1-SM form
-// is bound by shared-memory traffic.
-template <int CLS, class Epi>
-still_status run_gemm256_2sm(still_ctx* ctx, const Operand2D& A, const Operand2D& B,
-                             GemmParams p, const Epi& e, int ab_fmt, cudaStream_t s,
-                             const StoreView3D* view = nullptr) {
-  p.err = ctx->err;
-  ctx->prof.begin(CLS, s);
-  cudaError_t r = launch_gemm_2sm<256, CLS>(A, B, p, e, ab_fmt, ctx->nsm, s, view);
-  ctx->prof.end(CLS, s);
-  if (r == cudaErrorInvalidValue) return STILL_ERR_INVALID_ARG;
-  return r == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
-}
-
 StoreView3D store_view(void* ptr, int elem_bytes, int64_t nx, int64_t ny, int64_t nz,
                        int64_t ystride, int64_t zstride, int bx, bool swz) {
   StoreView3D v;
@@ -379,7 +366,8 @@ bool make_plan(const still_layer_config& c, bool lazy_q, int Kp, int64_t N, int 
   P.Np = rup(N, 64);
   P.tp = rup(t, 64);
   P.ldt = rup(t, 4);
-  P.G = (int)std::floor((pmax - pmin) / kPosGrain) + 2;
+  // the table starts at most one grain before pmin (Positions::origin)
+  P.G = (int)std::floor((pmax - pmin) / kPosGrain) + 3;
   const int64_t H = P.H, d = P.d, D = P.D, n = P.n, F = P.F, T = t;
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -389,7 +377,7 @@ bool make_plan(const still_layer_config& c, bool lazy_q, int Kp, int64_t N, int 
   };
   P.oX = take(H * N * std::max<int64_t>(3 * d, 2 * Kp) * 2);  // Kp > 0: the folded x~ rows
   P.oXT = take(H * 2 * d * 2 * P.Np * 2);
-  P.oCoarse = take((size_t)(P.G + kPosGrain) * (D / 2) * 8);  // coarse rows, then fine rows
+  P.oCoarse = take((size_t)(P.G + kPosGrain) * (D / 4) * 16);  // coarse rows, then fine rows
   P.oOmega = take((D / 2) * 4);
   P.oGD = take((size_t)P.Np * 8);
   P.oHrot = take(T * (d / 2) * 8);
@@ -407,7 +395,7 @@ bool make_plan(const still_layer_config& c, bool lazy_q, int Kp, int64_t N, int 
   P.oZn = lazy_q ? take(H * T * 2 * D * 2) : 0;  // RMSNorm(Z) hi | lo for the call's t latents
   const size_t fixed = off;
   // |k~|^2 partials + inverses; the folded path needs neither k nor per-call q
-  const int64_t kparts = std::max<int64_t>(EpiRopeCT<false>::kParts * (D / 256), Kp / 32);
+  const int64_t kparts = std::max<int64_t>(kKeyParts * (D / 256), Kp / 32);
   P.kb_b = Kp > 0 ? 0 : a256(N * 2 * D * 2);
   P.kss_b = a256(N * 4 * (kparts + 1));
   P.q_b = Kp > 0 ? 0 : a256(T * 2 * D * 2);
@@ -482,6 +470,10 @@ still_status ensure_ws(still_ctx* ctx, size_t bytes) {
 struct Positions {
   PosSegs segs;
   double pmin = 0, pmax = 0;
+  // Where the coarse compactor-RoPE table starts: at most kPosGrain before pmin, and such that
+  // in the longest segment of step 1 the table's rows start at tokens whose index is a multiple
+  // of kPosGrain (the 32 tokens of a warp of the key projection then share a row).
+  double origin = 0;
   bool frac = false;  // some position is not an integer
 };
 
@@ -503,6 +495,8 @@ still_status make_positions(const still_pos_segment* h_segments, int32_t n_segme
   int64_t acc = 0;
   double lo = INFINITY, hi = -INFINITY;
   int k = 0;
+  int64_t longest = 0;
+  double phase = 0;  // position that token 0 would have in the longest segment of step 1
   for (int i = 0; i < n_segments; ++i) {
     const still_pos_segment& s = h_segments[i];
     if (s.count < 0 || !std::isfinite(s.start) || !std::isfinite(s.step))
@@ -512,6 +506,10 @@ still_status make_positions(const still_pos_segment* h_segments, int32_t n_segme
       out.frac = true;
     const double last = s.start + (double)(s.count - 1) * s.step;
     if (!std::isfinite(last)) return STILL_ERR_INVALID_ARG;
+    if (s.step == 1.0 && s.count > longest) {
+      longest = s.count;
+      phase = s.start - (double)acc;
+    }
     lo = std::min(lo, std::min(s.start, last));
     hi = std::max(hi, std::max(s.start, last));
     out.segs.begin[k] = acc;
@@ -525,6 +523,12 @@ still_status make_positions(const still_pos_segment* h_segments, int32_t n_segme
   out.segs.begin[k] = acc;
   out.pmin = lo;
   out.pmax = hi;
+  out.origin = lo;
+  if (longest > 0) {
+    // the largest phase + m * kPosGrain up to lo; exact, or left at lo (huge positions)
+    const double o = phase + std::floor((lo - phase) / kPosGrain) * kPosGrain;
+    if (o <= lo && lo - o < kPosGrain) out.origin = o;
+  }
   return STILL_OK;
 }
 
@@ -570,7 +574,7 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
 
   bf16* X = reinterpret_cast<bf16*>(ws + P.oX);
   __half* XT = reinterpret_cast<__half*>(ws + P.oXT);
-  float2* coarse = reinterpret_cast<float2*>(ws + P.oCoarse);
+  float4* coarse = reinterpret_cast<float4*>(ws + P.oCoarse);
   float* omega = reinterpret_cast<float*>(ws + P.oOmega);
   float2* gd = reinterpret_cast<float2*>(ws + P.oGD);
   float2* hrot = reinterpret_cast<float2*>(ws + P.oHrot);
@@ -584,10 +588,10 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
   void* Z3 = ws + P.oZ3;
 
   KLAUNCH(STILL_K_STRIP, launch_strip(src, N, H, d, pos.segs, L.omega_b, c.rope_fix, X, XT, Np,
-                                      gd, pos.pmin, P.G, L.f16 ? 1 : 0, fold_kp(L), s));
+                                      gd, pos.origin, P.G, L.f16 ? 1 : 0, fold_kp(L), s));
   const int w_fmt = L.f16 ? 0 : 1;    // operand format of X, RMSNorm(Z), W_K and W_Q products
   const int zn_mode = L.f16 ? 2 : 1;  // RMSNorm(Z) as fp16 or bf16 hi | lo
-  KLAUNCH(STILL_K_TABLES, launch_rope_tables(coarse, omega, P.G, D, pos.pmin, L.omega_c, s));
+  KLAUNCH(STILL_K_TABLES, launch_rope_tables(coarse, omega, P.G, D, pos.origin, L.omega_c, s));
   KLAUNCH(STILL_K_TABLES, launch_heads_rot(hrot, t, d / 2, qstart, qstep, L.omega_b, c.rope_fix, s));
   bf16* Zn = P.lazy_q ? reinterpret_cast<bf16*>(ws + P.oZn) : nullptr;
   const int64_t rows = (int64_t)H * t;
@@ -639,7 +643,7 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
     uint8_t* g = ws + P.oCA;
     bf16* kb = reinterpret_cast<bf16*>(g);
     g += P.kb_b * nbl;
-    const int kparts = L.fold ? L.Kp / 32 : EpiRopeCT<false>::kParts * (D / 256);
+    const int kparts = L.fold ? L.Kp / 32 : kKeyParts * (D / 256);
     float* kss = reinterpret_cast<float*>(g);        // [nbl][N][kparts]
     float* kinv = kss + (size_t)nbl * N * kparts;    // [nbl][N]
     g += P.kss_b * nbl;
@@ -707,37 +711,30 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
       TRY(run_gemm256<STILL_K_KEYPROJ>(ctx, op(X, (int64_t)H * N, 2 * Kp),
                                        op(L.G, (int64_t)n * Kp, 2 * Kp), p, e, 1, s));
     } else {  // keyproj: rows = tokens of heads [h0, h0+nh), columns = cross heads [i0, i0+ni)
-      GemmParams p = gp((int)N, ni * D, nh, 1);
-      p.a_r1 = N;
-      p.n_fast = 1;  // X rows of a KV-head can exceed L2; the W_K block fits
-      add_pass(p, 0, 0, (int)(h0 * N), i0 * D, 2 * d);
-      add_pass(p, 2 * d, 0, (int)(h0 * N), i0 * D, d);
-      auto fill = [&](auto& e) {
-        e.out = kb;
-        e.sumsq = kss;
-        e.bias = Bw.bk + (size_t)i0 * D;
-        e.coarse = coarse;
-        e.fine = coarse + (size_t)P.G * (D / 2);
-        e.omega = omega;
-        e.gd = gd;
-        e.D = D;
-        e.nheads = ni;
-        e.ncoarse = P.G;
-        e.fp16 = exact || tk ? 1 : 0;  // k as fp16 hi / lo (block feeding another; one pass)
-        e.Ntok = N;
-      };
-      const StoreView3D kv = store_view(kb, 2, 2 * D, N, nbl, 2 * D, N * 2 * D, 16, false);
-      const Operand2D xop = op(X, (int64_t)H * N, 3 * d);
-      const Operand2D wop = op(Bw.WkT, (int64_t)n * D, 2 * d);
-      if (pos.frac) {
-        EpiRopeCT<true> e;
-        fill(e);
-        TRY(run_gemm256_2sm<STILL_K_KEYPROJ>(ctx, xop, wop, p, e, w_fmt, s, &kv));
-      } else {
-        EpiRopeCT<false> e;
-        fill(e);
-        TRY(run_gemm256_2sm<STILL_K_KEYPROJ>(ctx, xop, wop, p, e, w_fmt, s, &kv));
-      }
+      KeyProjParams kp;
+      kp.out = kb;
+      kp.sumsq = kss;
+      kp.bias = Bw.bk + (size_t)i0 * D;
+      kp.coarse = coarse;
+      kp.fine = coarse + (size_t)P.G * (D / 4);
+      kp.omega = omega;
+      kp.gd = gd;
+      kp.N = (int)N;
+      kp.D = D;
+      kp.nh = ni;
+      kp.heads = nh;
+      kp.ncoarse = P.G;
+      kp.a_row0 = (int)(h0 * N);
+      kp.b_row0 = i0 * D;
+      kp.err = ctx->err;
+      ctx->prof.begin(STILL_K_KEYPROJ, s);
+      // k as fp16 hi | lo for a block feeding another and for one-pass scores
+      const cudaError_t r = launch_key_proj(op(X, (int64_t)H * N, 3 * d),
+                                            op(Bw.WkT, (int64_t)n * D, 2 * d), kp, d, pos.frac,
+                                            exact || tk, w_fmt, ctx->nsm, s);
+      ctx->prof.end(STILL_K_KEYPROJ, s);
+      if (r == cudaErrorInvalidValue) return STILL_ERR_INVALID_ARG;
+      if (r != cudaSuccess) return STILL_ERR_CUDA;
     }  // key projection
     // scale / |k~_n| per key (the d_l logit scale folded in)
     // A block that feeds another forms q and k as fp16 hi / lo (about 22 bits; bf16 hi / lo
@@ -1212,7 +1209,7 @@ still_status load_layer(still_ctx* ctx, int32_t layer, const still_layer_config*
       TRY(dalloc(L, &B.WkT, (size_t)nD * 2 * d));
       TRY(dalloc(L, &B.bk, (size_t)nD));
       TRY(dalloc(L, &B.WvoT, (size_t)D * 2 * n * 2 * d));
-      CK(launch_transpose(static_cast<const bf16*>(w.Wk), 2 * d, nD, B.WkT, D, s));
+      CK(launch_transpose(static_cast<const bf16*>(w.Wk), 2 * d, nD, B.WkT, D, s, L.fold ? 0 : 1));
       if (L.f16) CK(launch_bf16_to_f16(B.WkT, (int64_t)nD * 2 * d, s));
       CK(launch_bias(static_cast<const bf16*>(w.bk), nullptr, nD, B.bk, D, s));
       // W_Q and b_Q: kept when the block's queries are formed per call, else temporaries.
