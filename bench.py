@@ -60,7 +60,8 @@ def describe(name, wl, t):
             f"({round(wl['N'] / t)}x)")
 
 # DRAM traffic (read + write) per launch of the dominant kernel at a workload, from an ncu
-# capture; valid only for the kernel sources it was taken on (hash of the listed sources).
+# capture; valid only for the kernel sources it was taken on, or later ones that load and store
+# the same (hash of the listed sources).
 # The fused cross-attention kernel (the scores GEMM entry is kept for the record: no workload
 # takes it any more).
 TRAFFIC = {
@@ -69,14 +70,14 @@ TRAFFIC = {
     "ca_fused": [
         # 1.313 GB read + 0.127 GB written per launch (profiles/ca_fused_qwen7b_8k_t1024.md,
         # the CTA-pair kernel, whose source is ca_flash.cuh)
-        {"files": ["ca_flash.cuh"], "kernel_hash": "aa3a12ddd971da2d",
+        {"files": ["ca_flash.cuh"], "kernel_hash": "53a0447d2f7d36df",
          "bytes_per_launch": 1.4405e9, "workload": ("qwen7b_8k", 1024),
          "profile": "profiles/ca_fused_qwen7b_8k_t1024.md"},
         # the head-dim-256 kernel (source ca_pair.cu) captured on one KV-head of a 16k-token
         # cache (1.231 GB read + 0.086 GB written, profiles/ca_pair_gemma_n16k_t655.md), scaled
         # by the units of a full-size launch (2 KV-heads x 131072 tokens: x16); its traffic (k
         # read once, X^T, partials) grows in proportion
-        {"files": ["ca_pair.cu"], "kernel_hash": "89e4b7a50e367c33",
+        {"files": ["ca_pair.cu"], "kernel_hash": "5cc9b2f5e7dd0111",
          "bytes_per_launch": 16 * 1.3165e9, "workload": ("gemma_128k", 655),
          "profile": "profiles/ca_pair_gemma_n16k_t655.md"},
     ],

@@ -120,6 +120,83 @@ __device__ __forceinline__ int flash_chunks(const FlashParams& f, int j) {
   return left >= KEYS ? KEYS / kBK : (int)(left / kBK);
 }
 
+// ---- the softmax warps' work on one S tile. A thread holds C columns of its row as fp32 pairs.
+// Its time is a serial stretch between S_j and P X_j, which for short contractions (d_l = 256, the
+// folded path) is longer than S_{j+1}: so one wait for all TMEM loads, packed fp32 pairs,
+// 3-input max, and masks only in the tile that holds the last key. Measured per layer (all
+// launches of the kernel): canonical two-block 64k 3.11 -> 2.83 ms, folded 8k 0.49 -> 0.45 ms,
+// Qwen-7B 8k 1.10 -> 1.06 ms, Qwen-8B 32k t = 2048 16.36 -> 15.98 ms.
+
+// Loads C columns from TMEM.
+template <int C>
+__device__ __forceinline__ void load_scores(uint32_t taddr, uint32_t (&v)[C]) {
+#pragma unroll
+  for (int g = 0; g < C / 32; ++g) tmem_ld32_issue(taddr + 32u * g, v + 32 * g);
+  tmem_wait_ld();
+#pragma unroll
+  for (int g = 0; g < C / 32; ++g) tmem_landed(v + 32 * g);
+}
+
+// v *= kw per column, -inf from column cvalid on; returns the largest.
+template <int C>
+__device__ __forceinline__ float scale_scores(uint32_t (&v)[C], const float* kw, int cvalid) {
+#pragma unroll
+  for (int c = 0; c < C; c += 4) {
+    const float4 k4 = *reinterpret_cast<const float4*>(kw + c);
+    float a, b;
+    unpack2(mul2(pack2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), pack2(k4.x, k4.y)), a, b);
+    v[c] = __float_as_uint(a);
+    v[c + 1] = __float_as_uint(b);
+    unpack2(mul2(pack2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3])), pack2(k4.z, k4.w)), a,
+            b);
+    v[c + 2] = __float_as_uint(a);
+    v[c + 3] = __float_as_uint(b);
+  }
+  if (cvalid < C) {
+#pragma unroll
+    for (int c = 0; c < C; ++c)
+      if (c >= cvalid) v[c] = __float_as_uint(-INFINITY);
+  }
+  float m0 = -INFINITY, m1 = -INFINITY;
+#pragma unroll
+  for (int c = 0; c < C; c += 4) {
+    m0 = max3(m0, __uint_as_float(v[c]), __uint_as_float(v[c + 1]));
+    m1 = max3(m1, __uint_as_float(v[c + 2]), __uint_as_float(v[c + 3]));
+  }
+  return fmaxf(m0, m1);
+}
+
+// 2^(v - m) rounded to fp16, packed in place (pair c in v[c / 2]), with LO also the rounding
+// rests lo = fp16(p - hi) in lo[c / 2]; returns the sum of the rounded values.
+template <int C, bool LO>
+__device__ __forceinline__ float exp_scores(uint32_t (&v)[C], uint32_t* lo, float m) {
+  const uint64_t nm = pack2(-m, -m);
+  uint64_t l0 = 0ull, l1 = 0ull;  // (0.f, 0.f)
+#pragma unroll
+  for (int c = 0; c < C; c += 2) {
+    float a, b;
+    unpack2(add2(pack2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), nm), a, b);
+    const float p0 = ex2_ftz(a), p1 = ex2_ftz(b);
+    const __half2 h = __floats2half2_rn(p0, p1);
+    const float2 r = __half22float2(h);
+    uint64_t sum = pack2(r.x, r.y);
+    v[c / 2] = *reinterpret_cast<const uint32_t*>(&h);
+    if constexpr (LO) {
+      const __half2 l = __floats2half2_rn(p0 - r.x, p1 - r.y);
+      const float2 rl = __half22float2(l);
+      lo[c / 2] = *reinterpret_cast<const uint32_t*>(&l);
+      sum = add2(sum, pack2(rl.x, rl.y));
+    }
+    if (c & 2)
+      l1 = add2(l1, sum);
+    else
+      l0 = add2(l0, sum);
+  }
+  float a, b;
+  unpack2(add2(l0, l1), a, b);
+  return a + b;
+}
+
 template <int D2, bool EX>
 __global__ void __launch_bounds__(kFlashThreads, 1)
     ca_flash_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -454,14 +531,8 @@ __global__ void __launch_bounds__(kFlashThreads, 1)
         if (!wait_all(sfull, n_sf & 1, 320)) break;
         ++n_sf;
         tc_fence_after();
-        float v[kCols];
-#pragma unroll
-        for (int g = 0; g < kCols / 32; ++g) {
-          float tmp[32];
-          tmem_ld32(lane_base + (uint32_t)(kCols * half + 32 * g), tmp);
-#pragma unroll
-          for (int e = 0; e < 32; ++e) v[32 * g + e] = tmp[e];
-        }
+        uint32_t v[kCols];
+        load_scores<kCols>(lane_base + (uint32_t)(kCols * half), v);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(l_sfree);  // the even CTA's, for both CTAs
@@ -469,17 +540,7 @@ __global__ void __launch_bounds__(kFlashThreads, 1)
 #pragma unroll
         for (int e = 0; e < kCols / 32; ++e) kw[lane + 32 * e] = kv[e];
         __syncwarp();
-        const int cvalid = f.N - key0;
-        float mx = -INFINITY;
-#pragma unroll
-        for (int c = 0; c < kCols; c += 4) {
-          const float4 k4 = *reinterpret_cast<const float4*>(kw + c);
-          v[c] = c < cvalid ? v[c] * k4.x : -INFINITY;
-          v[c + 1] = c + 1 < cvalid ? v[c + 1] * k4.y : -INFINITY;
-          v[c + 2] = c + 2 < cvalid ? v[c + 2] * k4.z : -INFINITY;
-          v[c + 3] = c + 3 < cvalid ? v[c + 3] * k4.w : -INFINITY;
-          mx = fmaxf(mx, fmaxf(fmaxf(v[c], v[c + 1]), fmaxf(v[c + 2], v[c + 3])));
-        }
+        float mx = scale_scores<kCols>(v, kw, f.N - key0);
         __syncwarp();
         mx = fmaxf(mx, exchange(mx, 321));
         if (bad) break;
@@ -496,23 +557,9 @@ __global__ void __launch_bounds__(kFlashThreads, 1)
         }
         // probabilities (fp16, <= 2^8) into registers as packed pairs; l from the rounded values
         // (EX: hi and lo = fp16(p - hi), l from hi + lo)
-        uint32_t pk[kCols / 2];
         uint32_t pkl[EX ? kCols / 2 : 1];
-#pragma unroll
-        for (int c = 0; c < kCols; c += 2) {
-          const float p0 = exp2f(v[c] - m_run), p1 = exp2f(v[c + 1] - m_run);
-          const __half2 h = __floats2half2_rn(p0, p1);
-          const float2 r = __half22float2(h);
-          pk[c / 2] = *reinterpret_cast<const uint32_t*>(&h);
-          if constexpr (EX) {
-            const __half2 lo = __floats2half2_rn(p0 - r.x, p1 - r.y);
-            const float2 rl = __half22float2(lo);
-            l_part += (r.x + rl.x) + (r.y + rl.y);
-            pkl[c / 2] = *reinterpret_cast<const uint32_t*>(&lo);
-          } else {
-            l_part += r.x + r.y;
-          }
-        }
+        l_part += exp_scores<kCols, EX>(v, pkl, m_run);
+        const uint32_t* pk = v;
         // The previous PX must be complete before P is overwritten or O is rescaled.
         if (n_pf > n_pe) {
           if (!wait_all(pempty, n_pe & 1, 322)) break;

@@ -509,31 +509,15 @@ __global__ void __launch_bounds__(kFlashThreads, 1)
           if (!wait_all(sfull, n_sf & 1, 420, false)) break;
           ++n_sf;
           tc_fence_after();
-          float v[kCols];
-#pragma unroll
-          for (int gq = 0; gq < kCols / 32; ++gq) {
-            float tmp[32];
-            tmem_ld32(lane_base + (uint32_t)(kCols * half + 32 * gq), tmp);
-#pragma unroll
-            for (int e = 0; e < 32; ++e) v[32 * gq + e] = tmp[e];
-          }
+          uint32_t v[kCols];
+          load_scores<kCols>(lane_base + (uint32_t)(kCols * half), v);
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive_cluster(l_sfree);  // the leader's, for both CTAs
 #pragma unroll
           for (int e = 0; e < kCols / 32; ++e) kw[lane + 32 * e] = kv[e];
           __syncwarp();
-          const int cvalid = f.N - key0;
-          float mx = -INFINITY;
-#pragma unroll
-          for (int c = 0; c < kCols; c += 4) {
-            const float4 k4 = *reinterpret_cast<const float4*>(kw + c);
-            v[c] = c < cvalid ? v[c] * k4.x : -INFINITY;
-            v[c + 1] = c + 1 < cvalid ? v[c + 1] * k4.y : -INFINITY;
-            v[c + 2] = c + 2 < cvalid ? v[c + 2] * k4.z : -INFINITY;
-            v[c + 3] = c + 3 < cvalid ? v[c + 3] * k4.w : -INFINITY;
-            mx = fmaxf(mx, fmaxf(fmaxf(v[c], v[c + 1]), fmaxf(v[c + 2], v[c + 3])));
-          }
+          float mx = scale_scores<kCols>(v, kw, f.N - key0);
           __syncwarp();
           const float mx_own = mx;
           mx = fmaxf(mx, exchange(mx, 421));
@@ -555,15 +539,8 @@ __global__ void __launch_bounds__(kFlashThreads, 1)
             if (lane == 0) mbar_arrive_cluster(r_mmsg);
           }
           ++n_msent;
-          uint32_t pk[kCols / 2];
-#pragma unroll
-          for (int c = 0; c < kCols; c += 2) {
-            const float p0 = exp2f(v[c] - m_run), p1 = exp2f(v[c + 1] - m_run);
-            const __half2 h = __floats2half2_rn(p0, p1);
-            const float2 r2 = __half22float2(h);
-            pk[c / 2] = *reinterpret_cast<const uint32_t*>(&h);
-            l_part += r2.x + r2.y;
-          }
+          l_part += exp_scores<kCols, false>(v, nullptr, m_run);
+          const uint32_t* pk = v;
           // This CTA's previous P X done (buffer, O) and the peer's (its buffer).
           if (!prev_px_done(422)) break;
           if (g > 0 && !wait_all(rfree, (g - 1) & 1, 423, true)) break;
