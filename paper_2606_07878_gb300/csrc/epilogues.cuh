@@ -150,14 +150,19 @@ struct EpiAffine {
   // are clipped by the copy engine.
   int32_t tma_f32 = 0;
   int32_t tile_cols_ = 256;  // the tile width BN, set by the launcher
+  // sums of squares have one slot per half tile: their chunks stay in one CTA
+  bool can_split() const { return sumsq == nullptr; }
+  static constexpr bool kAnyTile = true;  // its 32-column chunks are independent
 
   // The residual rows of this warp's columns are pulled into L2 while the main loop runs.
-  __device__ void prefetch(const GemmParams& p, const TileCoord& tc, int row, int half) const {
+  template <class Src>
+  __device__ void prefetch(const GemmParams& p, const TileCoord& tc, int row, const Src& src,
+                           int half) const {
     if (res_kind == 0 || tc.split != 0) return;
     const int r = tc.tm * kBM + row;
     if (r >= p.M) return;
     const int esz = res_kind == 1 ? 4 : 2;
-    for (int cc = 32 * half; cc < tile_cols_; cc += 64) {
+    for (int cc = src.first(half); cc < tile_cols_; cc += src.step()) {
       const int c0 = tc.tn * tile_cols_ + cc;
       if (c0 >= p.N) break;
       const char* base = static_cast<const char*>(res) + resm.at(tc.b, r, c0) * esz;
@@ -165,18 +170,19 @@ struct EpiAffine {
     }
   }
 
-  __device__ void operator()(const GemmParams& p, const TileCoord& tc, int row, uint32_t taddr,
+  template <class Src>
+  __device__ void operator()(const GemmParams& p, const TileCoord& tc, int row, const Src& src,
                              int half, uint4* stage, const CUtensorMap* tmc) const {
     const int r = tc.tm * kBM + row;
     const bool rvalid = r < p.M;
     float rscale = alpha;
     if (row_scale != nullptr && rvalid) rscale *= row_scale[rsm.at(tc.b, r, 0)];
     float ss = 0.f;
-    for (int cc = 32 * half; cc < tile_cols_; cc += 64) {
-      float v[32];
-      tmem_ld32(taddr + (uint32_t)cc, v);
+    for (int cc = src.first(half); cc < tile_cols_; cc += src.step()) {
       const int c0 = tc.tn * tile_cols_ + cc;
       if (c0 >= p.N) continue;  // uniform across the warp
+      float v[32];
+      src.load(cc, v);
       const int nv = min(32, p.N - c0);
 #pragma unroll
       for (int e = 0; e < 32; ++e) v[e] *= rscale;
@@ -219,15 +225,16 @@ struct EpiAffine {
         continue;
       }
       if (col_scale != nullptr) {
-        const float* cs = col_scale + csm.at(tc.b, 0, c0);
+        float cs[32];
+        load_cols(col_scale + csm.at(tc.b, 0, c0), nv, 1.f, cs);
 #pragma unroll
-        for (int e = 0; e < 32; ++e)
-          if (e < nv) v[e] *= cs[e];
+        for (int e = 0; e < 32; ++e) v[e] *= cs[e];
       }
       if (bias != nullptr) {
+        float add[32];
+        load_cols(bias + c0, nv, 0.f, add);
 #pragma unroll
-        for (int e = 0; e < 32; ++e)
-          if (e < nv) v[e] += bias[c0 + e];
+        for (int e = 0; e < 32; ++e) v[e] += add[e];
       }
       if (sumsq != nullptr) {
 #pragma unroll
@@ -265,6 +272,24 @@ struct EpiAffine {
       const int slot = ((c_tile % ss_seg) / tile_cols_) * 2 + half;
       const int64_t vec = ssm.at(tc.b, r, c_tile / ss_seg);
       sumsq[(vec / ss_block) * ss_parts * ss_block + slot * ss_block + vec % ss_block] = ss;
+    }
+  }
+
+  // 32 values of a per-column vector (the same in every lane), `fill` past the nv valid ones.
+  static __device__ __forceinline__ void load_cols(const float* src, int nv, float fill,
+                                                   float (&o)[32]) {
+    if (nv == 32 && (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const float4 x = reinterpret_cast<const float4*>(src)[q];
+        o[4 * q] = x.x;
+        o[4 * q + 1] = x.y;
+        o[4 * q + 2] = x.z;
+        o[4 * q + 3] = x.w;
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 32; ++e) o[e] = e < nv ? src[e] : fill;
     }
   }
 
@@ -396,19 +421,23 @@ struct EpiQuad {
   int64_t Ntok = 0;
   int32_t Kp = 0;
   int32_t tile_cols_ = 256;
+  bool can_split() const { return true; }
+  static constexpr bool kAnyTile = true;
 
-  __device__ void prefetch(const GemmParams&, const TileCoord&, int, int) const {}
+  template <class Src>
+  __device__ void prefetch(const GemmParams&, const TileCoord&, int, const Src&, int) const {}
 
-  __device__ void operator()(const GemmParams& p, const TileCoord& tc, int row, uint32_t taddr,
+  template <class Src>
+  __device__ void operator()(const GemmParams& p, const TileCoord& tc, int row, const Src& src,
                              int half, uint4*, const CUtensorMap*) const {
     const int r = tc.tm * kBM + row;
     const bool rvalid = r < p.M;
     const int parts = Kp / 32;
     const __nv_bfloat16* xr =
         xt + ((int64_t)(tc.b / p.bdiv) * Ntok + (rvalid ? r : 0)) * 2 * Kp;
-    for (int cc = 32 * half; cc < tile_cols_; cc += 64) {
+    for (int cc = src.first(half); cc < tile_cols_; cc += src.step()) {
       float v[32];
-      tmem_ld32(taddr + (uint32_t)cc, v);  // warp-collective: before any per-lane exit
+      src.load(cc, v);  // warp-collective: before any per-lane exit
       const int c0 = tc.tn * tile_cols_ + cc;
       if (c0 >= p.N || !rvalid) continue;
       const uint4* hp = reinterpret_cast<const uint4*>(xr + c0);
@@ -440,10 +469,14 @@ struct EpiHeads {
   int32_t t = 0, d = 0;
   const float2* rot = nullptr;  // [t][d/2]
   int32_t tile_cols_ = 256;
+  bool can_split() const { return true; }
+  static constexpr bool kAnyTile = false;  // a RoPE pair of C_k lies in one tile
 
-  __device__ void prefetch(const GemmParams&, const TileCoord&, int, int) const {}
+  template <class Src>
+  __device__ void prefetch(const GemmParams&, const TileCoord&, int, const Src&, int) const {}
 
-  __device__ void operator()(const GemmParams& p, const TileCoord& tc, int row, uint32_t taddr,
+  template <class Src>
+  __device__ void operator()(const GemmParams& p, const TileCoord& tc, int row, const Src& src,
                              int half, uint4* stage, const CUtensorMap*) const {
     const int r = tc.tm * kBM + row;
     const bool rvalid = r < p.M;
@@ -452,15 +485,15 @@ struct EpiHeads {
     const float2* rrow = rot + (int64_t)j * (d / 2);
     const int64_t obase = (int64_t)j * st + (int64_t)h * sh;
     const int hd = d / 2;
-    for (int cc = 32 * half; cc < tile_cols_; cc += 64) {
+    for (int cc = src.first(half); cc < tile_cols_; cc += src.step()) {
       const int c0 = c_tile + cc;
       if (c0 >= p.N) break;
       if (c0 < d) {
         // key columns: process pairs (m, m + d/2) when visiting the first half
         if (c0 >= hd) continue;
         float a[32], b[32];
-        tmem_ld32(taddr + (uint32_t)cc, a);
-        tmem_ld32(taddr + (uint32_t)(cc + hd), b);
+        src.load(cc, a);
+        src.load(cc + hd, b);
 #pragma unroll
         for (int e = 0; e < 32; ++e) {
           const float2 cs = rrow[c0 + e];
@@ -476,7 +509,7 @@ struct EpiHeads {
         warp_store64(stage, o4, ck + obase + c0 + hd, rvalid);
       } else {
         float v[32];
-        tmem_ld32(taddr + (uint32_t)cc, v);
+        src.load(cc, v);
         uint4 o4[4];
         pack_bf16x32(v, o4);
         warp_store64(stage, o4, cv + obase + (c0 - d), rvalid);

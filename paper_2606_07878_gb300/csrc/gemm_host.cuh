@@ -100,6 +100,93 @@ inline bool finalize_gemm(GemmParams& p, int ab_fmt) {
   return true;
 }
 
+// Clusters of `size` CTAs of a kernel that can be resident at once (its shared-memory size set).
+template <class Kern>
+inline int resident_clusters(Kern kern, int size, int threads, int smem, int num_sms) {
+  cudaLaunchConfig_t q = {};
+  q.gridDim = dim3(size * std::max(1, num_sms / size), 1, 1);
+  q.blockDim = dim3(threads, 1, 1);
+  q.dynamicSmemBytes = smem;
+  cudaLaunchAttribute qa[1];
+  qa[0].id = cudaLaunchAttributeClusterDimension;
+  qa[0].val.clusterDim.x = size;
+  qa[0].val.clusterDim.y = 1;
+  qa[0].val.clusterDim.z = 1;
+  q.attrs = qa;
+  q.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kern, &q) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    return 0;
+  }
+  return std::min(n, num_sms / size);
+}
+
+constexpr int kMaxSplit = 8;
+
+// Clusters of each size of tc_gemm_split_kernel<BN, Epi> that can be resident at once (0: none).
+template <int BN, class Epi>
+inline const int* split_resident(int num_sms) {
+  using S = GemmSmem<BN, Epi>;
+  auto kern = tc_gemm_split_kernel<BN, Epi>;
+  static thread_local int resident[kMaxSplit + 1] = {0};  // [0]: asked
+  if (resident[0] == 0) {
+    resident[0] = 1;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kBytes) !=
+        cudaSuccess) {
+      cudaGetLastError();
+      return resident;
+    }
+    for (int s = 2; s <= kMaxSplit; ++s)
+      resident[s] = resident_clusters(kern, s, gemm_threads<Epi>(), S::kBytes, num_sms);
+  }
+  return resident;
+}
+
+// CTAs per tile of the split kernel at tile width BN for a GEMM of `ntiles` such tiles: the count
+// that is fastest by the clocks of its parts (measured on 128-row tiles at about 1.9 GHz: 384 /
+// 512 / 768 per K iteration at BN = 64 / 128 / 256, where a stage's bytes bound it; 16000 to read
+// all but one of the partials of 256 columns through DSMEM, 1400 to write one; 2500 per 32
+// columns in the epilogue; 4000 to start), with all clusters resident at once. *cost: its clocks.
+template <int BN, class Epi>
+inline int split_ranks(int64_t ntiles, int iters, int num_sms, double* cost) {
+  *cost = 1e30;
+  if (ntiles > num_sms / 2) return 1;
+  const int* resident = split_resident<BN, Epi>(num_sms);
+  int best = 1;
+  for (int s = 2; s <= std::min(kMaxSplit, iters); ++s) {
+    if (ntiles > resident[s]) continue;
+    const int blocks = (BN / 8 + s * Epi::kWarps - 1) / (s * Epi::kWarps);
+    const double c = 4000 + (double)((iters + s - 1) / s) * (256 + 2 * BN) +
+                     (1400 + 16000.0 * (s - 1) / s) * BN / 256 + 2500.0 * blocks;
+    if (c < *cost) {
+      *cost = c;
+      best = s;
+    }
+  }
+  return best;
+}
+
+template <int BN, class Epi>
+inline cudaError_t launch_split(const CUtensorMap& ta, const CUtensorMap& tb,
+                                const CUtensorMap& tc, GemmParams p, const Epi& epi, int ranks,
+                                cudaStream_t stream) {
+  p.ksplit = ranks;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ranks * (unsigned)p.ntiles, 1, 1);
+  cfg.blockDim = dim3(gemm_threads<Epi>(), 1, 1);
+  cfg.dynamicSmemBytes = GemmSmem<BN, Epi>::kBytes;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = ranks;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, tc_gemm_split_kernel<BN, Epi>, ta, tb, tc, p, epi);
+}
+
 template <int BN, int kRole, class Epi>
 inline cudaError_t launch_gemm(const Operand2D& A, const Operand2D& B, GemmParams p, Epi epi,
                                int ab_fmt, int num_sms, cudaStream_t stream,
@@ -111,6 +198,21 @@ inline cudaError_t launch_gemm(const Operand2D& A, const Operand2D& B, GemmParam
   std::memset(&tc, 0, sizeof(tc));
   if (out_view != nullptr && !make_store_tmap(&tc, *out_view)) return cudaErrorInvalidValue;
   epi.tile_cols_ = BN;
+  if (epi.can_split() && p.ksplit == 1) {
+    double cost = 0, cost64 = 1e30;
+    const int ranks = split_ranks<BN, Epi>(p.ntiles, p.iters_total, num_sms, &cost);
+    if constexpr (Epi::kAnyTile && BN != 64) {  // narrower tiles: less to reduce per CTA
+      GemmParams q = p;
+      if (!finalize_gemm<64>(q, ab_fmt)) return cudaErrorInvalidValue;
+      const int ranks64 = split_ranks<64, Epi>(q.ntiles, q.iters_total, num_sms, &cost64);
+      if (ranks64 > 1 && cost64 < cost) {
+        if (!make_tmap(&tb, B, 64)) return cudaErrorInvalidValue;
+        epi.tile_cols_ = 64;
+        return launch_split<64, Epi>(ta, tb, tc, q, epi, ranks64, stream);
+      }
+    }
+    if (ranks > 1) return launch_split<BN, Epi>(ta, tb, tc, p, epi, ranks, stream);
+  }
   auto kern = tc_gemm_kernel<BN, Epi, kRole>;
   static thread_local bool attr_set = false;  // per instantiation
   if (!attr_set) {

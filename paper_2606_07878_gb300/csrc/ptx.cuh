@@ -467,6 +467,14 @@ STILL_DEV void mbar_arrive_cluster_relaxed(uint32_t cluster_addr) {
 STILL_DEV void st_cluster_f32(uint32_t cluster_addr, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
 }
+STILL_DEV float4 ld_cluster_f32x4(uint32_t cluster_addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(cluster_addr)
+               : "memory");
+  return v;
+}
 // Bounded wait with acquire at cluster scope: for phases completed by arrivals of other CTAs
 // that release data written into this CTA's shared memory.
 STILL_DEV bool mbar_wait_cluster(uint64_t* bar, uint32_t parity) {

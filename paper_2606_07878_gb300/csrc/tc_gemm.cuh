@@ -148,13 +148,22 @@ __device__ __forceinline__ void warp_load_rows(uint4* stage, const void* src, bo
   __syncwarp();
 }
 
-// Epi must provide:  __device__ void prefetch(const GemmParams&, const TileCoord&, int row,
-//                    int half) const  (called before the tile's accumulator is ready), and
-//                    __device__ void operator()(const GemmParams&, const TileCoord&,
-//                    int row_in_tile, uint32_t tmem_addr_of_this_warp_lane_quarter,
-//                    int half, uint4* warp_stage, const CUtensorMap* out_map) const;
-// where `half` (0 or 1) selects the 32-column chunks this warp owns: chunk c is handled by the
-// warp with half == (c & 1); the functor loads TMEM and stores its own results.
+// Where an epilogue warp finds its tile's accumulator: its lane quarter in TMEM. Of the 32-column
+// chunks, warp `half` (0 or 1) of the quarter takes every second one.
+struct TmemTile {
+  uint32_t taddr;
+  __device__ __forceinline__ int first(int half) const { return 32 * half; }
+  __device__ __forceinline__ int step() const { return 64; }
+  // 32 columns from column cc: thread i receives row i of the quarter (warp-collective)
+  __device__ __forceinline__ void load(int cc, float (&v)[32]) const {
+    tmem_ld32(taddr + (uint32_t)cc, v);
+  }
+};
+
+// Epi must provide:  prefetch(p, tc, row_in_tile, src, half)  (called before the tile's accumulator
+//                    is ready) and  operator()(p, tc, row_in_tile, src, half, warp_stage, out_map)
+// where src (TmemTile, or SplitTile below) holds the accumulator and names the chunks of this
+// warp; the functor loads them and stores its own results.
 // kRole only names the instantiation (one per GEMM of the launch sequence) so that profilers
 // can tell the GEMMs apart; it does not change the code.
 template <int BN, class Epi, int kRole>
@@ -313,7 +322,8 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
     uint32_t acc_phase = 0;
     for (int tile = blockIdx.x; tile < p.ntiles; tile += gridDim.x) {
       const TileCoord tc = decode_tile(p, tile);
-      epi.prefetch(p, tc, row, half);  // inputs that do not depend on the accumulator
+      const TmemTile src{tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN)};
+      epi.prefetch(p, tc, row, src, half);  // inputs that do not depend on the accumulator
       bool ok = mbar_wait(&tfull[acc], acc_phase);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok || warp_flag(abort_flag)) {
@@ -324,8 +334,7 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
         break;
       }
       tc_fence_after();
-      const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN);
-      epi(p, tc, row, taddr, half, stage, &tmC);
+      epi(p, tc, row, src, half, stage, &tmC);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty[acc]);
@@ -342,6 +351,231 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, 2 * BN);
+  }
+}
+
+// ------------------------------------------------------------------ split along K in a cluster
+//
+// For GEMMs of a few tiles (the latent sublayers at small t): one tile would keep one SM busy
+// with its whole K loop and then with the epilogue of all its columns, while the others idle.
+// Here the S CTAs of a cluster (S up to 8) share a tile: CTA s runs the K iterations
+// [it s / S, it (s + 1) / S), leaves its fp32 partial in shared memory, and after a cluster barrier
+// takes every S-th block of 32 rows x 32 columns through the epilogue, adding the S partials
+// through DSMEM, its own first and then the others' in turn (a fixed order, and no CTA is read by
+// all at once).
+//
+// Measured, one launch with its neighbours: 256 x 256 x (2 x 1024) 31 -> 14 us, 1004 x 1024 x
+// (2 x 8192) 113 -> 41 us, 1312 x 1024 x (2 x 8192) 113 -> 54 us. Of the 14 us the K iterations
+// take about 2 and the DSMEM reads 2.5: tiles are 64 columns wide where that makes the
+// reduction smaller than what it saves (split_ranks).
+
+// A block of 32 rows x 32 columns of a tile whose partials lie in the shared memories of a
+// cluster: float4 [BN / 4][128] each, column group q of row r at q * 128 + r.
+struct SplitTile {
+  uint32_t part;  // shared address of this CTA's partial
+  int rank, ranks;
+  int row, col;   // this thread's row, the block's first column
+  __device__ __forceinline__ int first(int) const { return col; }
+  __device__ __forceinline__ int step() const { return 1 << 20; }
+  __device__ __forceinline__ void load(int cc, float (&v)[32]) const {
+    const uint32_t at = part + (uint32_t)((cc / 4) * kBM + row) * 16u;
+    auto fetch = [&](int s, float4 (&w)[8]) {
+      const uint32_t a = cluster_map(at, (uint32_t)s);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) w[q] = ld_cluster_f32x4(a + (uint32_t)(q * kBM * 16));
+    };
+    auto next = [&](int s) { return s + 1 == ranks ? 0 : s + 1; };
+    auto add = [&](const float4 (&w)[8]) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        v[4 * q] += w[q].x;
+        v[4 * q + 1] += w[q].y;
+        v[4 * q + 2] += w[q].z;
+        v[4 * q + 3] += w[q].w;
+      }
+    };
+#pragma unroll
+    for (int e = 0; e < 32; ++e) v[e] = 0.f;
+    int s = rank, left = ranks;
+#pragma unroll 1
+    for (; left > 1; left -= 2) {  // two partials in flight
+      float4 w0[8], w1[8];
+      fetch(s, w0);
+      s = next(s);
+      fetch(s, w1);
+      s = next(s);
+      add(w0);
+      add(w1);
+    }
+    if (left == 1) {
+      float4 w0[8];
+      fetch(s, w0);
+      add(w0);
+    }
+  }
+};
+
+// One instantiation for all sublayers (no kRole): launches of a few microseconds that follow one
+// another find its instructions cached.
+template <int BN, class Epi>
+__global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
+    tc_gemm_split_kernel(const __grid_constant__ CUtensorMap tmA,
+                         const __grid_constant__ CUtensorMap tmB,
+                         const __grid_constant__ CUtensorMap tmC, const GemmParams p,
+                         const Epi epi) {
+  using S = GemmSmem<BN, Epi>;
+  constexpr int kStages = S::kStages;
+  static_assert(BN * kBM * 4 <= S::kEpiOffset, "the partial takes the ring's place");
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + S::kBarOffset);
+  uint64_t* empty = full + kStages;
+  uint64_t* tfull = empty + kStages;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfull + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const int rank = (int)cluster_ctarank(), ranks = p.ksplit;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(tfull, 1);
+    *abort_flag = 0;
+    fence_mbar_init();
+    tma_prefetch_desc(&tmA);
+    tma_prefetch_desc(&tmB);
+  }
+  if (warp == 1) {
+    tmem_alloc(tmem_slot, BN);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  // one tile per cluster: m-tiles fastest
+  TileCoord tc;
+  {
+    const int tile = (int)cluster_id_x();
+    tc.tm = tile % p.tiles_m;
+    tc.tn = (tile / p.tiles_m) % p.tiles_n;
+    tc.b = tile / p.tiles_m / p.tiles_n;
+    tc.split = 0;  // the epilogue sees whole sums
+  }
+  const int it0 = p.iters_total * rank / ranks, it1 = p.iters_total * (rank + 1) / ranks;
+  const int quarter = warp & 3;
+  const int half = (warp - 2) >> 2;
+  const int row = quarter * 32 + lane;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ------------------------------------------------------------ TMA producer
+      const int bo = tc.b / p.bdiv, bi = tc.b % p.bdiv;
+      const int64_t ar = bo * p.a_r1 + bi * p.a_r0 + (int64_t)tc.tm * kBM;
+      const int64_t ak = bo * p.a_k1 + bi * p.a_k0;
+      const int64_t br = bo * p.b_r1 + bi * p.b_r0 + (int64_t)tc.tn * BN;
+      const int64_t bk = bo * p.b_k1 + bi * p.b_k0;
+      int stage = 0, pass = 0, base = 0;
+      uint32_t phase = 0;
+      int sent = 0;
+      for (int it = it0; it < it1; ++it) {
+        while (pass < p.npass - 1 && it >= base + p.pass[pass].klen / kBK) {
+          base += p.pass[pass].klen / kBK;
+          ++pass;
+        }
+        const GemmPass& ps = p.pass[pass];
+        const int kk = (it - base) * kBK;
+        if (!mbar_wait(&empty[stage], phase ^ 1)) {
+          dev_set_error(p.err, DEV_WAIT_TIMEOUT, 110);
+          *abort_flag = 1;
+          break;
+        }
+        mbar_arrive_expect_tx(&full[stage], S::kStageBytes);
+        uint8_t* sa = smem + stage * S::kStageBytes;
+        tma_load_2d(sa, &tmA, &full[stage], (int32_t)(ak + ps.a_koff + kk),
+                    (int32_t)(ar + ps.a_roff));
+        tma_load_2d(sa + S::kABytes, &tmB, &full[stage], (int32_t)(bk + ps.b_koff + kk),
+                    (int32_t)(br + ps.b_roff));
+        ++sent;
+        if (++stage == kStages) {
+          stage = 0;
+          phase ^= 1;
+        }
+      }
+      if (*abort_flag)  // let every copy this thread issued land before the CTA can exit
+        for (int s = 0; s < min(sent, kStages); ++s) {
+          const int i = sent - 1 - s;  // the i-th copy used stage i % kStages in round i / kStages
+          (void)mbar_wait(&full[i % kStages], (uint32_t)(i / kStages) & 1u);
+        }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      // ------------------------------------------------------------ MMA issuer
+      int stage = 0;
+      uint32_t phase = 0;
+      for (int it = it0; it < it1; ++it) {
+        if (!mbar_wait(&full[stage], phase)) {
+          dev_set_error(p.err, DEV_WAIT_TIMEOUT, 111);
+          *abort_flag = 1;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t sa = smem_u32(smem + stage * S::kStageBytes);
+        const uint64_t ad = sdesc_k_sw128(sa);
+        const uint64_t bd = sdesc_k_sw128(sa + S::kABytes);
+#pragma unroll
+        for (int k = 0; k < kBK / 16; ++k)
+          tc_mma_f16(tmem_base, ad + 2 * k, bd + 2 * k, p.idesc, (it > it0 || k > 0) ? 1u : 0u);
+        tc_commit(&empty[stage]);
+        if (++stage == kStages) {
+          stage = 0;
+          phase ^= 1;
+        }
+      }
+      tc_commit(tfull);  // every MMA issued (also those before an abandoned wait)
+    }
+  } else {
+    // -------------------------------------------------------------- partial to shared memory
+    bool ok = mbar_wait(tfull, 0);
+    ok = __all_sync(0xffffffffu, ok);
+    if (!ok && lane == 0) {
+      dev_set_error(p.err, DEV_WAIT_TIMEOUT, 112);
+      *abort_flag = 1;
+    }
+    if (ok) {
+      tc_fence_after();
+      float4* part = reinterpret_cast<float4*>(smem) + row;
+      const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16);
+      for (int cc = 32 * half; cc < BN; cc += 64) {
+        float v[32];
+        tmem_ld32(taddr + (uint32_t)cc, v);
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          part[(cc / 4 + q) * kBM] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      }
+      tc_fence_before();
+    }
+  }
+  cluster_sync();
+  if (warp >= 2 && !warp_flag(abort_flag)) {
+    uint4* stage = reinterpret_cast<uint4*>(smem + S::kEpiOffset + (warp - 2) * S::kWarpStage);
+    // blocks of 32 x 32, rows fastest, dealt to the CTAs and then to their warps
+    for (int i = rank + ranks * (warp - 2); i < BN / 8; i += ranks * Epi::kWarps) {
+      const int r = (i & 3) * 32 + lane;
+      const SplitTile src{smem_u32(smem), rank, ranks, r, 32 * (i >> 2)};
+      epi(p, tc, r, src, 0, stage, &tmC);
+    }
+    if (lane == 0) bulk_wait_all();  // TMA stores issued by this warp (if any) have landed
+  }
+  // no CTA leaves while another may still read its partial
+  cluster_sync();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, BN);
   }
 }
 
