@@ -153,6 +153,7 @@ struct EpiAffine {
   // sums of squares have one slot per half tile: their chunks stay in one CTA
   bool can_split() const { return sumsq == nullptr; }
   static constexpr bool kAnyTile = true;  // its 32-column chunks are independent
+  static constexpr bool kPairs = true;    // has a 2-SM form
 
   // The residual rows of this warp's columns are pulled into L2 while the main loop runs.
   template <class Src>
@@ -423,6 +424,7 @@ struct EpiQuad {
   int32_t tile_cols_ = 256;
   bool can_split() const { return true; }
   static constexpr bool kAnyTile = true;
+  static constexpr bool kPairs = true;
 
   template <class Src>
   __device__ void prefetch(const GemmParams&, const TileCoord&, int, const Src&, int) const {}
@@ -470,6 +472,7 @@ struct EpiHeads {
   const float2* rot = nullptr;  // [t][d/2]
   int32_t tile_cols_ = 256;
   bool can_split() const { return true; }
+  static constexpr bool kPairs = false;
   static constexpr bool kAnyTile = false;  // a RoPE pair of C_k lies in one tile
 
   template <class Src>

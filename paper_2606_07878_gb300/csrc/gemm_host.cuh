@@ -100,6 +100,31 @@ inline bool finalize_gemm(GemmParams& p, int ab_fmt) {
   return true;
 }
 
+// Sets the kernel's shared-memory size and finds how many clusters of two CTAs can be resident.
+template <class Kern>
+inline cudaError_t resident_pairs(Kern kern, int threads, int smem, int num_sms, int* clusters) {
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t q = {};
+  q.gridDim = dim3(2 * std::max(1, num_sms / 2), 1, 1);
+  q.blockDim = dim3(threads, 1, 1);
+  q.dynamicSmemBytes = smem;
+  cudaLaunchAttribute qa[1];
+  qa[0].id = cudaLaunchAttributeClusterDimension;
+  qa[0].val.clusterDim.x = 2;
+  qa[0].val.clusterDim.y = 1;
+  qa[0].val.clusterDim.z = 1;
+  q.attrs = qa;
+  q.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kern, &q) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    n = num_sms / 2;
+  }
+  *clusters = std::max(1, std::min(n, num_sms / 2));
+  return cudaSuccess;
+}
+
 // Clusters of `size` CTAs of a kernel that can be resident at once (its shared-memory size set).
 template <class Kern>
 inline int resident_clusters(Kern kern, int size, int threads, int smem, int num_sms) {
@@ -187,6 +212,26 @@ inline cudaError_t launch_split(const CUtensorMap& ta, const CUtensorMap& tb,
   return cudaLaunchKernelEx(&cfg, tc_gemm_split_kernel<BN, Epi>, ta, tb, tc, p, epi);
 }
 
+// Pairs of CTAs of tc_gemm2_kernel when its waves take less time than those of the 1-SM kernel,
+// else 0. Measured clocks per K iteration, epilogue included: 720 for a 256 x 256 tile on two SMs,
+// 860 for a 128 x 256 tile on one (t = 1024, d_l = 1024). An odd number of m-tiles or a bad last
+// wave can make the pairs slower: t = 617, d_l = 2048, P v 488 us on single SMs, 584 on pairs.
+template <class Epi>
+inline int gemm2_clusters(const GemmParams& p, int num_sms) {
+  using S = Gemm2Smem<256, Epi>;
+  static thread_local int clusters = 0;
+  if (clusters == 0 && resident_pairs(tc_gemm2_kernel<256, Epi>, gemm_threads<Epi>(), S::kBytes,
+                                      num_sms, &clusters) != cudaSuccess) {
+    cudaGetLastError();
+    clusters = 0;
+    return 0;
+  }
+  const int64_t pairs = (int64_t)((p.tiles_m + 1) / 2) * p.tiles_n * p.batch;
+  const int64_t waves1 = (p.ntiles + num_sms - 1) / num_sms;
+  const int64_t waves2 = (pairs + clusters - 1) / clusters;
+  return waves2 * 720 < waves1 * 860 ? (int)std::min<int64_t>(pairs, clusters) : 0;
+}
+
 template <int BN, int kRole, class Epi>
 inline cudaError_t launch_gemm(const Operand2D& A, const Operand2D& B, GemmParams p, Epi epi,
                                int ab_fmt, int num_sms, cudaStream_t stream,
@@ -213,6 +258,25 @@ inline cudaError_t launch_gemm(const Operand2D& A, const Operand2D& B, GemmParam
     }
     if (ranks > 1) return launch_split<BN, Epi>(ta, tb, tc, p, epi, ranks, stream);
   }
+  if constexpr (BN == 256 && Epi::kPairs) {
+    const int clusters = p.ksplit == 1 ? gemm2_clusters<Epi>(p, num_sms) : 0;
+    if (clusters > 0) {
+      if (!make_tmap(&tb, B, BN / 2)) return cudaErrorInvalidValue;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(2 * (unsigned)clusters, 1, 1);
+      cfg.blockDim = dim3(gemm_threads<Epi>(), 1, 1);
+      cfg.dynamicSmemBytes = Gemm2Smem<BN, Epi>::kBytes;
+      cfg.stream = stream;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = 2;
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      return cudaLaunchKernelEx(&cfg, tc_gemm2_kernel<BN, Epi>, ta, tb, tc, p, epi);
+    }
+  }
   auto kern = tc_gemm_kernel<BN, Epi, kRole>;
   static thread_local bool attr_set = false;  // per instantiation
   if (!attr_set) {
@@ -224,31 +288,6 @@ inline cudaError_t launch_gemm(const Operand2D& A, const Operand2D& B, GemmParam
   const int grid = p.ntiles < num_sms ? p.ntiles : num_sms;
   kern<<<grid, gemm_threads<Epi>(), S::kBytes, stream>>>(ta, tb, tc, p, epi);
   return cudaGetLastError();
-}
-
-// Sets the kernel's shared-memory size and finds how many clusters of two CTAs can be resident.
-template <class Kern>
-inline cudaError_t resident_pairs(Kern kern, int threads, int smem, int num_sms, int* clusters) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t q = {};
-  q.gridDim = dim3(2 * std::max(1, num_sms / 2), 1, 1);
-  q.blockDim = dim3(threads, 1, 1);
-  q.dynamicSmemBytes = smem;
-  cudaLaunchAttribute qa[1];
-  qa[0].id = cudaLaunchAttributeClusterDimension;
-  qa[0].val.clusterDim.x = 2;
-  qa[0].val.clusterDim.y = 1;
-  qa[0].val.clusterDim.z = 1;
-  q.attrs = qa;
-  q.numAttrs = 1;
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, kern, &q) != cudaSuccess || n < 1) {
-    cudaGetLastError();
-    n = num_sms / 2;
-  }
-  *clusters = std::max(1, std::min(n, num_sms / 2));
-  return cudaSuccess;
 }
 
 }  // namespace still

@@ -1,0 +1,28 @@
+"""Latent sublayers wide enough for the GEMM on CTA pairs (256 x 256 tiles) against the oracle: an
+odd number of row tiles, rows and columns that end inside a tile, and several waves."""
+import pytest
+
+from gpu_helpers import Runner, assert_parity, oracle_layer
+from paper_2606_07878_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("H,d,D,n,F,t", [
+    (2, 64, 512, 4, 4096, 641),     # 11 row tiles (odd), FFN of 16 column tiles
+    (1, 128, 256, 16, 2880, 700),   # FFN width that ends inside a tile
+    (4, 64, 256, 8, 3072, 520),     # scores and P v over 32 batches
+])
+def test_wide_latent_sublayers_match_oracle(H, d, D, n, F, t):
+    wl = synth.tiny_workload(H=H, d=d, D=D, n=n, F=F, N=768, heavy=2, ts=(t,))
+    r = Runner(wl, t)
+    try:
+        K, V = synth.gen_kv(wl, 0, device=DEV)
+        Ck, Cv, _ = r.layer(0, K, V, t)
+        rk, rv, _, _ = oracle_layer(wl, r.W[0], K, V, t)
+        for name, ref, got in (("C_k", rk, Ck), ("C_v", rv, Cv)):
+            assert_parity(ref, synth.bf16_to_f64(got), name)
+    finally:
+        r.close()
