@@ -260,6 +260,7 @@ __global__ void __launch_bounds__(kFlashThreads, 1)
   cluster_sync();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  griddep_wait();
   // the even CTA's barriers, as seen from this CTA
   const uint32_t l_full = cluster_map(smem_u32(full), rank & ~1u);
   const uint32_t l_sfree = cluster_map(smem_u32(sfree), rank & ~1u);
@@ -687,19 +688,8 @@ inline cudaError_t launch_ca_flash(const Operand2D& Q, const Operand2D& K, const
     const cudaError_t e = resident_pairs(kern, kFlashThreads, S::kBytes, num_sms, &clusters);
     if (e != cudaSuccess) return e;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(kFlashThreads, 1, 1);
-  cfg.dynamicSmemBytes = S::kBytes;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cfg.gridDim = dim3(2 * (unsigned)std::min(f.nunits, clusters), 1, 1);
-  return cudaLaunchKernelEx(&cfg, kern, tq, tk, thi, tlo, f);
+  return launch_chained(kern, 2 * std::min(f.nunits, clusters), kFlashThreads, S::kBytes, stream, 2,
+                        tq, tk, thi, tlo, f);
 }
 
 // 2d = 512 (head dim 256): the same computation on clusters of four CTAs, two query tiles x

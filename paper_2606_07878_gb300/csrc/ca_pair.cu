@@ -53,6 +53,7 @@
 #include <algorithm>
 
 #include "ca_flash.cuh"
+#include "launch.cuh"
 
 namespace still {
 
@@ -179,6 +180,7 @@ __global__ void __launch_bounds__(kFlashThreads, 1)
   cluster_sync();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  griddep_wait();
   // the leader's barriers, as seen from this CTA
   const uint32_t l_full = cluster_map(smem_u32(full), rank & ~1u);
   const uint32_t l_sfree = cluster_map(smem_u32(sfree), rank & ~1u);
@@ -701,6 +703,7 @@ __global__ void __launch_bounds__(kFlashThreads, 1)
 // one-pass ones in every split's (O, l). See launch_ca_topk_repair.
 template <int D2>
 __global__ void __launch_bounds__(256) ca_topk_repair_kernel(const TopkRepairParams f) {
+  griddep_wait();
   constexpr float kLog2e = 1.4426950408889634f;
   constexpr int kG = D2 / 128;  // 4-column groups of O per lane
   constexpr int kQ = 8;         // 8-element q groups per lane (D <= 2048)
@@ -836,11 +839,11 @@ cudaError_t launch_ca_topk_repair(const TopkRepairParams& f, int d2, cudaStream_
   const int64_t rows = (int64_t)f.nb * f.t;
   const unsigned grid = (unsigned)((rows + 7) / 8);
   if (d2 == 512)
-    ca_topk_repair_kernel<512><<<grid, 256, 0, stream>>>(f);
+    launch_chained(ca_topk_repair_kernel<512>, grid, 256, 0, stream, 1, f);
   else if (d2 == 256)
-    ca_topk_repair_kernel<256><<<grid, 256, 0, stream>>>(f);
+    launch_chained(ca_topk_repair_kernel<256>, grid, 256, 0, stream, 1, f);
   else if (d2 == 128)
-    ca_topk_repair_kernel<128><<<grid, 256, 0, stream>>>(f);
+    launch_chained(ca_topk_repair_kernel<128>, grid, 256, 0, stream, 1, f);
   else
     return cudaErrorInvalidValue;
   return cudaGetLastError();
@@ -898,20 +901,9 @@ cudaError_t launch_ca_pair(const Operand2D& Q, const Operand2D& K, const Operand
     if (e != cudaSuccess) return e;
     attr_set[one_pass] = true;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(kFlashThreads, 1, 1);
-  cfg.dynamicSmemBytes = S::kBytes;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kPairCluster;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
   const int clusters = std::max(1, std::min(f.nunits, ca_pair_clusters(num_sms)));
-  cfg.gridDim = dim3(kPairCluster * clusters, 1, 1);
-  return cudaLaunchKernelEx(&cfg, kern, tq, tk, tx, f);
+  return launch_chained(kern, kPairCluster * clusters, kFlashThreads, S::kBytes, stream,
+                        kPairCluster, tq, tk, tx, f);
 }
 
 }  // namespace still

@@ -9,6 +9,7 @@
 #include <mutex>
 
 #include "epilogues.cuh"
+#include "launch.cuh"
 
 namespace still {
 
@@ -197,19 +198,8 @@ inline cudaError_t launch_split(const CUtensorMap& ta, const CUtensorMap& tb,
                                 const CUtensorMap& tc, GemmParams p, const Epi& epi, int ranks,
                                 cudaStream_t stream) {
   p.ksplit = ranks;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ranks * (unsigned)p.ntiles, 1, 1);
-  cfg.blockDim = dim3(gemm_threads<Epi>(), 1, 1);
-  cfg.dynamicSmemBytes = GemmSmem<BN, Epi>::kBytes;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = ranks;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, tc_gemm_split_kernel<BN, Epi>, ta, tb, tc, p, epi);
+  return launch_chained(tc_gemm_split_kernel<BN, Epi>, ranks * p.ntiles, gemm_threads<Epi>(),
+                        GemmSmem<BN, Epi>::kBytes, stream, ranks, ta, tb, tc, p, epi);
 }
 
 // Pairs of CTAs of tc_gemm2_kernel when its waves take less time than those of the 1-SM kernel,
@@ -262,19 +252,8 @@ inline cudaError_t launch_gemm(const Operand2D& A, const Operand2D& B, GemmParam
     const int clusters = p.ksplit == 1 ? gemm2_clusters<Epi>(p, num_sms) : 0;
     if (clusters > 0) {
       if (!make_tmap(&tb, B, BN / 2)) return cudaErrorInvalidValue;
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(2 * (unsigned)clusters, 1, 1);
-      cfg.blockDim = dim3(gemm_threads<Epi>(), 1, 1);
-      cfg.dynamicSmemBytes = Gemm2Smem<BN, Epi>::kBytes;
-      cfg.stream = stream;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = 2;
-      attr[0].val.clusterDim.y = 1;
-      attr[0].val.clusterDim.z = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      return cudaLaunchKernelEx(&cfg, tc_gemm2_kernel<BN, Epi>, ta, tb, tc, p, epi);
+      return launch_chained(tc_gemm2_kernel<BN, Epi>, 2 * clusters, gemm_threads<Epi>(),
+                            Gemm2Smem<BN, Epi>::kBytes, stream, 2, ta, tb, tc, p, epi);
     }
   }
   auto kern = tc_gemm_kernel<BN, Epi, kRole>;
@@ -286,8 +265,7 @@ inline cudaError_t launch_gemm(const Operand2D& A, const Operand2D& B, GemmParam
     attr_set = true;
   }
   const int grid = p.ntiles < num_sms ? p.ntiles : num_sms;
-  kern<<<grid, gemm_threads<Epi>(), S::kBytes, stream>>>(ta, tb, tc, p, epi);
-  return cudaGetLastError();
+  return launch_chained(kern, grid, gemm_threads<Epi>(), S::kBytes, stream, 1, ta, tb, tc, p, epi);
 }
 
 }  // namespace still

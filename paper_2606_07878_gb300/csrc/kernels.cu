@@ -4,6 +4,7 @@
 #include <type_traits>
 
 #include "kernels.cuh"
+#include "launch.cuh"
 
 namespace still {
 
@@ -223,6 +224,7 @@ __global__ void __launch_bounds__(256) strip_kernel(KVSource src, int64_t N, int
 // entries, fine[q][i] at i * w_m. Angles formed and reduced in fp64.
 __global__ void rope_tables_kernel(float4* coarse, float* omega, int G, int D, double origin,
                                    const double* __restrict__ omega_c) {
+  griddep_wait();
   const int quarter = D / 4;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)(G + kPosGrain) * quarter) return;
@@ -244,6 +246,7 @@ __global__ void rope_tables_kernel(float4* coarse, float* omega, int G, int D, d
 // (1, 0) when use_rope is 0.
 __global__ void heads_rot_kernel(float2* rot, int t, int hd, double pstart, double pstep,
                                  const double* __restrict__ omega, int use_rope) {
+  griddep_wait();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)t * hd) return;
   const int j = (int)(idx / hd), m = (int)(idx % hd);
@@ -259,6 +262,7 @@ __global__ void q_rope_kernel(const float* __restrict__ qhat, int t_max, int b0,
                               int D, double qstart, double qstep, const double* omega_c,
                               int use_rope, __nv_bfloat16* __restrict__ qhl, int fp16,
                               float qscale) {
+  griddep_wait();
   const int half = D / 2, q4 = half / 4;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)t * q4) return;
@@ -318,6 +322,7 @@ template <typename OutT>
 __global__ void __launch_bounds__(256) softmax_kernel(const float* __restrict__ S, int64_t ncols,
                                                       int64_t ldS, OutT* __restrict__ P,
                                                       int64_t ldP) {
+  griddep_wait();
   __shared__ float red_m[8], red_l[8];
   const int64_t row = blockIdx.x;
   const float* s = S + row * ldS;
@@ -374,6 +379,7 @@ template <typename OutT, int PER, bool HILO = false>
 __global__ void __launch_bounds__(256) softmax_reg_kernel(const float* __restrict__ S,
                                                           int64_t ncols, int64_t ldS,
                                                           OutT* __restrict__ P, int64_t ldP) {
+  griddep_wait();
   __shared__ float red[8];
   const int64_t row = blockIdx.x;
   const float* s = S + row * ldS;
@@ -473,6 +479,7 @@ __global__ void __launch_bounds__(256) ca_merge_kernel(const float* __restrict__
                                                        int nsplit, int b0, int nb, int n, int t,
                                                        int d2, int f16,
                                                        __nv_bfloat16* __restrict__ PX) {
+  griddep_wait();
   const int64_t rows = (int64_t)nb * t;
   const int64_t rj = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -516,6 +523,7 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const void* __restrict__ i
                                                       int64_t rows, int D, int64_t ldi, float eps,
                                                       __nv_bfloat16* __restrict__ out,
                                                       int64_t ldo, int hilo) {
+  griddep_wait();
   const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
@@ -558,6 +566,7 @@ __global__ void bf16_to_f16_kernel(uint16_t* p, int64_t n) {
 }
 
 __global__ void scale_rows_kernel(float* x, const float* inv, int64_t rows, int D) {
+  griddep_wait();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= rows * D) return;
   x[idx] *= inv[idx / D];
@@ -565,6 +574,7 @@ __global__ void scale_rows_kernel(float* x, const float* inv, int64_t rows, int 
 
 __global__ void inv_norms_kernel(const float* __restrict__ parts, int64_t nvec, int nparts,
                                  int64_t block, float eps, float alpha, float* __restrict__ out) {
+  griddep_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nvec) return;
   const float* p = parts + (i / block) * nparts * block + i % block;
@@ -644,6 +654,7 @@ __global__ void f32_hilo_kernel(const float* __restrict__ x, int64_t rows, int C
 __global__ void beta_kernel(const __nv_bfloat16* __restrict__ Z, int64_t rows, int t, int H,
                             int D, const float* __restrict__ w, float beta_max, float offset,
                             float* __restrict__ beta) {
+  griddep_wait();
   const int64_t row = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
@@ -954,6 +965,7 @@ __global__ void decode_merge_kernel(const __grid_constant__ DecodeStack st,
                                     const float* __restrict__ part_o,
                                     const float2* __restrict__ part_ml, int64_t rows, int nch,
                                     int d) {
+  griddep_wait();
   extern __shared__ float2 mls[];  // the row's (m, l) per chunk, then (weight, -)
   const int64_t row = blockIdx.x;
   const int c = threadIdx.x;
@@ -1001,8 +1013,9 @@ size_t decode_workspace_bytes(int64_t rows, int nslots, int d, int layers) {
 template <int D, int R>
 static cudaError_t launch_decode_chunks(const DecodeStack& st, int nslots, int nrb, float* part_o,
                                         float2* part_ml, cudaStream_t s) {
-  decode_chunk_kernel<D, R><<<dim3(nslots * nrb, st.layer[0].H, st.n), 32 * DecShape<D>::kWarps, 0,
-                              s>>>(st, nslots, nrb, part_o, part_ml);
+  const dim3 grid(nslots * nrb, st.layer[0].H, st.n);
+  decode_chunk_kernel<D, R><<<grid, 32 * DecShape<D>::kWarps, 0, s>>>(st, nslots, nrb, part_o,
+                                                                      part_ml);
   return cudaGetLastError();
 }
 
@@ -1034,8 +1047,8 @@ cudaError_t launch_decode_biased(const DecodeStack& st, void* ws, int num_sms, c
   if (e != cudaSuccess) return e;
   *launches = 1;
   if (nslots == 1) return cudaSuccess;
-  decode_merge_kernel<<<dim3((unsigned)rows, st.n), a.d, (size_t)nslots * sizeof(float2), s>>>(
-      st, part_o, part_ml, rows, nslots, a.d);
+  launch_chained(decode_merge_kernel, dim3((unsigned)rows, st.n), a.d, nslots * sizeof(float2), s,
+                 1, st, part_o, part_ml, rows, nslots, a.d);
   *launches = 2;
   return cudaGetLastError();
 }
@@ -1058,7 +1071,8 @@ cudaError_t launch_beta(const __nv_bfloat16* Z, int t, int H, int D, const float
                         float beta_max, float offset, float* beta, cudaStream_t s) {
   const int64_t rows = (int64_t)H * t;
   if (rows == 0) return cudaSuccess;
-  beta_kernel<<<blocks_for(rows, 8), 256, 0, s>>>(Z, rows, t, H, D, w, beta_max, offset, beta);
+  launch_chained(beta_kernel, blocks_for(rows, 8), 256, 0, s, 1, Z, rows, t, H, D, w, beta_max,
+                 offset, beta);
   return cudaGetLastError();
 }
 
@@ -1081,21 +1095,24 @@ cudaError_t launch_strip(const KVSource& src, int64_t N, int H, int d, const Pos
     attr = true;
   }
   strip_kernel<<<(unsigned)(Np / kStripTok), 256, smem, s>>>(src, N, H, d, segs, omega, rope_fix,
-                                                             vec, x16, Kp, X, XT, Np, gd, origin, G);
+                                                             vec, x16, Kp, X, XT, Np, gd, origin,
+                                                             G);
   return cudaGetLastError();
 }
 
 cudaError_t launch_heads_rot(float2* rot, int t, int hd, double pstart, double pstep,
                              const double* omega, int use_rope, cudaStream_t s) {
   const int64_t n = (int64_t)t * hd;
-  heads_rot_kernel<<<blocks_for(n, 256), 256, 0, s>>>(rot, t, hd, pstart, pstep, omega, use_rope);
+  launch_chained(heads_rot_kernel, blocks_for(n, 256), 256, 0, s, 1, rot, t, hd, pstart, pstep,
+                 omega, use_rope);
   return cudaGetLastError();
 }
 
 cudaError_t launch_rope_tables(float4* coarse, float* omega, int G, int D, double origin,
                                const double* omega_c, cudaStream_t s) {
   const int64_t n = (int64_t)(G + kPosGrain) * (D / 4);
-  rope_tables_kernel<<<blocks_for(n, 256), 256, 0, s>>>(coarse, omega, G, D, origin, omega_c);
+  launch_chained(rope_tables_kernel, blocks_for(n, 256), 256, 0, s, 1, coarse, omega, G, D, origin,
+                 omega_c);
   return cudaGetLastError();
 }
 
@@ -1104,8 +1121,8 @@ cudaError_t launch_q_rope(const float* qhat, int t_max, int b0, int nb, int t, i
                           __nv_bfloat16* qhl, int fp16, float qscale, cudaStream_t s) {
   if (D % 256 != 0) return cudaErrorInvalidValue;
   const int64_t n = (int64_t)t * (D / 8);
-  q_rope_kernel<<<blocks_for(n, 256), 256, 0, s>>>(qhat, t_max, b0, nb, t, D, qstart, qstep,
-                                                    omega_c, use_rope, qhl, fp16, qscale);
+  launch_chained(q_rope_kernel, blocks_for(n, 256), 256, 0, s, 1, qhat, t_max, b0, nb, t, D, qstart,
+                 qstep, omega_c, use_rope, qhl, fp16, qscale);
   return cudaGetLastError();
 }
 
@@ -1116,15 +1133,20 @@ static bool softmax_reg(const float* S, int64_t rows, int64_t ncols, int64_t ldS
   OutT* Pt = static_cast<OutT*>(P);
   if ((ldS % 4) != 0 || (ldP % 4) != 0) return false;
   if (need <= 1024)
-    softmax_reg_kernel<OutT, 4, HILO><<<(unsigned)rows, 256, 0, s>>>(S, ncols, ldS, Pt, ldP);
+    launch_chained(softmax_reg_kernel<OutT, 4, HILO>, (unsigned)rows, 256, 0, s, 1, S, ncols, ldS,
+                   Pt, ldP);
   else if (need <= 2048)
-    softmax_reg_kernel<OutT, 8, HILO><<<(unsigned)rows, 256, 0, s>>>(S, ncols, ldS, Pt, ldP);
+    launch_chained(softmax_reg_kernel<OutT, 8, HILO>, (unsigned)rows, 256, 0, s, 1, S, ncols, ldS,
+                   Pt, ldP);
   else if (need <= 4096)
-    softmax_reg_kernel<OutT, 16, HILO><<<(unsigned)rows, 256, 0, s>>>(S, ncols, ldS, Pt, ldP);
+    launch_chained(softmax_reg_kernel<OutT, 16, HILO>, (unsigned)rows, 256, 0, s, 1, S, ncols, ldS,
+                   Pt, ldP);
   else if (need <= 8192)
-    softmax_reg_kernel<OutT, 32, HILO><<<(unsigned)rows, 256, 0, s>>>(S, ncols, ldS, Pt, ldP);
+    launch_chained(softmax_reg_kernel<OutT, 32, HILO>, (unsigned)rows, 256, 0, s, 1, S, ncols, ldS,
+                   Pt, ldP);
   else if (need <= 16384)
-    softmax_reg_kernel<OutT, 64, HILO><<<(unsigned)rows, 256, 0, s>>>(S, ncols, ldS, Pt, ldP);
+    launch_chained(softmax_reg_kernel<OutT, 64, HILO>, (unsigned)rows, 256, 0, s, 1, S, ncols, ldS,
+                   Pt, ldP);
   else
     return false;
   return true;
@@ -1153,11 +1175,11 @@ cudaError_t launch_softmax(const float* S, int64_t rows, int64_t ncols, int64_t 
                : softmax_reg<__nv_bfloat16>(S, rows, ncols, ldS, P, ldP, s))
     return cudaGetLastError();
   if (out_fp16)
-    softmax_kernel<__half><<<(unsigned)rows, 256, 0, s>>>(S, ncols, ldS,
-                                                          static_cast<__half*>(P), ldP);
+    launch_chained(softmax_kernel<__half>, (unsigned)rows, 256, 0, s, 1, S, ncols, ldS,
+                   static_cast<__half*>(P), ldP);
   else
-    softmax_kernel<__nv_bfloat16><<<(unsigned)rows, 256, 0, s>>>(
-        S, ncols, ldS, static_cast<__nv_bfloat16*>(P), ldP);
+    launch_chained(softmax_kernel<__nv_bfloat16>, (unsigned)rows, 256, 0, s, 1, S, ncols, ldS,
+                   static_cast<__nv_bfloat16*>(P), ldP);
   return cudaGetLastError();
 }
 
@@ -1166,15 +1188,15 @@ cudaError_t launch_ca_merge(const float* O, const float2* stats, int nsplit, int
   const int64_t total = (int64_t)nb * t * d2;
   if (total == 0) return cudaSuccess;
   if (d2 % 4 != 0) return cudaErrorInvalidValue;
-  ca_merge_kernel<<<blocks_for((int64_t)nb * t, 8), 256, 0, s>>>(O, stats, nsplit, b0, nb, n, t,
-                                                                  d2, f16, PX);
+  launch_chained(ca_merge_kernel, blocks_for((int64_t)nb * t, 8), 256, 0, s, 1, O, stats, nsplit,
+                 b0, nb, n, t, d2, f16, PX);
   return cudaGetLastError();
 }
 
 cudaError_t launch_rmsnorm(const void* in, int in_bf16, int64_t rows, int D, int64_t ldi,
                            float eps, __nv_bfloat16* out, int64_t ldo, int hilo, cudaStream_t s) {
-  rmsnorm_kernel<<<blocks_for(rows, 8), 256, 0, s>>>(in, in_bf16, rows, D, ldi, eps, out, ldo,
-                                                     hilo);
+  launch_chained(rmsnorm_kernel, blocks_for(rows, 8), 256, 0, s, 1, in, in_bf16, rows, D, ldi, eps,
+                 out, ldo, hilo);
   return cudaGetLastError();
 }
 
@@ -1185,15 +1207,15 @@ cudaError_t launch_bf16_to_f16(void* p, int64_t n, cudaStream_t s) {
 }
 
 cudaError_t launch_scale_rows(float* x, const float* inv, int64_t rows, int D, cudaStream_t s) {
-  scale_rows_kernel<<<blocks_for(rows * D, 256), 256, 0, s>>>(x, inv, rows, D);
+  launch_chained(scale_rows_kernel, blocks_for(rows * D, 256), 256, 0, s, 1, x, inv, rows, D);
   return cudaGetLastError();
 }
 
 cudaError_t launch_inv_norms(const float* parts, int64_t nvec, int nparts, int64_t block, float eps,
                              float alpha, float* out, cudaStream_t s) {
   if (block < 1) return cudaErrorInvalidValue;
-  inv_norms_kernel<<<blocks_for(nvec, 256), 256, 0, s>>>(parts, nvec, nparts, block, eps, alpha,
-                                                         out);
+  launch_chained(inv_norms_kernel, blocks_for(nvec, 256), 256, 0, s, 1, parts, nvec, nparts, block,
+                 eps, alpha, out);
   return cudaGetLastError();
 }
 

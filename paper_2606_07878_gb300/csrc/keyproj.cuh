@@ -214,6 +214,7 @@ __global__ void __launch_bounds__(kKeyThreads, 1)
   cluster_sync();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  griddep_wait();
   const uint32_t l_afull = cluster_map(smem_u32(afull), rank & ~1u);
   const uint32_t l_bfull = cluster_map(smem_u32(bfull), rank & ~1u);
   const uint32_t l_tempty = cluster_map(smem_u32(tempty), rank & ~1u);
@@ -573,19 +574,8 @@ inline cudaError_t launch_key_proj_as(const Operand2D& X, const Operand2D& W, Ke
   // and a phase gives every pair several tiles
   const int64_t band_tiles = (int64_t)kBand * (p.nh * (p.D / 256));
   p.pbands = (int)std::max<int64_t>({1, kPhaseBytes / band_bytes, 4 * clusters / band_tiles});
-  cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(kKeyThreads, 1, 1);
-  cfg.dynamicSmemBytes = S::kBytes;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cfg.gridDim = dim3(2 * (unsigned)std::min<int64_t>(total, clusters), 1, 1);
-  return cudaLaunchKernelEx(&cfg, kern, ta, tb, p);
+  return launch_chained(kern, 2 * (int)std::min<int64_t>(total, clusters), kKeyThreads, S::kBytes,
+                        stream, 2, ta, tb, p);
 }
 
 inline cudaError_t launch_key_proj(const Operand2D& X, const Operand2D& W, const KeyProjParams& p,

@@ -56,6 +56,14 @@ STILL_DEV void prefetch_l2(const void* p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<uint64_t>(p)));
 }
 
+// ------------------------------------------------------------------------------- launch chain
+// Kernels of a launch sequence after its first one are launched with programmatic stream
+// serialization (launch.cuh): such a kernel may begin while the last CTAs of the one before it
+// still run. Every thread executes griddep_wait before it touches global memory that others read
+// or write; it returns when the previous kernel has completed, which has itself waited for its
+// own predecessor, so all earlier work is done and visible.
+STILL_DEV void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------------------------- fp32 pairs
 // Packed fp32 operations of sm_100 and later: each half rounds as the scalar operation does.
 

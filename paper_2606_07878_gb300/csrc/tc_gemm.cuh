@@ -211,6 +211,7 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  griddep_wait();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -443,6 +444,7 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
   cluster_sync();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  griddep_wait();
   const uint32_t l_full = cluster_map(smem_u32(full), rank & ~1u);
   const uint32_t l_tempty = cluster_map(smem_u32(tempty), rank & ~1u);
 
@@ -707,6 +709,7 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  griddep_wait();
   // one tile per cluster: m-tiles fastest
   TileCoord tc;
   {
