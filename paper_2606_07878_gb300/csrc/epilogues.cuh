@@ -174,10 +174,16 @@ struct EpiAffine {
   template <class Src>
   __device__ void operator()(const GemmParams& p, const TileCoord& tc, int row, const Src& src,
                              int half, uint4* stage, const CUtensorMap* tmc) const {
-    const int r = tc.tm * kBM + row;
-    const bool rvalid = r < p.M;
+    // A warp whose 32 rows all lie past M has nothing to do. In the warp that M ends in, the
+    // lanes past it repeat the last row and store nothing, so that the warp stays converged (on a
+    // path of their own they doubled the epilogue of the last row of tiles: q/k projection of
+    // 1,000 rows 112 us, of 992 or 1,024 rows 68).
+    const int tr = tc.tm * kBM + row;
+    if (tr - (int)(threadIdx.x & 31) >= p.M) return;
+    const bool rvalid = tr < p.M;
+    const int r = min(tr, p.M - 1);
     float rscale = alpha;
-    if (row_scale != nullptr && rvalid) rscale *= row_scale[rsm.at(tc.b, r, 0)];
+    if (row_scale != nullptr) rscale *= row_scale[rsm.at(tc.b, r, 0)];
     float ss = 0.f;
     for (int cc = src.first(half); cc < tile_cols_; cc += src.step()) {
       const int c0 = tc.tn * tile_cols_ + cc;
@@ -187,12 +193,12 @@ struct EpiAffine {
       const int nv = min(32, p.N - c0);
 #pragma unroll
       for (int e = 0; e < 32; ++e) v[e] *= rscale;
-      // Residual rows read coalesced by the whole warp (before the invalid-row exit: every
-      // lane takes part). Not on the TMA-store path, whose staging area may still be in use.
+      // Residual rows read coalesced by the whole warp. Not on the TMA-store path, whose
+      // staging area may still be in use.
       const bool res_vec = res_kind != 0 && tc.split == 0 && vec_ok && !tma_f32 && nv == 32;
       float resv[32];
       if (res_vec) {
-        const int64_t o = rvalid ? resm.at(tc.b, r, c0) : 0;
+        const int64_t o = resm.at(tc.b, r, c0);
         if (res_kind == 1) {
           uint4 u[8];
           warp_load_rows<8>(stage, static_cast<const float*>(res) + o, rvalid, u);
@@ -217,13 +223,6 @@ struct EpiAffine {
             }
           }
         }
-      }
-      if (!rvalid) {  // keep the warp-collective stores; the row itself is not written
-        if (tma_f32)
-          store32_tma(tc, row, c0, v, stage, tmc);
-        else
-          store32(p, tc.b, r, c0, v, tc.split, false, stage);
-        continue;
       }
       if (col_scale != nullptr) {
         float cs[32];
@@ -321,7 +320,7 @@ struct EpiAffine {
     const bool full = vec_ok && (c0 + 32 <= p.N);  // uniform across the warp
     const int64_t so = (int64_t)split * split_stride;
     if (full) {
-      const int64_t o = rvalid ? om.at(b, r, c0) + so : 0;
+      const int64_t o = om.at(b, r, c0) + so;
       uint4 a4[4], b4[4];
       if (kind == OUT_F32) {
         float* dst = static_cast<float*>(out) + o;
@@ -439,9 +438,9 @@ struct EpiQuad {
         xt + ((int64_t)(tc.b / p.bdiv) * Ntok + (rvalid ? r : 0)) * 2 * Kp;
     for (int cc = src.first(half); cc < tile_cols_; cc += src.step()) {
       float v[32];
-      src.load(cc, v);  // warp-collective: before any per-lane exit
+      src.load(cc, v);
       const int c0 = tc.tn * tile_cols_ + cc;
-      if (c0 >= p.N || !rvalid) continue;
+      if (c0 >= p.N) continue;
       const uint4* hp = reinterpret_cast<const uint4*>(xr + c0);
       const uint4* lp = reinterpret_cast<const uint4*>(xr + Kp + c0);
       float acc = 0.f;
@@ -457,7 +456,7 @@ struct EpiQuad {
           acc = fmaf(v[8 * q + 2 * k + 1], h2.y + l2.y, acc);
         }
       }
-      part[((int64_t)tc.b * parts + c0 / 32) * Ntok + r] = acc;
+      if (rvalid) part[((int64_t)tc.b * parts + c0 / 32) * Ntok + r] = acc;
     }
   }
 };
