@@ -711,7 +711,7 @@ int ca_pair_clusters(int num_sms);
 // kernel used: delta = 2^(e - m) - 2^(c - m) is added to the split's l and delta X_key to its O.
 // A split whose weight outside its candidates exceeds `guard` of its l is recomputed exactly
 // over all its keys. Candidates below 2^-cut of the row's largest weight are left as they are.
-// Deterministic: splits and candidates in a fixed order, one warp per row.
+// Deterministic: splits, candidates and ranges of keys are added in a fixed order.
 struct TopkRepairParams {
   const __half* q = nullptr;          // [nb * t][2D] fp16 hi | lo (times the q scale)
   const __half* k = nullptr;          // [nb * N][2D] fp16 hi | lo

@@ -699,62 +699,72 @@ __global__ void __launch_bounds__(kFlashThreads, 1)
   }
 }
 
-// One warp per (batch b, row r): the exact logits of the row's repair candidates replace the
-// one-pass ones in every split's (O, l). See launch_ca_topk_repair.
+// A CTA of 8 warps repairs 8 consecutive rows (b, r): the exact logits of a row's candidates
+// replace the one-pass ones in every split's (O, l). See launch_ca_topk_repair.
+//
+// Bound by the latency of the candidates' k rows (8 KB each at d_l = 2048): a row has 1 to 32 of
+// them, 4 on average, and with a warp per row a CTA waited for its longest row. Here each row's
+// warp only selects; the CTA's candidates form one list that its warps share out, with q and k
+// read as the logit needs them (few registers, so 24 warps a SM); then each row's warp adds its
+// own corrections. A row whose guard fires is recomputed by the whole CTA, a range of keys per
+// warp. Measured: 12,345 tokens, 128 heads, t = 617:
+// 2082 -> 687 us; 131,072 tokens, t = 655: 3701 -> 1216 (2 or 4 CTAs a SM: 756, 761 and 1356,
+// 1423; the k rows, q and O alone are 0.5 ms of memory time at 12,345 tokens).
 template <int D2>
-__global__ void __launch_bounds__(256) ca_topk_repair_kernel(const TopkRepairParams f) {
+__global__ void __launch_bounds__(256, 3) ca_topk_repair_kernel(const TopkRepairParams f) {
   griddep_wait();
   constexpr float kLog2e = 1.4426950408889634f;
   constexpr int kG = D2 / 128;  // 4-column groups of O per lane
-  constexpr int kQ = 8;         // 8-element q groups per lane (D <= 2048)
+  constexpr int kRows = 8;
+  __shared__ int s_key[kRows][32];
+  __shared__ float s_c[kRows][32];  // the one-pass logits, then the weight corrections
+  __shared__ float s_m[kRows];
+  __shared__ int s_cnt[kRows], s_scan[kRows];
+  __shared__ float s_l[kRows];
+  __shared__ __align__(16) float s_o[kRows][D2];
   const int64_t rows = (int64_t)f.nb * f.t;
-  const int64_t rj = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (rj >= rows) return;
-  const int b = (int)(rj / f.t);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t row0 = (int64_t)blockIdx.x * kRows;
+  const int64_t rj = row0 + warp;
+  const bool rvalid = rj < rows;
   float M = -INFINITY;
-  for (int s = 0; s < f.nsplit; ++s) M = fmaxf(M, f.stats[s * rows + rj].x);
-  uint4 qh[kQ], ql[kQ];
-  const __half* qrow = f.q + rj * 2 * (int64_t)f.D;
-#pragma unroll
-  for (int it = 0; it < kQ; ++it) {
-    const int i = 8 * lane + 256 * it;
-    qh[it] = i < f.D ? *reinterpret_cast<const uint4*>(qrow + i) : make_uint4(0, 0, 0, 0);
-    ql[it] = i < f.D ? *reinterpret_cast<const uint4*>(qrow + f.D + i) : make_uint4(0, 0, 0, 0);
-  }
+  if (rvalid)
+    for (int s = 0; s < f.nsplit; ++s) M = fmaxf(M, f.stats[s * rows + rj].x);
   // exact logit of one key in log2 units (q_hi k_hi + q_hi k_lo + q_lo k_hi, fp32), the same
   // value in every lane
-  auto logit = [&](int key) -> float {
-    const __half* krow = f.k + ((int64_t)b * f.N + key) * 2 * (int64_t)f.D;
+  auto logit = [&](int64_t row, int key) -> float {
+    const int64_t kr = (int64_t)((int)row / f.t) * f.N + key;
+    const __half* krow = f.k + kr * 2 * (int64_t)f.D;
+    const __half* qrow = f.q + row * 2 * (int64_t)f.D;
+    const float kinv = f.kinv[kr];
     float acc = 0.f;
+#pragma unroll 4
+    for (int i = 8 * lane; i < f.D; i += 256) {
+      const uint4 qh = *reinterpret_cast<const uint4*>(qrow + i);
+      const uint4 ql = *reinterpret_cast<const uint4*>(qrow + f.D + i);
+      const uint4 kh = *reinterpret_cast<const uint4*>(krow + i);
+      const uint4 kl = *reinterpret_cast<const uint4*>(krow + f.D + i);
+      const __half2* a = reinterpret_cast<const __half2*>(&qh);
+      const __half2* al = reinterpret_cast<const __half2*>(&ql);
+      const __half2* c = reinterpret_cast<const __half2*>(&kh);
+      const __half2* cl = reinterpret_cast<const __half2*>(&kl);
 #pragma unroll
-    for (int it = 0; it < kQ; ++it) {
-      const int i = 8 * lane + 256 * it;
-      if (i < f.D) {
-        const uint4 kh = *reinterpret_cast<const uint4*>(krow + i);
-        const uint4 kl = *reinterpret_cast<const uint4*>(krow + f.D + i);
-        const __half2* a = reinterpret_cast<const __half2*>(&qh[it]);
-        const __half2* al = reinterpret_cast<const __half2*>(&ql[it]);
-        const __half2* c = reinterpret_cast<const __half2*>(&kh);
-        const __half2* cl = reinterpret_cast<const __half2*>(&kl);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float2 x = __half22float2(a[e]), xl = __half22float2(al[e]);
-          const float2 y = __half22float2(c[e]), yl = __half22float2(cl[e]);
-          acc = fmaf(x.x, y.x, fmaf(x.x, yl.x, fmaf(xl.x, y.x, acc)));
-          acc = fmaf(x.y, y.y, fmaf(x.y, yl.y, fmaf(xl.y, y.y, acc)));
-        }
+      for (int e = 0; e < 4; ++e) {
+        const float2 x = __half22float2(a[e]), xl = __half22float2(al[e]);
+        const float2 y = __half22float2(c[e]), yl = __half22float2(cl[e]);
+        acc = fmaf(x.x, y.x, fmaf(x.x, yl.x, fmaf(xl.x, y.x, acc)));
+        acc = fmaf(x.y, y.y, fmaf(x.y, yl.y, fmaf(xl.y, y.y, acc)));
       }
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    return acc * (f.kinv[(int64_t)b * f.N + key] * kLog2e);
+    return acc * (kinv * kLog2e);
   };
-  const __nv_bfloat16* xbase = f.X + (int64_t)(b / f.bdiv) * f.N * 3 * f.d;
   float oacc[kG][4];
   // oacc += w * X_key (hi, plus lo on the K~ half)
-  auto add_x = [&](int key, float w) {
-    const __nv_bfloat16* xr = xbase + (int64_t)key * 3 * f.d;
+  auto add_x = [&](int64_t row, int key, float w) {
+    const __nv_bfloat16* xr =
+        f.X + ((int64_t)((int)row / f.t / f.bdiv) * f.N + key) * 3 * (int64_t)f.d;
 #pragma unroll
     for (int gq = 0; gq < kG; ++gq) {
       const int col = 4 * lane + 128 * gq;
@@ -776,54 +786,112 @@ __global__ void __launch_bounds__(256) ca_topk_repair_kernel(const TopkRepairPar
       oacc[gq][3] = fmaf(w, x23.y, oacc[gq][3]);
     }
   };
-  const int nc = f.nlists * kTopK;
-  for (int s = 0; s < f.nsplit; ++s) {
-    const int64_t sr = s * rows + rj;
-    const float2 st = f.stats[sr];
-    if (!(st.x >= M - f.cut)) continue;  // this split's weights are negligible in the row
-    const int* ck = f.cand_key + sr * nc;
-    const float* cc = f.cand_c + sr * nc;
+  auto zero = [&] {
 #pragma unroll
     for (int gq = 0; gq < kG; ++gq) oacc[gq][0] = oacc[gq][1] = oacc[gq][2] = oacc[gq][3] = 0.f;
-    float4* orow = reinterpret_cast<float4*>(f.O + sr * D2);
-    float wc = 0.f;  // the candidates' one-pass weights
-    for (int sl = 0; sl < nc; ++sl)
-      if (ck[sl] >= 0) wc += exp2f(cc[sl] - st.x);
-    if (st.y - wc > f.guard * st.y) {
-      // weight spread beyond the candidates: every key of the split, exact, in key order
-      const int j0 = (int)(((int64_t)f.tiles_k * s) / f.nsplit);
-      const int j1 = (int)(((int64_t)f.tiles_k * (s + 1)) / f.nsplit);
-      const int k1 = min(j1 * f.keys_per_tile, f.N);
+  };
+  const int nc = f.nlists * kTopK;  // at most 32: one slot per lane
+  for (int s = 0; s < f.nsplit; ++s) {
+    const int64_t sr = s * rows + rj;
+    const float2 st = rvalid ? f.stats[sr] : make_float2(-INFINITY, 0.f);
+    int cnt = 0;
+    bool scan = false;
+    // a split below the cut: its weights are negligible in the row
+    if (rvalid && st.x >= M - f.cut) {
+      const int key = lane < nc ? f.cand_key[sr * nc + lane] : -1;
+      const float c = key >= 0 ? f.cand_c[sr * nc + lane] : 0.f;
+      float wc = key >= 0 ? exp2f(c - st.x) : 0.f;  // the candidates' one-pass weights
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) wc += __shfl_xor_sync(0xffffffffu, wc, off);
+      // weight spread beyond the candidates: every key of the split, exact
+      scan = st.y - wc > f.guard * st.y;
+      const bool take = !scan && key >= 0 && c >= M - f.cut;
+      const uint32_t ball = __ballot_sync(0xffffffffu, take);
+      if (take) {
+        const int slot = __popc(ball & ((1u << lane) - 1));
+        s_key[warp][slot] = key;
+        s_c[warp][slot] = c;
+      }
+      cnt = __popc(ball);
+    }
+    if (lane == 0) {
+      s_cnt[warp] = cnt;
+      s_scan[warp] = scan;
+      s_m[warp] = st.x;
+    }
+    __syncthreads();
+    int total = 0;
+    uint32_t scans = 0;
+#pragma unroll
+    for (int w = 0; w < kRows; ++w) {
+      total += s_cnt[w];
+      scans |= s_scan[w] ? 1u << w : 0u;
+    }
+    // this warp's share of the list
+    for (int i = total * warp / kRows; i < total * (warp + 1) / kRows; ++i) {
+      int w = 0, slot = i;
+      while (slot >= s_cnt[w]) slot -= s_cnt[w++];
+      const float e = logit(row0 + w, s_key[w][slot]);
+      __syncwarp();
+      if (lane == 0) s_c[w][slot] = exp2f(e - s_m[w]) - exp2f(s_c[w][slot] - s_m[w]);
+    }
+    __syncthreads();
+    if (cnt > 0) {
+      float4* orow = reinterpret_cast<float4*>(f.O + sr * D2);
+      float dl = 0.f;
+      zero();
+#pragma unroll 2
+      for (int i = 0; i < cnt; ++i) {
+        const float delta = s_c[warp][i];
+        dl += delta;
+        add_x(rj, s_key[warp][i], delta);
+      }
+#pragma unroll
+      for (int gq = 0; gq < kG; ++gq) {
+        float4 o = orow[lane + 32 * gq];
+        o.x += oacc[gq][0];
+        o.y += oacc[gq][1];
+        o.z += oacc[gq][2];
+        o.w += oacc[gq][3];
+        orow[lane + 32 * gq] = o;
+      }
+      if (lane == 0) f.stats[sr].y = st.y + dl;
+    }
+    for (; scans != 0; scans &= scans - 1) {  // the same rows in every thread
+      const int w = __ffs(scans) - 1;
+      const int j0 = (int)(((int64_t)f.tiles_k * s) / f.nsplit) * f.keys_per_tile;
+      const int j1 = min((int)(((int64_t)f.tiles_k * (s + 1)) / f.nsplit) * f.keys_per_tile, f.N);
+      const int len = max(0, j1 - j0);
+      const int k1 = j0 + (int)((int64_t)len * (warp + 1) / kRows);
+      const float m = s_m[w];
       float lsum = 0.f;
-      for (int key = j0 * f.keys_per_tile; key < k1; ++key) {
-        const float w = exp2f(logit(key) - st.x);
-        lsum += w;
-        add_x(key, w);
+      zero();
+      for (int key = j0 + (int)((int64_t)len * warp / kRows); key < k1; ++key) {
+        const float wt = exp2f(logit(row0 + w, key) - m);
+        lsum += wt;
+        add_x(row0 + w, key, wt);
       }
 #pragma unroll
       for (int gq = 0; gq < kG; ++gq)
-        orow[lane + 32 * gq] = make_float4(oacc[gq][0], oacc[gq][1], oacc[gq][2], oacc[gq][3]);
-      if (lane == 0) f.stats[sr].y = lsum;
-      continue;
-    }
-    float dl = 0.f;
-    for (int sl = 0; sl < nc; ++sl) {
-      const int key = ck[sl];  // warp-uniform
-      if (key < 0 || !(cc[sl] >= M - f.cut)) continue;
-      const float delta = exp2f(logit(key) - st.x) - exp2f(cc[sl] - st.x);
-      dl += delta;
-      add_x(key, delta);
-    }
+        *reinterpret_cast<float4*>(&s_o[warp][4 * lane + 128 * gq]) =
+            make_float4(oacc[gq][0], oacc[gq][1], oacc[gq][2], oacc[gq][3]);
+      if (lane == 0) s_l[warp] = lsum;
+      __syncthreads();
+      const int64_t or_ = s * rows + row0 + w;
+      for (int col = threadIdx.x; col < D2; col += 256) {  // partial sums in key order
+        float o = 0.f;
 #pragma unroll
-    for (int gq = 0; gq < kG; ++gq) {
-      float4 o = orow[lane + 32 * gq];
-      o.x += oacc[gq][0];
-      o.y += oacc[gq][1];
-      o.z += oacc[gq][2];
-      o.w += oacc[gq][3];
-      orow[lane + 32 * gq] = o;
+        for (int x = 0; x < kRows; ++x) o += s_o[x][col];
+        f.O[or_ * D2 + col] = o;
+      }
+      if (threadIdx.x == 0) {
+        float l = 0.f;
+#pragma unroll
+        for (int x = 0; x < kRows; ++x) l += s_l[x];
+        f.stats[or_].y = l;
+      }
+      __syncthreads();
     }
-    if (lane == 0) f.stats[sr].y = st.y + dl;
   }
 }
 
@@ -831,21 +899,16 @@ __global__ void __launch_bounds__(256) ca_topk_repair_kernel(const TopkRepairPar
 
 cudaError_t launch_ca_topk_repair(const TopkRepairParams& f, int d2, cudaStream_t stream) {
   if (f.D <= 0 || f.D % 8 != 0 || f.D > 2048 || f.d * 2 != d2 || f.t <= 0 || f.nb <= 0 ||
-      f.N <= 0 || f.nsplit < 1 || f.nlists < 1 || f.tiles_k < f.nsplit ||
+      f.N <= 0 || f.nsplit < 1 || f.nlists < 1 ||
+      f.nlists * kTopK > 32 || f.tiles_k < f.nsplit || (int64_t)f.nb * f.t > 0x7fffffff ||
       (int64_t)f.tiles_k * f.keys_per_tile < f.N || f.q == nullptr || f.k == nullptr ||
       f.X == nullptr || f.O == nullptr || f.stats == nullptr || f.cand_key == nullptr ||
       f.cand_c == nullptr || f.bdiv < 1)
     return cudaErrorInvalidValue;
   const int64_t rows = (int64_t)f.nb * f.t;
   const unsigned grid = (unsigned)((rows + 7) / 8);
-  if (d2 == 512)
-    launch_chained(ca_topk_repair_kernel<512>, grid, 256, 0, stream, 1, f);
-  else if (d2 == 256)
-    launch_chained(ca_topk_repair_kernel<256>, grid, 256, 0, stream, 1, f);
-  else if (d2 == 128)
-    launch_chained(ca_topk_repair_kernel<128>, grid, 256, 0, stream, 1, f);
-  else
-    return cudaErrorInvalidValue;
+  if (d2 != 512) return cudaErrorInvalidValue;  // one-pass scores are taken at d = 256 only
+  launch_chained(ca_topk_repair_kernel<512>, grid, 256, 0, stream, 1, f);
   return cudaGetLastError();
 }
 
