@@ -149,6 +149,9 @@ struct EpiAffine {
   // launcher (boxes of 32 x 32 fp32, 128-byte swizzled staging); rows / columns past the view
   // are clipped by the copy engine.
   int32_t tma_f32 = 0;
+  // Columns [N, pad_n) of the last tile are stored as zeros (vec_ok outputs only; pad_n a multiple
+  // of 32): a last chunk that N ends in then goes out in vectors too. 0: nothing past N.
+  int32_t pad_n = 0;
   int32_t tile_cols_ = 256;  // the tile width BN, set by the launcher
   // sums of squares have one slot per half tile: their chunks stay in one CTA
   bool can_split() const { return sumsq == nullptr; }
@@ -187,12 +190,16 @@ struct EpiAffine {
     float ss = 0.f;
     for (int cc = src.first(half); cc < tile_cols_; cc += src.step()) {
       const int c0 = tc.tn * tile_cols_ + cc;
-      if (c0 >= p.N) continue;  // uniform across the warp
+      if (c0 >= max(p.N, pad_n)) continue;  // uniform across the warp
       float v[32];
       src.load(cc, v);
       const int nv = min(32, p.N - c0);
 #pragma unroll
       for (int e = 0; e < 32; ++e) v[e] *= rscale;
+      if (nv < 32 && pad_n > 0) {
+#pragma unroll
+        for (int e = 0; e < 32; ++e) v[e] = e < nv ? v[e] : 0.f;
+      }
       // Residual rows read coalesced by the whole warp. Not on the TMA-store path, whose
       // staging area may still be in use.
       const bool res_vec = res_kind != 0 && tc.split == 0 && vec_ok && !tma_f32 && nv == 32;
@@ -317,7 +324,7 @@ struct EpiAffine {
   __device__ __forceinline__ void store32(const GemmParams& p, int b, int r, int c0,
                                           const float (&v)[32], int split, bool rvalid,
                                           uint4* stage) const {
-    const bool full = vec_ok && (c0 + 32 <= p.N);  // uniform across the warp
+    const bool full = vec_ok && (c0 + 32 <= max(p.N, pad_n));  // uniform across the warp
     const int64_t so = (int64_t)split * split_stride;
     if (full) {
       const int64_t o = om.at(b, r, c0) + so;
