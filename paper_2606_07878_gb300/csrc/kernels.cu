@@ -28,88 +28,128 @@ __device__ __forceinline__ int64_t kv_offset(const KVSource& src, int64_t n, int
                 : n * src.sN + (int64_t)h * src.sH;
 }
 
-// Eight consecutive bf16 of a K / V row as fp32 (one 16-byte load when aligned).
-__device__ __forceinline__ void load8(const __nv_bfloat16* p, bool vec, float (&v)[8]) {
-  if (vec) {
-    const uint4 u = *reinterpret_cast<const uint4*>(p);
-    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+// Eight consecutive bf16 of a K / V row (one 16-byte load when aligned).
+__device__ __forceinline__ uint4 load8(const __nv_bfloat16* p, bool vec) {
+  if (vec) return *reinterpret_cast<const uint4*>(p);
+  const uint16_t* q = reinterpret_cast<const uint16_t*>(p);
+  uint32_t w[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[k]));
-      v[2 * k] = f.x;
-      v[2 * k + 1] = f.y;
-    }
-  } else {
+  for (int k = 0; k < 4; ++k) w[k] = q[2 * k] | (uint32_t)q[2 * k + 1] << 16;
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+__device__ __forceinline__ void widen8(const uint4& u, float (&v)[8]) {
+  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = __bfloat162float(p[e]);
+  for (int k = 0; k < 4; ++k) {
+    const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[k]));
+    v[2 * k] = f.x;
+    v[2 * k + 1] = f.y;
   }
 }
 
-// One CTA = 32 tokens x all KV-heads. The base-RoPE angles of the tile's tokens are formed
-// once (fp64, reduced mod 2 pi) and reused by every KV-head. Keys: inverse rotation of pairs
-// (m, m + d/2) (Sec. 2.2, RoPE-fix); values pass through. Writes X (bf16 hi | key lo) and XT
-// (fp16 hi for all 2d features, fp16 lo for the key half; the value half's lo is exactly zero
-// and is never read). Rows are moved in 16-byte pieces; the transpose for XT goes through
-// shared memory with an odd word pitch (conflict-free column reads).
+// One CTA = 32 tokens x the KV-heads of its share (blockIdx.y of gridDim.y). A thread handles the
+// same tokens and pairs of every head: it forms its base-RoPE angles once (fp64, reduced mod
+// 2 pi) and keeps them in registers. Keys: inverse rotation of pairs (m, m + d/2) (Sec. 2.2,
+// RoPE-fix); values pass through. Writes X (bf16 hi | key lo) and XT (fp16 hi for all 2d features,
+// fp16 lo for the key half; the value half's lo is exactly zero and is never read). Rows are
+// moved in 16-byte pieces; the transpose for XT goes through shared memory with an odd word pitch
+// (conflict-free column reads). The next head's rows are loaded while this head's XT is written.
 // Kp > 0 writes X in the layout of the folded key path instead: rows of 2 Kp elements,
 // [x~ hi | x~ lo] with x~ = [unRoPE(K) | V | 1 | 0 ...] (Kp >= 2d + 1, a multiple of 64).
-__global__ void __launch_bounds__(256) strip_kernel(KVSource src, int64_t N, int H, int d,
-                                                    PosSegs segs, const double* __restrict__ omega,
-                                                    int rope_fix, int vec, int x16, int Kp,
-                                                    __nv_bfloat16* __restrict__ X,
-                                                    __half* __restrict__ XT, int64_t Np,
-                                                    float2* __restrict__ gd, double origin, int G) {
-  extern __shared__ __align__(16) uint8_t sm[];
+//
+// Bound by memory (long caches) or by one CTA's chain of heads and the fp64 rate of its angles
+// (short ones). Measured before (angles in shared memory,
+// no load ahead, no shares) and now: 131,072 tokens of 8 heads of 256 channels 1291 -> 719 us
+// (4.8 GB: 6.7 TB/s), 65,536 of 8 x 128 268 -> 189, 8,003 of 4 x 128 33 -> 25, three windows of
+// 1,024 of 8 x 128 33 -> 14 each.
+template <int HD>
+__global__ void __launch_bounds__(256, HD == 256 ? 2 : 3)
+    strip_kernel(KVSource src, int64_t N, int H, PosSegs segs, const double* __restrict__ omega,
+                 int rope_fix, int vec, int x16, int Kp, __nv_bfloat16* __restrict__ X,
+                 __half* __restrict__ XT, int64_t Np, float2* __restrict__ gd, double origin,
+                 int G) {
+  constexpr int half = HD / 2;
+  constexpr int ph = 2 * HD + 2, pl = HD + 2;  // pitches (halves) of the transpose tiles
+  constexpr int kg = half / 8, vg = HD / 8;    // 8-element groups per token: key pairs, values
+  constexpr int kK = (kStripTok * kg + 255) / 256, kV = kStripTok * vg / 256;  // per thread
   __shared__ double tpos[kStripTok];
-  const int half = d / 2;
-  const int ph = 2 * d + 2, pl = d + 2;  // pitches (halves) of the transpose tiles
-  float2* rot = reinterpret_cast<float2*>(sm);  // [kStripTok][half]: (cos, sin)
-  __half* thi = reinterpret_cast<__half*>(rot + kStripTok * half);  // [kStripTok][ph]
-  __half* tlo = thi + kStripTok * ph;                                 // [kStripTok][pl]
+  extern __shared__ __align__(16) uint8_t sm[];
+  __half* thi = reinterpret_cast<__half*>(sm);  // [kStripTok][ph]
+  __half* tlo = thi + kStripTok * ph;           // [kStripTok][pl]
   const int64_t n0 = (int64_t)blockIdx.x * kStripTok;
+  const int h0 = H * blockIdx.y / gridDim.y, h1 = H * (blockIdx.y + 1) / gridDim.y;
+  uint4 ka[kK], kb[kK], va[kV];
+  auto load = [&](int h) {
+    bool second;
+#pragma unroll
+    for (int q = 0; q < kK; ++q) {
+      const int it = threadIdx.x + 256 * q, m0 = 8 * (it % kg);
+      const int64_t n = n0 + it / kg;
+      ka[q] = kb[q] = make_uint4(0, 0, 0, 0);
+      if (it < kStripTok * kg && n < N) {
+        const int64_t off = kv_offset(src, n, h, second);
+        const __nv_bfloat16* kr = (second ? src.K2 : src.K) + off;
+        ka[q] = load8(kr + m0, vec);
+        kb[q] = load8(kr + half + m0, vec);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kV; ++q) {
+      const int it = threadIdx.x + 256 * q;
+      const int64_t n = n0 + it / vg;
+      va[q] = make_uint4(0, 0, 0, 0);
+      if (n < N) {
+        const int64_t off = kv_offset(src, n, h, second);
+        va[q] = load8((second ? src.V2 : src.V) + off + 8 * (it % vg), vec);
+      }
+    }
+  };
+  load(h0);
   if (threadIdx.x < kStripTok) {
     // token position (fp64) once per token; also the compactor-RoPE coarse index and residual
     const int64_t n = n0 + threadIdx.x;
     const double pos = n < N ? seg_position(segs, n) : origin;
     tpos[threadIdx.x] = pos;
-    if (n < N) {
+    if (n < N && blockIdx.y == 0) {
       int g = (int)floor((pos - origin) / (double)kPosGrain);
       g = max(0, min(g, G - 1));
       gd[n] = make_float2((float)g, (float)(pos - (origin + (double)g * kPosGrain)));
     }
   }
   __syncthreads();
-  for (int it = threadIdx.x; it < kStripTok * half; it += blockDim.x) {
-    const int tok = it / half, m = it % half;
-    const int64_t n = n0 + tok;
-    float sw = 0.f, cw = 1.f;
-    if (rope_fix && n < N) sincos_reduced(tpos[tok] * omega[m], &sw, &cw);
-    rot[it] = make_float2(cw, sw);
-  }
-  __syncthreads();
-  const int d3 = Kp > 0 ? 2 * Kp : 3 * d;  // X row pitch
-  const int lo0 = Kp > 0 ? Kp : 2 * d;     // column of the key lo part
-  const int64_t ld = 2 * Np;
-  const int kg = half / 8, vg = d / 8;  // 8-element groups per token: key pairs, values
-  for (int h = 0; h < H; ++h) {
-    // keys: group g holds pairs m = 8g .. 8g + 7
-    for (int it = threadIdx.x; it < kStripTok * kg; it += blockDim.x) {
-      const int tok = it / kg, m0 = 8 * (it % kg);
-      const int64_t n = n0 + tok;
-      float a[8], b[8];
-      if (n < N) {
-        bool second;
-        const int64_t off = kv_offset(src, n, h, second);
-        const __nv_bfloat16* kr = (second ? src.K2 : src.K) + off;
-        float ka[8], kb[8];
-        load8(kr + m0, vec, ka);
-        load8(kr + half + m0, vec, kb);
+  float2 rot[kK][8];  // (cos, sin)
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const float2 cs = rot[tok * half + m0 + e];
-          a[e] = ka[e] * cs.x + kb[e] * cs.y;
-          b[e] = -ka[e] * cs.y + kb[e] * cs.x;
-        }
+  for (int q = 0; q < kK; ++q) {
+    const int it = threadIdx.x + 256 * q, tok = it / kg, m0 = 8 * (it % kg);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      float sw = 0.f, cw = 1.f;
+      if (rope_fix && it < kStripTok * kg && n0 + tok < N)
+        sincos_reduced(tpos[tok] * omega[m0 + e], &sw, &cw);
+      rot[q][e] = make_float2(cw, sw);
+    }
+  }
+  const int d3 = Kp > 0 ? 2 * Kp : 3 * HD;  // X row pitch
+  const int lo0 = Kp > 0 ? Kp : 2 * HD;     // column of the key lo part
+  const int64_t ld = 2 * Np;
+  for (int h = h0; h < h1; ++h) {
+    // keys: group g holds pairs m = 8g .. 8g + 7
+#pragma unroll
+    for (int q = 0; q < kK; ++q) {
+      const int it = threadIdx.x + 256 * q, tok = it / kg, m0 = 8 * (it % kg);
+      if (kStripTok * kg % 256 != 0 && it >= kStripTok * kg) break;
+      const int64_t n = n0 + tok;
+      float a[8], b[8], xa[8], xb[8];
+      widen8(ka[q], xa);
+      widen8(kb[q], xb);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const float2 cs = rot[q][e];
+        a[e] = xa[e] * cs.x + xb[e] * cs.y;
+        b[e] = -xa[e] * cs.y + xb[e] * cs.x;
+      }
+      if (n < N) {
         uint32_t ah[4], al[4], bh[4], bl[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -122,23 +162,10 @@ __global__ void __launch_bounds__(256) strip_kernel(KVSource src, int64_t N, int
           }
         }
         __nv_bfloat16* xr = X + ((int64_t)h * N + n) * d3;
-        if (vec) {
-          *reinterpret_cast<uint4*>(xr + m0) = make_uint4(ah[0], ah[1], ah[2], ah[3]);
-          *reinterpret_cast<uint4*>(xr + half + m0) = make_uint4(bh[0], bh[1], bh[2], bh[3]);
-          *reinterpret_cast<uint4*>(xr + lo0 + m0) = make_uint4(al[0], al[1], al[2], al[3]);
-          *reinterpret_cast<uint4*>(xr + lo0 + half + m0) = make_uint4(bl[0], bl[1], bl[2], bl[3]);
-        } else {
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            reinterpret_cast<uint32_t*>(xr + m0)[k] = ah[k];
-            reinterpret_cast<uint32_t*>(xr + half + m0)[k] = bh[k];
-            reinterpret_cast<uint32_t*>(xr + lo0 + m0)[k] = al[k];
-            reinterpret_cast<uint32_t*>(xr + lo0 + half + m0)[k] = bl[k];
-          }
-        }
-      } else {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) a[e] = b[e] = 0.f;
+        *reinterpret_cast<uint4*>(xr + m0) = make_uint4(ah[0], ah[1], ah[2], ah[3]);
+        *reinterpret_cast<uint4*>(xr + half + m0) = make_uint4(bh[0], bh[1], bh[2], bh[3]);
+        *reinterpret_cast<uint4*>(xr + lo0 + m0) = make_uint4(al[0], al[1], al[2], al[3]);
+        *reinterpret_cast<uint4*>(xr + lo0 + half + m0) = make_uint4(bl[0], bl[1], bl[2], bl[3]);
       }
       __half* hr = thi + tok * ph;
       __half* lr = tlo + tok * pl;
@@ -155,36 +182,25 @@ __global__ void __launch_bounds__(256) strip_kernel(KVSource src, int64_t N, int
       }
     }
     // values: group g holds features 8g .. 8g + 7 (bf16 values are exact in fp16)
-    for (int it = threadIdx.x; it < kStripTok * vg; it += blockDim.x) {
-      const int tok = it / vg, f0 = 8 * (it % vg);
+#pragma unroll
+    for (int q = 0; q < kV; ++q) {
+      const int it = threadIdx.x + 256 * q, tok = it / vg, f0 = 8 * (it % vg);
       const int64_t n = n0 + tok;
       float v[8];
-      if (n < N) {
-        bool second;
-        const int64_t off = kv_offset(src, n, h, second);
-        const __nv_bfloat16* vr = (second ? src.V2 : src.V) + off + f0;
-        load8(vr, vec, v);
-        __nv_bfloat16* xr = X + ((int64_t)h * N + n) * d3 + d + f0;
-        if (x16) {  // values in fp16 (bf16 values in the fp16 range convert exactly)
+      widen8(va[q], v);
+      uint32_t w[4];
 #pragma unroll
-          for (int e = 0; e < 8; ++e) reinterpret_cast<__half*>(xr)[e] = __float2half_rn(v[e]);
-        } else if (vec) {
-          *reinterpret_cast<uint4*>(xr) = *reinterpret_cast<const uint4*>(vr);
-        } else {
-#pragma unroll
-          for (int e = 0; e < 8; ++e) xr[e] = vr[e];
-        }
-      } else {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = 0.f;
+      for (int k = 0; k < 4; ++k) {
+        const __half2 x = __floats2half2_rn(v[2 * k], v[2 * k + 1]);
+        w[k] = *reinterpret_cast<const uint32_t*>(&x);
+        *reinterpret_cast<uint32_t*>(thi + tok * ph + HD + f0 + 2 * k) = w[k];
       }
-      __half* hr = thi + tok * ph + d + f0;
-#pragma unroll
-      for (int e = 0; e < 8; e += 2)
-        *reinterpret_cast<__half2*>(hr + e) = __floats2half2_rn(v[e], v[e + 1]);
+      if (n < N)  // x16: values in fp16 (bf16 values in the fp16 range convert exactly)
+        *reinterpret_cast<uint4*>(X + ((int64_t)h * N + n) * d3 + HD + f0) =
+            x16 ? make_uint4(w[0], w[1], w[2], w[3]) : va[q];
     }
     if (Kp > 0) {  // folded layout: [.. | 1 | 0 ...] after the values, zeros after the key lo
-      const int nc = (Kp - 2 * d) / 8, nz = (Kp - d) / 8;  // 16-byte groups per token
+      const int nc = (Kp - 2 * HD) / 8, nz = (Kp - HD) / 8;  // 16-byte groups per token
       for (int it = threadIdx.x; it < kStripTok * (nc + nz); it += blockDim.x) {
         const int tok = it / (nc + nz), q = it % (nc + nz);
         const int64_t n = n0 + tok;
@@ -192,14 +208,16 @@ __global__ void __launch_bounds__(256) strip_kernel(KVSource src, int64_t N, int
         __nv_bfloat16* xr = X + ((int64_t)h * N + n) * d3;
         uint4 val = make_uint4(0, 0, 0, 0);
         if (q == 0) val.x = x16 ? 0x3C00u : 0x3F80u;  // 1.0 in the first element (fp16 / bf16)
-        *reinterpret_cast<uint4*>(xr + (q < nc ? 2 * d + 8 * q : Kp + d + 8 * (q - nc))) = val;
+        *reinterpret_cast<uint4*>(xr + (q < nc ? 2 * HD + 8 * q : Kp + HD + 8 * (q - nc))) = val;
       }
     }
     __syncthreads();
+    if (h + 1 < h1) load(h + 1);
     // XT: feature rows of 32 tokens, 8 tokens (16 B) per store; hi rows [0, 2d), lo rows [0, d)
     constexpr int kTg = kStripTok / 8;
-    const int nhi = 2 * d * kTg;
-    for (int it = threadIdx.x; it < 3 * d * kTg; it += blockDim.x) {
+    constexpr int nhi = 2 * HD * kTg;
+#pragma unroll 2
+    for (int it = threadIdx.x; it < 3 * HD * kTg; it += 256) {
       const bool lo = it >= nhi;
       const int q = lo ? it - nhi : it;
       const int f = q / kTg, t0 = 8 * (q % kTg);
@@ -212,7 +230,7 @@ __global__ void __launch_bounds__(256) strip_kernel(KVSource src, int64_t N, int
         const __half2 pr = __halves2half2(x0, x1);
         w[k] = *reinterpret_cast<const uint32_t*>(&pr);
       }
-      __half* dst = XT + ((int64_t)h * 2 * d + f) * ld + (lo ? Np : 0) + n0 + t0;
+      __half* dst = XT + ((int64_t)h * 2 * HD + f) * ld + (lo ? Np : 0) + n0 + t0;
       *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
     }
     __syncthreads();
@@ -1076,28 +1094,47 @@ cudaError_t launch_beta(const __nv_bfloat16* Z, int t, int H, int D, const float
   return cudaGetLastError();
 }
 
+template <int HD>
+static cudaError_t launch_strip_d(const KVSource& src, int64_t N, int H, const PosSegs& segs,
+                                  const double* omega, int rope_fix, int vec, int x16, int Kp,
+                                  __nv_bfloat16* X, __half* XT, int64_t Np, float2* gd,
+                                  double origin, int G, int num_sms, cudaStream_t s) {
+  constexpr int smem = kStripTok * (2 * HD + 2 + HD + 2) * 2;
+  static bool attr = false;
+  if (!attr) {
+    cudaFuncSetAttribute(strip_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    attr = true;
+  }
+  // Shares of the heads only while the token tiles leave SMs without two CTAs: each share forms
+  // the tile's angles again, at the fp64 rate.
+  const int64_t tiles = Np / kStripTok;
+  const int shares = (int)std::max<int64_t>(1, std::min<int64_t>(H, 2 * num_sms / tiles));
+  strip_kernel<HD><<<dim3((unsigned)tiles, shares), 256, smem, s>>>(
+      src, N, H, segs, omega, rope_fix, vec, x16, Kp, X, XT, Np, gd, origin, G);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_strip(const KVSource& src, int64_t N, int H, int d, const PosSegs& segs,
                          const double* omega, int rope_fix, __nv_bfloat16* X, __half* XT,
                          int64_t Np, float2* gd, double origin, int G, int x16, int Kp,
-                         cudaStream_t s) {
-  if (d % 16 != 0 || Np % kStripTok != 0 || (Kp != 0 && (Kp % 64 != 0 || Kp < 2 * d + 1)))
+                         int num_sms, cudaStream_t s) {
+  if (Np < kStripTok || Np % kStripTok != 0 || (Kp != 0 && (Kp % 64 != 0 || Kp < 2 * d + 1)))
     return cudaErrorInvalidValue;
-  const size_t smem = (size_t)kStripTok * (d / 2) * sizeof(float2) +
-                      (size_t)kStripTok * ((2 * d + 2) + (d + 2)) * 2;
   auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
   const bool second = src.n_split < N;
   const int vec = al16(src.K) && al16(src.V) && src.sN % 8 == 0 && src.sH % 8 == 0 &&
                   (!second || (al16(src.K2) && al16(src.V2) && src.sN2 % 8 == 0 &&
                                src.sH2 % 8 == 0));
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(strip_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024);
-    attr = true;
+  auto launch = [&](auto hd) {
+    return launch_strip_d<decltype(hd)::value>(src, N, H, segs, omega, rope_fix, vec, x16, Kp, X,
+                                               XT, Np, gd, origin, G, num_sms, s);
+  };
+  switch (d) {
+    case 64: return launch(std::integral_constant<int, 64>{});
+    case 128: return launch(std::integral_constant<int, 128>{});
+    case 256: return launch(std::integral_constant<int, 256>{});
   }
-  strip_kernel<<<(unsigned)(Np / kStripTok), 256, smem, s>>>(src, N, H, d, segs, omega, rope_fix,
-                                                             vec, x16, Kp, X, XT, Np, gd, origin,
-                                                             G);
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_heads_rot(float2* rot, int t, int hd, double pstart, double pstep,

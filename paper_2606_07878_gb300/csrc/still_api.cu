@@ -588,7 +588,8 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
   void* Z3 = ws + P.oZ3;
 
   KLAUNCH(STILL_K_STRIP, launch_strip(src, N, H, d, pos.segs, L.omega_b, c.rope_fix, X, XT, Np,
-                                      gd, pos.origin, P.G, L.f16 ? 1 : 0, fold_kp(L), s));
+                                      gd, pos.origin, P.G, L.f16 ? 1 : 0, fold_kp(L), ctx->nsm,
+                                      s));
   const int w_fmt = L.f16 ? 0 : 1;    // operand format of X, RMSNorm(Z), W_K and W_Q products
   const int zn_mode = L.f16 ? 2 : 1;  // RMSNorm(Z) as fp16 or bf16 hi | lo
   KLAUNCH(STILL_K_TABLES, launch_rope_tables(coarse, omega, P.G, D, pos.origin, L.omega_c, s));
