@@ -273,8 +273,10 @@ __global__ void heads_rot_kernel(float2* rot, int t, int hd, double pstart, doub
   rot[idx] = make_float2(c, s);
 }
 
-// Thread = (latent j, 4 consecutive pairs m); the angles are formed once and reused for every
-// batch. Columns are in pair-chunk order: pair m sits at f1 = (m / 128) * 256 + m % 128 and its
+// Thread = (latent j, 4 consecutive pairs m) x a share of the batches (blockIdx.y); the angles are
+// formed once and reused for every batch of the share. Bound by memory once enough rows are in
+// flight. Measured with one share and now: 64 batches of 164 x 1024 51 -> 26 us,
+// 32 of 251 x 1024 32 -> 25; from t = 655 up unchanged at 87% of the memory rate (one share). Columns are in pair-chunk order: pair m sits at f1 = (m / 128) * 256 + m % 128 and its
 // partner at f1 + 128, so four consecutive pairs are four consecutive columns.
 __global__ void q_rope_kernel(const float* __restrict__ qhat, int t_max, int b0, int nb, int t,
                               int D, double qstart, double qstep, const double* omega_c,
@@ -293,7 +295,9 @@ __global__ void q_rope_kernel(const float* __restrict__ qhat, int t_max, int b0,
     if (use_rope) sincos_reduced((qstart + (double)j * qstep) * omega_c[m0 + e], &s[e], &c[e]);
   }
   const int f1 = (m0 / 128) * 256 + (m0 % 128), f2 = f1 + 128;
-  for (int bb = 0; bb < nb; ++bb) {
+  const int bb1 = (int)((int64_t)nb * (blockIdx.y + 1) / gridDim.y);
+#pragma unroll 2
+  for (int bb = (int)((int64_t)nb * blockIdx.y / gridDim.y); bb < bb1; ++bb) {
     const float* q = qhat + ((int64_t)(b0 + bb) * t_max + j) * D;
     const float4 x4 = *reinterpret_cast<const float4*>(q + f1);
     const float4 y4 = *reinterpret_cast<const float4*>(q + f2);
@@ -491,46 +495,59 @@ __global__ void omega_kernel(double* out, int half, int width, double base) {
 // Key-split merge of the fused cross-attention. Split s holds, per row, the unnormalised
 // O_s = sum_k 2^(v_k - m_s) X_k and l_s = sum_k 2^(v_k - m_s) (v, m in log2 units). With
 // M = max_s m_s:  O = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s, summed in split order.
-// One warp per row; each lane owns 4-column groups (16-byte loads).
+// One warp per row; lane k holds the weight of split k (at most 32), and each lane owns G groups
+// of 4 columns (16-byte loads, those of several splits in flight). Measured with the statistics
+// read and the weights formed again per column group, and now: 131,072 tokens, t = 655 198 -> 129
+// us, 65,536 tokens, t = 1311 37 -> 27, 8,003 tokens, t = 251 21 -> 15.
+template <int G>
 __global__ void __launch_bounds__(256) ca_merge_kernel(const float* __restrict__ O,
                                                        const float2* __restrict__ stats,
                                                        int nsplit, int b0, int nb, int n, int t,
-                                                       int d2, int f16,
-                                                       __nv_bfloat16* __restrict__ PX) {
+                                                       int f16, __nv_bfloat16* __restrict__ PX) {
   griddep_wait();
+  constexpr int d2 = 128 * G;
   const int64_t rows = (int64_t)nb * t;
   const int64_t rj = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (rj >= rows) return;
-  float M = -INFINITY;
-  for (int k = 0; k < nsplit; ++k) M = fmaxf(M, stats[k * rows + rj].x);
+  const float2 st = lane < nsplit ? stats[lane * rows + rj] : make_float2(-INFINITY, 0.f);
+  float M = st.x;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+  const float wl = exp2f(st.x - M);
+  float4 acc[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) acc[g] = make_float4(0.f, 0.f, 0.f, 0.f);
   float L = 0.f;
+#pragma unroll 4
   for (int k = 0; k < nsplit; ++k) {
-    const float2 st = stats[k * rows + rj];
-    L += exp2f(st.x - M) * st.y;
+    const float4* orow = reinterpret_cast<const float4*>(O + (k * rows + rj) * d2) + lane;
+    const float w = __shfl_sync(0xffffffffu, wl, k);
+    L += w * __shfl_sync(0xffffffffu, st.y, k);
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const float4 o = orow[32 * g];
+      acc[g].x += w * o.x;
+      acc[g].y += w * o.y;
+      acc[g].z += w * o.z;
+      acc[g].w += w * o.w;
+    }
   }
   const float invL = 1.f / L;
   const int j = (int)(rj % t), bb = (int)(rj / t);
   const int b = b0 + bb, h = b / n, i = b % n;
   const int64_t ld = 2 * (int64_t)n * d2;
   __nv_bfloat16* row = PX + ((int64_t)h * t + j) * ld + (int64_t)i * d2;
-  for (int c = 4 * lane; c < d2; c += 128) {
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int k = 0; k < nsplit; ++k) {
-      const float w = exp2f(stats[k * rows + rj].x - M);
-      const float4 o = *reinterpret_cast<const float4*>(O + (k * rows + rj) * d2 + c);
-      acc.x += w * o.x;
-      acc.y += w * o.y;
-      acc.z += w * o.z;
-      acc.w += w * o.w;
-    }
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const int c = 4 * lane + 128 * g;
     uint32_t h01, l01, h23, l23;
     if (f16) {  // fp16 hi | lo
-      split_pack_f16(acc.x * invL, acc.y * invL, h01, l01);
-      split_pack_f16(acc.z * invL, acc.w * invL, h23, l23);
+      split_pack_f16(acc[g].x * invL, acc[g].y * invL, h01, l01);
+      split_pack_f16(acc[g].z * invL, acc[g].w * invL, h23, l23);
     } else {
-      split_pack(acc.x * invL, acc.y * invL, h01, l01);
-      split_pack(acc.z * invL, acc.w * invL, h23, l23);
+      split_pack(acc[g].x * invL, acc[g].y * invL, h01, l01);
+      split_pack(acc[g].z * invL, acc[g].w * invL, h23, l23);
     }
     *reinterpret_cast<uint2*>(row + c) = make_uint2(h01, h23);
     *reinterpret_cast<uint2*>(row + (int64_t)n * d2 + c) = make_uint2(l01, l23);
@@ -1155,11 +1172,15 @@ cudaError_t launch_rope_tables(float4* coarse, float* omega, int G, int D, doubl
 
 cudaError_t launch_q_rope(const float* qhat, int t_max, int b0, int nb, int t, int D,
                           double qstart, double qstep, const double* omega_c, int use_rope,
-                          __nv_bfloat16* qhl, int fp16, float qscale, cudaStream_t s) {
+                          __nv_bfloat16* qhl, int fp16, float qscale, int num_sms,
+                          cudaStream_t s) {
   if (D % 256 != 0) return cudaErrorInvalidValue;
   const int64_t n = (int64_t)t * (D / 8);
-  launch_chained(q_rope_kernel, blocks_for(n, 256), 256, 0, s, 1, qhat, t_max, b0, nb, t, D, qstart,
-                 qstep, omega_c, use_rope, qhl, fp16, qscale);
+  const unsigned tiles = blocks_for(n, 256);
+  // shares of the batches until each SM has three CTAs
+  const unsigned shares = std::max(1u, std::min((unsigned)nb, 3u * num_sms / tiles));
+  launch_chained(q_rope_kernel, dim3(tiles, shares), 256, 0, s, 1, qhat, t_max, b0, nb, t, D,
+                 qstart, qstep, omega_c, use_rope, qhl, fp16, qscale);
   return cudaGetLastError();
 }
 
@@ -1224,10 +1245,18 @@ cudaError_t launch_ca_merge(const float* O, const float2* stats, int nsplit, int
                             int n, int t, int d2, int f16, __nv_bfloat16* PX, cudaStream_t s) {
   const int64_t total = (int64_t)nb * t * d2;
   if (total == 0) return cudaSuccess;
-  if (d2 % 4 != 0) return cudaErrorInvalidValue;
-  launch_chained(ca_merge_kernel, blocks_for((int64_t)nb * t, 8), 256, 0, s, 1, O, stats, nsplit,
-                 b0, nb, n, t, d2, f16, PX);
-  return cudaGetLastError();
+  if (nsplit < 1 || nsplit > 32) return cudaErrorInvalidValue;
+  auto launch = [&](auto groups) {
+    launch_chained(ca_merge_kernel<decltype(groups)::value>, blocks_for((int64_t)nb * t, 8), 256,
+                   0, s, 1, O, stats, nsplit, b0, nb, n, t, f16, PX);
+    return cudaGetLastError();
+  };
+  switch (d2) {
+    case 128: return launch(std::integral_constant<int, 1>{});
+    case 256: return launch(std::integral_constant<int, 2>{});
+    case 512: return launch(std::integral_constant<int, 4>{});
+  }
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_rmsnorm(const void* in, int in_bf16, int64_t rows, int D, int64_t ldi,

@@ -99,7 +99,8 @@ cudaError_t launch_rope_tables(float4* coarse, float* omega, int G, int D, doubl
 // fp16: hi/lo in fp16 of (q * qscale) instead of bf16 of q (qscale a power of two).
 cudaError_t launch_q_rope(const float* qhat, int t_max, int b0, int nb, int t, int D,
                           double qstart, double qstep, const double* omega_c, int use_rope,
-                          __nv_bfloat16* qhl, int fp16, float qscale, cudaStream_t s);
+                          __nv_bfloat16* qhl, int fp16, float qscale, int num_sms,
+                          cudaStream_t s);
 
 // One-block kernel whose bounded wait on an mbarrier can only expire (failure-detection test).
 cudaError_t launch_wait_timeout_selftest(int* err, unsigned long long limit_ns, cudaStream_t s);

@@ -748,7 +748,7 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
     if (!L.fold)
       KLAUNCH(STILL_K_QROPE, launch_q_rope(qsrc, q_tmax, q_b0, nbl, t, D, qstart, qstep,
                                            L.omega_c, c.compactor_rope, qhl,
-                                           exact || tk ? 1 : 0, qscale, s));
+                                           exact || tk ? 1 : 0, qscale, ctx->nsm, s));
     {
       // S, the online softmax and P X in one kernel; per-split partials merged in order.
       FlashParams fp;
