@@ -119,7 +119,11 @@ __device__ __forceinline__ void pack_f32x16(const float* v, uint4 (&o)[4]) {
 // Host contract: csm, resm and (when vec_ok) om are contiguous in c (c0 == 1) with cdiv a
 // multiple of 32, so every 32-column chunk maps to 32 consecutive elements; ss_seg is a
 // multiple of the tile width.
-struct EpiAffine {
+// kChunkSums: one slot per 32-column chunk, so that a tile's chunks may lie in several CTAs, at the
+// price of more partials. A type of its own: as a run-time choice it cost the other projections
+// 1% to 4%.
+template <bool kChunkSums>
+struct EpiAffineT {
   static constexpr int kWarps = 8;  // two per lane quarter: alternating 32-column chunks
   static constexpr int kStages = 0;  // default pipeline depth
   int32_t kind = OUT_F32;
@@ -139,7 +143,7 @@ struct EpiAffine {
   float* sumsq = nullptr;  // partial sums of v^2 over segments of ss_seg columns
   AffineMap ssm;           // (b, r, c / ss_seg) -> vector index
   int32_t ss_seg = 1 << 30;
-  int32_t ss_parts = 2;    // slots per vector = 2 * ss_seg / tile width
+  int32_t ss_parts = 2;    // slots per vector: 2 * ss_seg / tile width, kChunkSums ss_seg / 32
   // Vectors in blocks of ss_block consecutive indices, stored part-major (see launch_inv_norms),
   // so that a warp's 32 rows write 32 consecutive floats of one part.
   int64_t ss_block = 1;
@@ -153,10 +157,9 @@ struct EpiAffine {
   // of 32): a last chunk that N ends in then goes out in vectors too. 0: nothing past N.
   int32_t pad_n = 0;
   int32_t tile_cols_ = 256;  // the tile width BN, set by the launcher
-  // sums of squares have one slot per half tile: their chunks stay in one CTA
-  bool can_split() const { return sumsq == nullptr; }
+  bool can_split() const { return sumsq == nullptr || kChunkSums; }
   static constexpr bool kAnyTile = true;  // its 32-column chunks are independent
-  static constexpr bool kPairs = true;    // has a 2-SM form
+  static constexpr bool kPairs = !kChunkSums;  // has a 2-SM form
 
   // The residual rows of this warp's columns are pulled into L2 while the main loop runs.
   template <class Src>
@@ -247,6 +250,10 @@ struct EpiAffine {
 #pragma unroll
         for (int e = 0; e < 32; ++e)
           if (e < nv) ss += v[e] * v[e];
+        if constexpr (kChunkSums) {
+          if (rvalid) store_sum(tc.b, r, c0, (c0 % ss_seg) / 32, ss);
+          ss = 0.f;
+        }
       }
       if (gelu) {
 #pragma unroll
@@ -274,12 +281,15 @@ struct EpiAffine {
       else
         store32(p, tc.b, r, c0, v, tc.split, rvalid, stage);
     }
-    if (sumsq != nullptr && rvalid) {
+    if (!kChunkSums && sumsq != nullptr && rvalid) {
       const int c_tile = tc.tn * tile_cols_;
-      const int slot = ((c_tile % ss_seg) / tile_cols_) * 2 + half;
-      const int64_t vec = ssm.at(tc.b, r, c_tile / ss_seg);
-      sumsq[(vec / ss_block) * ss_parts * ss_block + slot * ss_block + vec % ss_block] = ss;
+      store_sum(tc.b, r, c_tile, ((c_tile % ss_seg) / tile_cols_) * 2 + half, ss);
     }
+  }
+
+  __device__ __forceinline__ void store_sum(int b, int r, int c, int slot, float ss) const {
+    const int64_t vec = ssm.at(b, r, c / ss_seg);
+    sumsq[(vec / ss_block) * ss_parts * ss_block + slot * ss_block + vec % ss_block] = ss;
   }
 
   // 32 values of a per-column vector (the same in every lane), `fill` past the nv valid ones.
@@ -373,6 +383,8 @@ struct EpiAffine {
     }
   }
 };
+
+using EpiAffine = EpiAffineT<false>;
 
 // Cache positions given as segments: position of token idx = start[k] + (idx - begin[k]) * step[k].
 struct PosSegs {

@@ -312,6 +312,7 @@ struct Plan {
   int H, d, D, n, F, t;
   int64_t N, Np, tp, ldt;
   int G;
+  int sq_parts;   // sum-of-squares partials per self-attention q~ / k~ vector
   bool flash;     // fused cross-attention kernel (2d of 128 or 256) for the last block
   int ca_units;   // (h, i) pairs per cross-attention group
   int sa_heads;   // KV-heads per self-attention group
@@ -339,6 +340,22 @@ size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 // path reaches 0.020 once t passes 4000. In a layer of two blocks the next block's queries
 // amplify it further.
 bool value_hilo(const still_layer_config&) { return true; }
+
+// Largest latent count whose q/k projection has so few tiles (of 128 rows x 256 columns, for all H
+// banks) that it can be split over CTAs. Up to it the projection writes one sum-of-squares partial
+// per 32 columns (256 rows at d_l = 256, 4 heads: 20.4 -> 12.4 us); above, one per 128 columns,
+// which is less to write and read.
+int64_t split_latents(int64_t H, int64_t n, int64_t D) { return 76 / (2 * n * D / 256) * 128 / H; }
+
+// Partials per vector at t latents, and the bytes of one vector's partials and inverse norm summed
+// over them: never less for more latents, so that a workspace reserved for more serves fewer.
+int sumsq_parts(int64_t H, int64_t n, int64_t D, int64_t t) {
+  return (int)(t <= split_latents(H, n, D) ? D / 32 : 2 * (D / 256));
+}
+int64_t sumsq_bytes(int64_t H, int64_t n, int64_t D, int64_t t) {
+  const int64_t ts = std::min(t, split_latents(H, n, D));
+  return 4 * std::max(ts * (D / 32 + 1), t * (2 * (D / 256) + 1));
+}
 
 // The cross-attention scores of a one-block layer of head dim 256 (the kernel on clusters of
 // two CTAs) take one fp16 MMA pass (q_hi . k_hi) instead of three split-bf16 passes, and a
@@ -409,10 +426,11 @@ bool make_plan(const still_layer_config& c, bool lazy_q, int Kp, int64_t N, int 
   P.cand_b = one_pass_scores(c) && Kp == 0 ? 2 * a256(T * kTopLists * kTopK * 4) * kMaxFlashSplit
                                            : 0;
   // lazy q^: fp32 q~ of the unit and its sum-of-squares partials + inverse norms
+  P.sq_parts = sumsq_parts(H, n, D, T);
   P.qt_b = lazy_q ? a256(T * D * 4) + a256(T * 4 * (2 * (D / 256) + 1)) : 0;
   P.ca_unit_bytes = P.kb_b + P.kss_b + P.q_b + P.P_b + P.O_b + P.qt_b + P.cand_b;
   P.qk_b = a256(2 * n * T * 2 * D * 2);
-  P.sss_b = a256(2 * n * T * 4 * (2 * (D / 256) + 1));
+  P.sss_b = a256(2 * n * sumsq_bytes(H, n, D, T));
   P.vT_b = a256(n * D * P.tp * 2 * hl);
   P.Ssa_b = a256(n * T * P.ldt * 4);
   P.Psa_b = a256(n * T * P.tp * 2 * hl);
@@ -682,7 +700,7 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
       e.ssm.r0 = 1;
       e.ssm.c0 = t;
       e.ss_seg = D;
-      e.ss_parts = 2 * (D / 256);
+      e.ss_parts = 2 * (D / 256);  // as at weight load: the same bits
       e.ss_block = t;
       e.vec_ok = 1;
       TRY(run_gemm256<STILL_K_LOAD>(ctx, op(Zn, (int64_t)H * t, 2 * D), op(Bw.WqT, (int64_t)n * D, D),
@@ -868,7 +886,7 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
     uint8_t* g = ws + P.oSA;
     bf16* qk = reinterpret_cast<bf16*>(g);
     g += P.qk_b * nh;
-    const int sparts = 2 * (D / 256);
+    const int sparts = P.sq_parts;
     float* sss = reinterpret_cast<float*>(g);                 // [nh][2n][t][sparts]
     float* sinv = sss + (size_t)nh * 2 * n * t * sparts;       // [nh][2n][t]
     g += P.sss_b * nh;
@@ -881,28 +899,30 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
       GemmParams p = gp(nh * t, 2 * n * D);
       add_pass(p, 0, 0, h0 * t, 0, D);
       add_pass(p, D, 0, h0 * t, 0, D);
-      EpiAffine e;
-      e.kind = vkind;
-      e.out = qk;
-      e.lo_off = D;
-      e.om.rdiv = t;
-      e.om.r1 = (int64_t)2 * n * t * 2 * D;
-      e.om.r0 = 2 * D;
-      e.om.cdiv = D;
-      e.om.c1 = (int64_t)t * 2 * D;
-      e.om.c0 = 1;
-      e.bias = Bw.sbqk;
-      e.sumsq = sss;
-      e.ssm.rdiv = t;
-      e.ssm.r1 = (int64_t)2 * n * t;
-      e.ssm.r0 = 1;
-      e.ssm.c0 = t;
-      e.ss_seg = D;
-      e.ss_parts = sparts;
-      e.ss_block = t;
-      e.vec_ok = 1;
-      TRY(run_gemm256<STILL_K_SA_PROJ>(ctx, op(A1, rows, 2 * D), op(Bw.SqkT, (int64_t)2 * n * D, D),
-                                       p, e, vfmt, s));
+      auto project = [&](auto e) -> still_status {
+        e.kind = vkind;
+        e.out = qk;
+        e.lo_off = D;
+        e.om.rdiv = t;
+        e.om.r1 = (int64_t)2 * n * t * 2 * D;
+        e.om.r0 = 2 * D;
+        e.om.cdiv = D;
+        e.om.c1 = (int64_t)t * 2 * D;
+        e.om.c0 = 1;
+        e.bias = Bw.sbqk;
+        e.sumsq = sss;
+        e.ssm.rdiv = t;
+        e.ssm.r1 = (int64_t)2 * n * t;
+        e.ssm.r0 = 1;
+        e.ssm.c0 = t;
+        e.ss_seg = D;
+        e.ss_parts = sparts;
+        e.ss_block = t;
+        e.vec_ok = 1;
+        return run_gemm256<STILL_K_SA_PROJ>(ctx, op(A1, rows, 2 * D),
+                                            op(Bw.SqkT, (int64_t)2 * n * D, D), p, e, vfmt, s);
+      };
+      TRY(sparts == D / 32 ? project(EpiAffineT<true>()) : project(EpiAffine()));
     }
     KLAUNCH(STILL_K_NORMS,
             launch_inv_norms(sss, (int64_t)nh * 2 * n * t, sparts, t, c.l2_eps, 1.f, sinv, s));
