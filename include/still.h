@@ -437,7 +437,7 @@ still_status still_get_device_status(still_ctx* ctx, void* stream, int32_t* h_de
 /* Kernel classes of the launch sequence, for launch counts and timings. */
 typedef enum {
   STILL_K_STRIP = 0,    /* RoPE-fix + [K; V] concat (hi/lo)                 */
-  STILL_K_TABLES,       /* compactor-RoPE angle table                       */
+  STILL_K_TABLES,       /* angle tables: compactor RoPE, output heads       */
   STILL_K_KEYPROJ,      /* k = RoPE_c(X W_K + b_K) (2-pass tcgen05 GEMM)    */
   STILL_K_QROPE,        /* q = RoPE_c(q^) at the latent query positions     */
   STILL_K_SCORES,       /* (unused: the scores are fused into STILL_K_CA_FUSED) */

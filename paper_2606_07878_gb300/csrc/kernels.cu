@@ -237,51 +237,48 @@ __global__ void __launch_bounds__(256, HD == 256 ? 2 : 3)
   }
 }
 
-// Compactor-RoPE tables of (cos, cos, sin, sin) of two neighbouring pairs 2 q and 2 q + 1: rows
-// [0, G) hold coarse[g][q] at (origin + g * kPosGrain) * w_m, then, in the next kPosGrain * D/4
-// entries, fine[q][i] at i * w_m. Angles formed and reduced in fp64.
-__global__ void rope_tables_kernel(float4* coarse, float* omega, int G, int D, double origin,
-                                   const double* __restrict__ omega_c) {
+// The call's angle tables (see RopeTables): coarse rows, then the fine table, then the output heads'
+// rotations, an entry per thread. Angles formed and reduced in fp64, whose rate bounds it. One
+// launch for all three; in CTAs of the strip launch they held up its token tiles (8,003 tokens:
+// the call 953 -> 961 us).
+__global__ void rope_tables_kernel(const RopeTables tb) {
   griddep_wait();
-  const int quarter = D / 4;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (int64_t)(G + kPosGrain) * quarter) return;
-  const int g = (int)(idx / quarter);
-  const int64_t f = idx - (int64_t)G * quarter;  // index into the fine table when >= 0
-  const int q = g < G ? (int)(idx % quarter) : (int)(f / kPosGrain);
-  float s[2], c[2];
+  const int quarter = tb.D / 4;
+  const int64_t ncoarse = (int64_t)tb.G * quarter, nkey = ncoarse + (int64_t)kPosGrain * quarter;
+  if (idx < nkey) {
+    const int g = (int)(idx / quarter);
+    const int64_t f = idx - ncoarse;  // index into the fine table when >= 0
+    const int q = g < tb.G ? (int)(idx % quarter) : (int)(f / kPosGrain);
+    float s[2], c[2];
 #pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    const double w = omega_c[2 * q + e];
-    const double ang = g < G ? (origin + (double)g * kPosGrain) * w : (double)(f % kPosGrain) * w;
-    sincos_reduced(ang, &s[e], &c[e]);
-    if (g == 0) omega[2 * q + e] = (float)w;
+    for (int e = 0; e < 2; ++e) {
+      const double w = tb.omega_c[2 * q + e];
+      const double ang =
+          g < tb.G ? (tb.origin + (double)g * kPosGrain) * w : (double)(f % kPosGrain) * w;
+      sincos_reduced(ang, &s[e], &c[e]);
+      if (g == 0) tb.omega[2 * q + e] = (float)w;
+    }
+    tb.coarse[idx] = make_float4(c[0], c[1], s[0], s[1]);
+  } else if (idx - nkey < (int64_t)tb.t * tb.hd) {
+    const int64_t r = idx - nkey;
+    const int j = (int)(r / tb.hd), m = (int)(r % tb.hd);
+    float s = 0.f, c = 1.f;
+    if (tb.use_rope) sincos_reduced((tb.qstart + (double)j * tb.qstep) * tb.omega_b[m], &s, &c);
+    tb.hrot[r] = make_float2(c, s);
   }
-  coarse[idx] = make_float4(c[0], c[1], s[0], s[1]);
-}
-
-// rot[j][m] = (cos, sin)(p_j * omega[m]), p_j = pstart + j * pstep, angle reduced in fp64;
-// (1, 0) when use_rope is 0.
-__global__ void heads_rot_kernel(float2* rot, int t, int hd, double pstart, double pstep,
-                                 const double* __restrict__ omega, int use_rope) {
-  griddep_wait();
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (int64_t)t * hd) return;
-  const int j = (int)(idx / hd), m = (int)(idx % hd);
-  float s = 0.f, c = 1.f;
-  if (use_rope) sincos_reduced((pstart + (double)j * pstep) * omega[m], &s, &c);
-  rot[idx] = make_float2(c, s);
 }
 
 // Thread = (latent j, 4 consecutive pairs m) x a share of the batches (blockIdx.y); the angles are
-// formed once and reused for every batch of the share. Bound by memory once enough rows are in
-// flight. Measured with one share and now: 64 batches of 164 x 1024 51 -> 26 us,
-// 32 of 251 x 1024 32 -> 25; from t = 655 up unchanged at 87% of the memory rate (one share). Columns are in pair-chunk order: pair m sits at f1 = (m / 128) * 256 + m % 128 and its
-// partner at f1 + 128, so four consecutive pairs are four consecutive columns.
-__global__ void q_rope_kernel(const float* __restrict__ qhat, int t_max, int b0, int nb, int t,
-                              int D, double qstart, double qstep, const double* omega_c,
-                              int use_rope, __nv_bfloat16* __restrict__ qhl, int fp16,
-                              float qscale) {
+// formed once and reused for every batch of the share. Columns are in pair-chunk order: pair m
+// sits at f1 = (m / 128) * 256 + m % 128 and its partner at f1 + 128, so four consecutive pairs
+// are four consecutive columns. Bound by memory once enough rows are in flight. Measured with one
+// share and now: 64 batches of 164 x 1024 51 -> 26 us, 32 of 251 x 1024 32 -> 25; from t = 655 up
+// unchanged at 87% of the memory rate (one share).
+__global__ void q_rope_kernel(const float* __restrict__ qhat, const float* __restrict__ scale,
+                              int t_max, int b0, int nb, int t, int D, double qstart,
+                              double qstep, const double* omega_c, int use_rope,
+                              __nv_bfloat16* __restrict__ qhl, int fp16, float qscale) {
   griddep_wait();
   const int half = D / 2, q4 = half / 4;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -301,7 +298,15 @@ __global__ void q_rope_kernel(const float* __restrict__ qhat, int t_max, int b0,
     const float* q = qhat + ((int64_t)(b0 + bb) * t_max + j) * D;
     const float4 x4 = *reinterpret_cast<const float4*>(q + f1);
     const float4 y4 = *reinterpret_cast<const float4*>(q + f2);
-    const float x[4] = {x4.x, x4.y, x4.z, x4.w}, y[4] = {y4.x, y4.y, y4.z, y4.w};
+    float x[4] = {x4.x, x4.y, x4.z, x4.w}, y[4] = {y4.x, y4.y, y4.z, y4.w};
+    if (scale != nullptr) {
+      const float f = scale[(int64_t)bb * t + j];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        x[e] *= f;
+        y[e] *= f;
+      }
+    }
     float a[4], b[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
@@ -1154,24 +1159,14 @@ cudaError_t launch_strip(const KVSource& src, int64_t N, int H, int d, const Pos
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_heads_rot(float2* rot, int t, int hd, double pstart, double pstep,
-                             const double* omega, int use_rope, cudaStream_t s) {
-  const int64_t n = (int64_t)t * hd;
-  launch_chained(heads_rot_kernel, blocks_for(n, 256), 256, 0, s, 1, rot, t, hd, pstart, pstep,
-                 omega, use_rope);
+cudaError_t launch_rope_tables(const RopeTables& tb, cudaStream_t s) {
+  const int64_t n = ((int64_t)tb.G + kPosGrain) * (tb.D / 4) + (int64_t)tb.t * tb.hd;
+  launch_chained(rope_tables_kernel, blocks_for(n, 256), 256, 0, s, 1, tb);
   return cudaGetLastError();
 }
 
-cudaError_t launch_rope_tables(float4* coarse, float* omega, int G, int D, double origin,
-                               const double* omega_c, cudaStream_t s) {
-  const int64_t n = (int64_t)(G + kPosGrain) * (D / 4);
-  launch_chained(rope_tables_kernel, blocks_for(n, 256), 256, 0, s, 1, coarse, omega, G, D, origin,
-                 omega_c);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_q_rope(const float* qhat, int t_max, int b0, int nb, int t, int D,
-                          double qstart, double qstep, const double* omega_c, int use_rope,
+cudaError_t launch_q_rope(const float* qhat, const float* scale, int t_max, int b0, int nb, int t,
+                          int D, double qstart, double qstep, const double* omega_c, int use_rope,
                           __nv_bfloat16* qhl, int fp16, float qscale, int num_sms,
                           cudaStream_t s) {
   if (D % 256 != 0) return cudaErrorInvalidValue;
@@ -1179,8 +1174,8 @@ cudaError_t launch_q_rope(const float* qhat, int t_max, int b0, int nb, int t, i
   const unsigned tiles = blocks_for(n, 256);
   // shares of the batches until each SM has three CTAs
   const unsigned shares = std::max(1u, std::min((unsigned)nb, 3u * num_sms / tiles));
-  launch_chained(q_rope_kernel, dim3(tiles, shares), 256, 0, s, 1, qhat, t_max, b0, nb, t, D,
-                 qstart, qstep, omega_c, use_rope, qhl, fp16, qscale);
+  launch_chained(q_rope_kernel, dim3(tiles, shares), 256, 0, s, 1, qhat, scale, t_max, b0, nb,
+                 t, D, qstart, qstep, omega_c, use_rope, qhl, fp16, qscale);
   return cudaGetLastError();
 }
 

@@ -81,24 +81,31 @@ cudaError_t launch_decode_biased(const DecodeStack& st, void* ws, int num_sms, c
 // become fp16 subnormals, absolute error <= 2^-25).
 cudaError_t launch_bf16_to_f16(void* p, int64_t n, cudaStream_t s);
 
-// rot[j][m] = (cos, sin)((pstart + j * pstep) * omega[m]) for j < t, m < hd (angle reduced
-// modulo 2 pi in fp64); (1, 0) when use_rope is 0. The output heads' re-rotation table.
-cudaError_t launch_heads_rot(float2* rot, int t, int hd, double pstart, double pstep,
-                             const double* omega, int use_rope, cudaStream_t s);
-
-// Compactor-RoPE tables: coarse[g][q] = (cos, cos, sin, sin) of pairs m = 2 q and 2 q + 1 at
-// (origin + g * kPosGrain) * w_m for g < G, then fine[q][i] at i * w_m for i < kPosGrain, at
-// coarse + G * D/4; omega[m] = w_m (fp32), w_m = omega_c[m] = theta_c^(-2m/D) (fp64 table),
-// angles reduced in fp64.
-cudaError_t launch_rope_tables(float4* coarse, float* omega, int G, int D, double origin,
-                               const double* omega_c, cudaStream_t s);
+// Angle tables of a call. Compactor RoPE: coarse[g][q] = (cos, cos, sin, sin) of pairs m = 2 q and
+// 2 q + 1 at (origin + g * kPosGrain) * w_m for g < G, then fine[q][i] at i * w_m for
+// i < kPosGrain, at coarse + G * D/4; omega[m] = w_m (fp32), w_m = omega_c[m] = theta_c^(-2m/D)
+// (fp64 table). Output heads' re-rotation: hrot[j][m] = (cos, sin)((qstart + j * qstep) *
+// omega_b[m]) for j < t, m < hd; (1, 0) when use_rope is 0. Angles are reduced modulo 2 pi in fp64.
+struct RopeTables {
+  float4* coarse = nullptr;
+  float* omega = nullptr;
+  const double* omega_c = nullptr;
+  int32_t G = 0, D = 0;
+  double origin = 0;
+  float2* hrot = nullptr;
+  const double* omega_b = nullptr;
+  int32_t t = 0, hd = 0, use_rope = 0;
+  double qstart = 0, qstep = 0;
+};
+cudaError_t launch_rope_tables(const RopeTables& tables, cudaStream_t s);
 
 // Per-call cross-attention queries: q = RoPE_c(q^, p_j) for latents j < t, batches
 // b in [b0, b0 + nb) (b = h * n + i), as hi/lo bf16 [nb * t][2D]. q^ is [H*n][t_max][D] fp32
-// in pair-chunk column order; p_j = qstart + j * qstep.
+// in pair-chunk column order; p_j = qstart + j * qstep. scale: factors [nb * t] of the rows of q^
+// (row b, j at b * t + j, b from 0), or null.
 // fp16: hi/lo in fp16 of (q * qscale) instead of bf16 of q (qscale a power of two).
-cudaError_t launch_q_rope(const float* qhat, int t_max, int b0, int nb, int t, int D,
-                          double qstart, double qstep, const double* omega_c, int use_rope,
+cudaError_t launch_q_rope(const float* qhat, const float* scale, int t_max, int b0, int nb, int t,
+                          int D, double qstart, double qstep, const double* omega_c, int use_rope,
                           __nv_bfloat16* qhl, int fp16, float qscale, int num_sms,
                           cudaStream_t s);
 

@@ -608,10 +608,23 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
   KLAUNCH(STILL_K_STRIP, launch_strip(src, N, H, d, pos.segs, L.omega_b, c.rope_fix, X, XT, Np,
                                       gd, pos.origin, P.G, L.f16 ? 1 : 0, fold_kp(L), ctx->nsm,
                                       s));
+  RopeTables tables;
+  tables.coarse = coarse;
+  tables.omega = omega;
+  tables.omega_c = L.omega_c;
+  tables.G = P.G;
+  tables.D = D;
+  tables.origin = pos.origin;
+  tables.hrot = hrot;
+  tables.omega_b = L.omega_b;
+  tables.t = t;
+  tables.hd = d / 2;
+  tables.use_rope = c.rope_fix;
+  tables.qstart = qstart;
+  tables.qstep = qstep;
+  KLAUNCH(STILL_K_TABLES, launch_rope_tables(tables, s));
   const int w_fmt = L.f16 ? 0 : 1;    // operand format of X, RMSNorm(Z), W_K and W_Q products
   const int zn_mode = L.f16 ? 2 : 1;  // RMSNorm(Z) as fp16 or bf16 hi | lo
-  KLAUNCH(STILL_K_TABLES, launch_rope_tables(coarse, omega, P.G, D, pos.origin, L.omega_c, s));
-  KLAUNCH(STILL_K_TABLES, launch_heads_rot(hrot, t, d / 2, qstart, qstep, L.omega_b, c.rope_fix, s));
   bf16* Zn = P.lazy_q ? reinterpret_cast<bf16*>(ws + P.oZn) : nullptr;
   const int64_t rows = (int64_t)H * t;
   const int n2d = n * 2 * d;
@@ -679,6 +692,7 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
     float* qt = reinterpret_cast<float*>(g);
     float* qss = reinterpret_cast<float*>(g + a256((size_t)t * D * 4) * nbl);
     const float* qsrc = L.qhat;  // [.][t_max][D], batch index b0 + local
+    const float* qscale_rows = nullptr;
     int q_tmax = c.t_max, q_b0 = b0;
     if (q_call) {
       // q~ = RMSNorm(Z) W_Q + b_Q (2-pass), as at weight load, for this group's (h, i) only
@@ -706,10 +720,10 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
       TRY(run_gemm256<STILL_K_LOAD>(ctx, op(Zn, (int64_t)H * t, 2 * D), op(Bw.WqT, (int64_t)n * D, D),
                                     p, e, w_fmt, s));
       const int64_t nq = (int64_t)nbl * t;
-      float* qinv = qss + nq * (2 * (D / 256));
+      float* qinv = qss + nq * (2 * (D / 256));  // applied by the rotation
       KLAUNCH(STILL_K_NORMS, launch_inv_norms(qss, nq, 2 * (D / 256), t, c.l2_eps, 1.f, qinv, s));
-      KLAUNCH(STILL_K_NORMS, launch_scale_rows(qt, qinv, nq, D, s));
       qsrc = qt;
+      qscale_rows = qinv;
       q_tmax = t;
       q_b0 = 0;
     }
@@ -764,8 +778,8 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
     KLAUNCH(STILL_K_NORMS, launch_inv_norms(kss, (int64_t)nbl * N, kparts, N, c.l2_eps,
                                             scale / qscale, kinv, s));
     if (!L.fold)
-      KLAUNCH(STILL_K_QROPE, launch_q_rope(qsrc, q_tmax, q_b0, nbl, t, D, qstart, qstep,
-                                           L.omega_c, c.compactor_rope, qhl,
+      KLAUNCH(STILL_K_QROPE, launch_q_rope(qsrc, qscale_rows, q_tmax, q_b0, nbl, t, D, qstart,
+                                           qstep, L.omega_c, c.compactor_rope, qhl,
                                            exact || tk ? 1 : 0, qscale, ctx->nsm, s));
     {
       // S, the online softmax and P X in one kernel; per-split partials merged in order.
