@@ -31,17 +31,6 @@ STILL_DEV bool warp_flag(volatile int* flag) {
   return __shfl_sync(0xffffffffu, *flag, 0) != 0;
 }
 
-// Registers per thread of a warpgroup from here on (every warp of the warpgroup executes it). An
-// increase waits for registers that other warpgroups of the CTA have given up.
-template <int N>
-STILL_DEV void set_max_regs_dec() {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
-}
-template <int N>
-STILL_DEV void set_max_regs_inc() {
-  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
-}
-
 STILL_DEV uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
@@ -152,21 +141,6 @@ STILL_DEV bool mbar_wait(uint64_t* bar, uint32_t parity) {
       if (mbar_try_wait(a, parity)) return true;
     if (globaltimer_ns() - t0 > STILL_WAIT_NS) return false;
   }
-}
-
-// ------------------------------------------------------------------------------- cp.async
-
-// 16 bytes into shared memory; with !ok nothing is read and the destination is zeroed.
-STILL_DEV void cp_async16(uint32_t dst, const void* src, bool ok) {
-  const int n = ok ? 16 : 0;
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n)
-               : "memory");
-}
-STILL_DEV void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-// Wait until at most N committed groups of this thread are pending.
-template <int N>
-STILL_DEV void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
 // ------------------------------------------------------------------------------- TMA
@@ -316,21 +290,6 @@ __host__ __device__ constexpr uint32_t idesc_f16(int M, int N, int ab_fmt) {
          | ((uint32_t)ab_fmt << 10)         // B format            [10, 13)
          | ((uint32_t)(N >> 3) << 17)       // N >> 3              [17, 23)
          | ((uint32_t)(M >> 4) << 24);      // M >> 4              [24, 29)
-}
-
-// 32 lanes x 16 consecutive fp32 columns: thread i of the warp receives lane (base + i).
-STILL_DEV void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-        "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // 32 lanes x 32 consecutive fp32 columns: thread i of the warp receives lane (base + i).

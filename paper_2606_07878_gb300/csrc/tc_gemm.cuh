@@ -88,24 +88,6 @@ struct GemmSmem {
 // Coalesced row store for one warp: lane i holds 64 bytes (v[0..3]) for its own row, to be
 // written at dst (16-byte aligned) if valid. The warp exchanges them through its staging area
 // so that each store instruction writes 8 rows x 64 contiguous bytes (whole 32-byte sectors).
-// As warp_store64 with 32 bytes per lane: each store instruction writes 16 rows x 32 bytes.
-__device__ __forceinline__ void warp_store32(uint4* stage, const uint4 (&v)[2], void* dst,
-                                             bool valid) {
-  const int lane = threadIdx.x & 31;
-  stage[lane * 3] = v[0];
-  stage[lane * 3 + 1] = v[1];
-  __syncwarp();
-  const unsigned long long mine = reinterpret_cast<unsigned long long>(dst);
-#pragma unroll
-  for (int it = 0; it < 2; ++it) {
-    const int r = it * 16 + (lane >> 1), q = lane & 1;
-    const unsigned long long d = __shfl_sync(0xffffffffu, mine, r);
-    const int ok = __shfl_sync(0xffffffffu, valid ? 1 : 0, r);
-    if (ok) reinterpret_cast<uint4*>(d)[q] = stage[r * 3 + q];
-  }
-  __syncwarp();
-}
-
 __device__ __forceinline__ void warp_store64(uint4* stage, const uint4 (&v)[4], void* dst,
                                              bool valid) {
   const int lane = threadIdx.x & 31;
