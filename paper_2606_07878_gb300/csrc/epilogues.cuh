@@ -5,6 +5,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <utility>
+
 #include "tc_gemm.cuh"
 
 namespace still {
@@ -159,7 +161,8 @@ struct EpiAffineT {
   int32_t tile_cols_ = 256;  // the tile width BN, set by the launcher
   bool can_split() const { return sumsq == nullptr || kChunkSums; }
   static constexpr bool kAnyTile = true;  // its 32-column chunks are independent
-  static constexpr bool kPairs = !kChunkSums;  // has a 2-SM form
+  static constexpr bool kPairs = !kChunkSums;  // has a 2-SM form, of these tile widths:
+  using Widths = std::integer_sequence<int, 256>;
 
   // The residual rows of this warp's columns are pulled into L2 while the main loop runs.
   template <class Src>
@@ -443,6 +446,7 @@ struct EpiQuad {
   bool can_split() const { return true; }
   static constexpr bool kAnyTile = true;
   static constexpr bool kPairs = true;
+  using Widths = std::integer_sequence<int, 192, 160>;  // Kp is 192 or 320
 
   template <class Src>
   __device__ void prefetch(const GemmParams&, const TileCoord&, int, const Src&, int) const {}

@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <utility>
 
 #include "epilogues.cuh"
 #include "launch.cuh"
@@ -202,24 +203,73 @@ inline cudaError_t launch_split(const CUtensorMap& ta, const CUtensorMap& tb,
                         GemmSmem<BN, Epi>::kBytes, stream, ranks, ta, tb, tc, p, epi);
 }
 
-// Pairs of CTAs of tc_gemm2_kernel when its waves take less time than those of the 1-SM kernel,
-// else 0. Measured clocks per K iteration, epilogue included: 720 for a 256 x 256 tile on two SMs,
-// 860 for a 128 x 256 tile on one (t = 1024, d_l = 1024). An odd number of m-tiles or a bad last
-// wave can make the pairs slower: t = 617, d_l = 2048, P v 488 us on single SMs, 584 on pairs.
-template <class Epi>
-inline int gemm2_clusters(const GemmParams& p, int num_sms) {
-  using S = Gemm2Smem<256, Epi>;
+// Clocks of tc_gemm2_kernel per K iteration of a 256 x bn tile on two SMs, epilogue included:
+// measured 720 at 256 columns (t = 1024, d_l = 1024) and, with the key norms' epilogue, 0.90 of
+// that at 160; taken as that at 192 too, the width that 192 columns take.
+inline int gemm2_clocks(int bn) { return bn < 256 ? 650 : 720; }
+
+// Resident pairs of tc_gemm2_kernel<BN, Epi> (0: none).
+template <int BN, class Epi>
+inline int gemm2_resident(int num_sms) {
   static thread_local int clusters = 0;
-  if (clusters == 0 && resident_pairs(tc_gemm2_kernel<256, Epi>, gemm_threads<Epi>(), S::kBytes,
-                                      num_sms, &clusters) != cudaSuccess) {
+  if (clusters == 0 && resident_pairs(tc_gemm2_kernel<BN, Epi>, gemm_threads<Epi>(),
+                                      Gemm2Smem<BN, Epi>::kBytes, num_sms, &clusters) !=
+                           cudaSuccess) {
     cudaGetLastError();
     clusters = 0;
-    return 0;
   }
+  return clusters;
+}
+
+// Time of a GEMM on pairs in clocks per K iteration: waves of its tiles.
+template <int BN, class Epi>
+inline int64_t gemm2_cost(const GemmParams& p, int num_sms) {
+  const int clusters = gemm2_resident<BN, Epi>(num_sms);
+  if (clusters == 0) return INT64_MAX;
+  const int64_t pairs = (int64_t)((p.tiles_m + 1) / 2) * ((p.N + BN - 1) / BN) * p.batch;
+  return (pairs + clusters - 1) / clusters * gemm2_clocks(BN);
+}
+
+template <int BN, class Epi>
+inline cudaError_t launch_pairs(const CUtensorMap& ta, const Operand2D& B, const CUtensorMap& tc,
+                                GemmParams p, Epi epi, int ab_fmt, int num_sms,
+                                cudaStream_t stream) {
+  CUtensorMap tb;
+  if (!finalize_gemm<BN>(p, ab_fmt) || !make_tmap(&tb, B, BN / 2)) return cudaErrorInvalidValue;
+  epi.tile_cols_ = BN;
   const int64_t pairs = (int64_t)((p.tiles_m + 1) / 2) * p.tiles_n * p.batch;
-  const int64_t waves1 = (p.ntiles + num_sms - 1) / num_sms;
-  const int64_t waves2 = (pairs + clusters - 1) / clusters;
-  return waves2 * 720 < waves1 * 860 ? (int)std::min<int64_t>(pairs, clusters) : 0;
+  const int clusters = (int)std::min<int64_t>(pairs, gemm2_resident<BN, Epi>(num_sms));
+  return launch_chained(tc_gemm2_kernel<BN, Epi>, 2 * clusters, gemm_threads<Epi>(),
+                        Gemm2Smem<BN, Epi>::kBytes, stream, 2, ta, tb, tc, p, epi);
+}
+
+// Launches the 2-SM kernel at the width of Epi::Widths that is fastest, if its waves are shorter
+// than the 1-SM kernel's (860 clocks per K iteration of a 128 x 256 tile). *launched says whether.
+// An odd number of m-tiles or a bad last wave can make the pairs slower: t = 617, d_l = 2048, P v
+// 488 us on single SMs, 584 on pairs. The key norms of the folded path have 320 columns, two tiles
+// of 160 or two of 256 with 192 columns of padding (170 -> 152 us at 8,192 tokens of 4 heads), or
+// 192. For the latent GEMMs widths of 192 and 224 gave the call 0.4% at t = 617 (better last
+// waves) and nothing elsewhere, and are not offered.
+template <class Epi, int... W>
+inline cudaError_t try_pairs(std::integer_sequence<int, W...>, const CUtensorMap& ta,
+                             const Operand2D& B, const CUtensorMap& tc, const GemmParams& p,
+                             const Epi& epi, int ab_fmt, int num_sms, cudaStream_t stream,
+                             bool* launched) {
+  int width = 0;
+  int64_t best = ((int64_t)p.ntiles + num_sms - 1) / num_sms * 860;
+  auto consider = [&](int64_t cost, int bn) {
+    if (cost < best) {
+      best = cost;
+      width = bn;
+    }
+  };
+  (consider(gemm2_cost<W, Epi>(p, num_sms), W), ...);
+  *launched = width != 0;
+  cudaError_t e = cudaSuccess;
+  ((width == W ? (void)(e = launch_pairs<W, Epi>(ta, B, tc, p, epi, ab_fmt, num_sms, stream))
+               : (void)0),
+   ...);
+  return e;
 }
 
 template <int BN, int kRole, class Epi>
@@ -249,11 +299,11 @@ inline cudaError_t launch_gemm(const Operand2D& A, const Operand2D& B, GemmParam
     if (ranks > 1) return launch_split<BN, Epi>(ta, tb, tc, p, epi, ranks, stream);
   }
   if constexpr (BN == 256 && Epi::kPairs) {
-    const int clusters = p.ksplit == 1 ? gemm2_clusters<Epi>(p, num_sms) : 0;
-    if (clusters > 0) {
-      if (!make_tmap(&tb, B, BN / 2)) return cudaErrorInvalidValue;
-      return launch_chained(tc_gemm2_kernel<BN, Epi>, 2 * clusters, gemm_threads<Epi>(),
-                            Gemm2Smem<BN, Epi>::kBytes, stream, 2, ta, tb, tc, p, epi);
+    if (p.ksplit == 1) {
+      bool launched = false;
+      const cudaError_t e = try_pairs(typename Epi::Widths(), ta, B, tc, p, epi, ab_fmt, num_sms,
+                                      stream, &launched);
+      if (launched) return e;
     }
   }
   auto kern = tc_gemm_kernel<BN, Epi, kRole>;

@@ -353,6 +353,8 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
 // P v 150 -> 128, head outputs 126 -> 107, v projection 103 -> 93, FFN 160 -> 147.
 template <int BN, class Epi>
 struct Gemm2Smem {
+  // MMAs of M = 256 take N in steps of 32; a B half must end on a swizzle atom of 8 rows
+  static_assert(BN > 128 && BN <= 256 && BN % 32 == 0, "tile width");
   static constexpr int kStages = 6;
   static constexpr int kABytes = kBM * kBK * 2;
   static constexpr int kBBytes = (BN / 2) * kBK * 2;
@@ -419,7 +421,7 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
     tma_prefetch_desc(&tmB);
   }
   if (warp == 1) {
-    tmem_alloc_2sm(tmem_slot, 2 * BN);
+    tmem_alloc_2sm(tmem_slot, 512);  // two accumulators of BN > 128 columns
     tmem_relinquish_2sm();
   }
   tc_fence_before();
@@ -584,7 +586,7 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
   cluster_sync();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc_2sm(tmem_base, 2 * BN);
+    tmem_dealloc_2sm(tmem_base, 512);
   }
 }
 

@@ -1,5 +1,6 @@
-"""Latent sublayers wide enough for the GEMM on CTA pairs (256 x 256 tiles) against the oracle: an
-odd number of row tiles, rows and columns that end inside a tile, and several waves."""
+"""Latent sublayers and folded key norms wide enough for the GEMM on CTA pairs (tiles of 256 x 160 to
+256 columns) against the oracle: an odd number of row tiles, rows and columns that end inside a
+tile, and several waves."""
 import pytest
 
 from gpu_helpers import Runner, assert_parity, oracle_layer
@@ -22,6 +23,22 @@ def test_wide_latent_sublayers_match_oracle(H, d, D, n, F, t):
         K, V = synth.gen_kv(wl, 0, device=DEV)
         Ck, Cv, _ = r.layer(0, K, V, t)
         rk, rv, _, _ = oracle_layer(wl, r.W[0], K, V, t)
+        for name, ref, got in (("C_k", rk, Ck), ("C_v", rv, Cv)):
+            assert_parity(ref, synth.bf16_to_f64(got), name)
+    finally:
+        r.close()
+
+
+@pytest.mark.parametrize("d,D", [(128, 512), (64, 256)])  # 320 and 192 columns of key norms
+def test_folded_key_norms_match_oracle(d, D):
+    t = 48
+    wl = synth.tiny_workload(H=4, d=d, D=D, n=4, F=0, N=3001, heavy=2, ts=(t,))
+    over = dict(compactor_rope=0)
+    r = Runner(wl, t, cfg_over=over)
+    try:
+        K, V = synth.gen_kv(wl, 0, device=DEV)
+        Ck, Cv, _ = r.layer(0, K, V, t)
+        rk, rv, _, _ = oracle_layer(wl, r.W[0], K, V, t, cfg_over=dict(compactor_rope=False))
         for name, ref, got in (("C_k", rk, Ck), ("C_v", rv, Cv)):
             assert_parity(ref, synth.bf16_to_f64(got), name)
     finally:
