@@ -347,15 +347,11 @@ bool value_hilo(const still_layer_config&) { return true; }
 // which is less to write and read.
 int64_t split_latents(int64_t H, int64_t n, int64_t D) { return 76 / (2 * n * D / 256) * 128 / H; }
 
-// Partials per vector at t latents, and the bytes of one vector's partials and inverse norm summed
-// over them: never less for more latents, so that a workspace reserved for more serves fewer.
-int sumsq_parts(int64_t H, int64_t n, int64_t D, int64_t t) {
-  return (int)(t <= split_latents(H, n, D) ? D / 32 : 2 * (D / 256));
-}
-int64_t sumsq_bytes(int64_t H, int64_t n, int64_t D, int64_t t) {
-  const int64_t ts = std::min(t, split_latents(H, n, D));
-  return 4 * std::max(ts * (D / 32 + 1), t * (2 * (D / 256) + 1));
-}
+// Sum-of-squares partials per self-attention q~ / k~ vector, and the bytes that T vectors' partials
+// and inverse norms take.
+int narrow_parts(int64_t D) { return (int)(2 * (D / 256)); }
+int wide_parts(int64_t D) { return (int)(D / 32); }
+size_t sumsq_bytes(int64_t vectors, int parts) { return a256(4 * vectors * (parts + 1)); }
 
 // The cross-attention scores of a one-block layer of head dim 256 (the kernel on clusters of
 // two CTAs) take one fp16 MMA pass (q_hi . k_hi) instead of three split-bf16 passes, and a
@@ -383,8 +379,8 @@ bool make_plan(const still_layer_config& c, bool lazy_q, int Kp, int64_t N, int 
   P.Np = rup(N, 64);
   P.tp = rup(t, 64);
   P.ldt = rup(t, 4);
-  // the table starts at most one grain before pmin (Positions::origin)
-  P.G = (int)std::floor((pmax - pmin) / kPosGrain) + 3;
+  // rows of the coarse table, which starts less than one grain before pmin (Positions::origin)
+  P.G = (int)std::floor((pmax - pmin) / kPosGrain) + 2;
   const int64_t H = P.H, d = P.d, D = P.D, n = P.n, F = P.F, T = t;
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -426,17 +422,14 @@ bool make_plan(const still_layer_config& c, bool lazy_q, int Kp, int64_t N, int 
   P.cand_b = one_pass_scores(c) && Kp == 0 ? 2 * a256(T * kTopLists * kTopK * 4) * kMaxFlashSplit
                                            : 0;
   // lazy q^: fp32 q~ of the unit and its sum-of-squares partials + inverse norms
-  P.sq_parts = sumsq_parts(H, n, D, T);
   P.qt_b = lazy_q ? a256(T * D * 4) + a256(T * 4 * (2 * (D / 256) + 1)) : 0;
   P.ca_unit_bytes = P.kb_b + P.kss_b + P.q_b + P.P_b + P.O_b + P.qt_b + P.cand_b;
   P.qk_b = a256(2 * n * T * 2 * D * 2);
-  P.sss_b = a256(2 * n * sumsq_bytes(H, n, D, T));
   P.vT_b = a256(n * D * P.tp * 2 * hl);
   P.Ssa_b = a256(n * T * P.ldt * 4);
   P.Psa_b = a256(n * T * P.tp * 2 * hl);
   P.Ssah_b = (size_t)T * P.ldt * 4;
   P.Psah_b = (size_t)T * P.tp * 2 * hl;
-  P.sa_unit_bytes = P.qk_b + P.sss_b + P.vT_b + P.Ssa_b + P.Psa_b;
   if (fixed >= limit) return false;
   const size_t avail = limit - fixed;
   // Cross-attention groups: whole KV-heads when possible, else a part of one head.
@@ -446,13 +439,19 @@ bool make_plan(const still_layer_config& c, bool lazy_q, int Kp, int64_t N, int 
   if (u >= n)
     u = (u / n) * n;
   P.ca_units = (int)u;
-  int64_t sh = std::min<int64_t>(H, (int64_t)(avail / P.sa_unit_bytes));
-  size_t sa_bytes;
-  if (sh >= 1) {
-    P.sa_heads = (int)sh;
-    P.sa_sub = (int)n;
-    sa_bytes = P.sa_unit_bytes * P.sa_heads;
-  } else {
+  // Self-attention groups with that many partials per vector; false when nothing fits.
+  size_t sa_bytes = 0;
+  auto plan_sa = [&](int parts) {
+    P.sq_parts = parts;
+    P.sss_b = sumsq_bytes(2 * n * T, parts);
+    P.sa_unit_bytes = P.qk_b + P.sss_b + P.vT_b + P.Ssa_b + P.Psa_b;
+    const int64_t sh = std::min<int64_t>(H, (int64_t)(avail / P.sa_unit_bytes));
+    if (sh >= 1) {
+      P.sa_heads = (int)sh;
+      P.sa_sub = (int)n;
+      sa_bytes = P.sa_unit_bytes * P.sa_heads;
+      return true;
+    }
     // One bank at a time, its self heads in sub-groups (scores and probabilities per head).
     const size_t bank = P.qk_b + P.sss_b + P.vT_b;
     const size_t head = P.Ssah_b + P.Psah_b;
@@ -460,10 +459,32 @@ bool make_plan(const still_layer_config& c, bool lazy_q, int Kp, int64_t N, int 
     P.sa_heads = 1;
     P.sa_sub = (int)std::min<int64_t>(n, (int64_t)((avail - bank - 1024) / head));
     sa_bytes = bank + a256(P.sa_sub * P.Ssah_b) + a256(P.sa_sub * P.Psah_b);
+    return true;
+  };
+  // The finer sums only where their bytes cost no group: a limit that holds the call with one
+  // partial per 128 columns holds it with the same groups here.
+  if (!plan_sa(narrow_parts(D))) return false;
+  if (T <= split_latents(H, n, D)) {
+    const int heads = P.sa_heads, sub = P.sa_sub;
+    if (!plan_sa(wide_parts(D)) || P.sa_heads != heads || P.sa_sub != sub)
+      plan_sa(narrow_parts(D));
   }
   P.oCA = off;
   P.oSA = off;  // the two phases reuse the same region
   P.total = off + std::max(P.ca_unit_bytes * P.ca_units, sa_bytes);
+  return true;
+}
+
+// Workspace of every call of up to N tokens and up to t latents. A call's need grows with both but
+// for the finer sums of squares, which end at split_latents: the larger of the two sides.
+bool plan_reserve(const still_layer_config& c, bool lazy_q, int Kp, int64_t N, int t, size_t limit,
+                  size_t* bytes) {
+  Plan P;
+  if (!make_plan(c, lazy_q, Kp, N, t, 0.0, (double)(N - 1), limit, P)) return false;
+  *bytes = P.total;
+  const int64_t ts = split_latents(c.n_kv_heads, c.n_cross_heads, c.d_latent);
+  if (ts >= 1 && ts < t && make_plan(c, lazy_q, Kp, N, (int)ts, 0.0, (double)(N - 1), limit, P))
+    *bytes = std::max(*bytes, P.total);
   return true;
 }
 
@@ -936,7 +957,7 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
         return run_gemm256<STILL_K_SA_PROJ>(ctx, op(A1, rows, 2 * D),
                                             op(Bw.SqkT, (int64_t)2 * n * D, D), p, e, vfmt, s);
       };
-      TRY(sparts == D / 32 ? project(EpiAffineT<true>()) : project(EpiAffine()));
+      TRY(sparts == wide_parts(D) ? project(EpiAffineT<true>()) : project(EpiAffine()));
     }
     KLAUNCH(STILL_K_NORMS,
             launch_inv_norms(sss, (int64_t)nh * 2 * n * t, sparts, t, c.l2_eps, 1.f, sinv, s));
@@ -1975,13 +1996,10 @@ still_status still_workspace_size(const still_ctx* ctx, int64_t max_tokens, int3
   if (ctx == nullptr || bytes == nullptr || ctx->layers.empty() || !ctx->layers[0].loaded)
     return ctx == nullptr || bytes == nullptr ? STILL_ERR_INVALID_ARG : STILL_ERR_NOT_LOADED;
   if (max_tokens < 1 || max_t < 1 || max_t > max_tokens) return STILL_ERR_SHAPE;
-  Plan P;
-  if (!make_plan(ctx->layers[0].cfg, queries_per_call(ctx->layers[0]), fold_kp(ctx->layers[0]),
-                 max_tokens, max_t, 0.0,
-                 (double)(max_tokens - 1), ctx->ws_limit, P))
-    return STILL_ERR_OOM;
-  *bytes = P.total;
-  return STILL_OK;
+  const LayerW& L = ctx->layers[0];
+  return plan_reserve(L.cfg, queries_per_call(L), fold_kp(L), max_tokens, max_t, ctx->ws_limit, bytes)
+             ? STILL_OK
+             : STILL_ERR_OOM;
 }
 
 still_status still_reserve_workspace(still_ctx* ctx, int64_t max_tokens, int32_t max_t) {
@@ -2067,6 +2085,29 @@ int64_t still_param_count(const still_layer_config* cfg, int32_t t) {
   const int64_t B = cfg->n_blocks, Bc = cfg->cross_every_block ? B : 1;
   return H * t * D + Bc * (2 * nc * D * D + 4 * d * nc * D) + B * (4 * ns * D * D) +
          B * (2 * F * D) + (2 * D * d + D);
+}
+
+// Host-only views of the library's rules, for its tests; not part of the ABI in still.h.
+
+// The plan of a call: bytes, (h, i) pairs per cross-attention group, KV-heads and self heads per
+// self-attention group, sum-of-squares partials per vector. 0 when the limit is too small.
+int still_internal_plan(const still_layer_config* cfg, int32_t lazy_q, int32_t Kp, int64_t N,
+                        int32_t t, double pmin, double pmax, size_t limit, int64_t out[5]) {
+  Plan P;
+  if (!make_plan(*cfg, lazy_q != 0, Kp, N, t, pmin, pmax, limit, P)) return 0;
+  out[0] = (int64_t)P.total;
+  out[1] = P.ca_units;
+  out[2] = P.sa_heads;
+  out[3] = P.sa_sub;
+  out[4] = P.sq_parts;
+  return 1;
+}
+
+// Bytes that still_reserve_workspace takes; 0 when the limit is too small.
+size_t still_internal_reserve(const still_layer_config* cfg, int32_t lazy_q, int32_t Kp, int64_t N,
+                              int32_t t, size_t limit) {
+  size_t bytes = 0;
+  return plan_reserve(*cfg, lazy_q != 0, Kp, N, t, limit, &bytes) ? bytes : 0;
 }
 
 }  // extern "C"

@@ -73,6 +73,25 @@ def test_noalloc_smaller_groups_meet_the_oracle_bar():
         r.close()
 
 
+@pytest.mark.parametrize("H,d,D,n,F,N,t", [
+    (1, 64, 256, 4, 1024, 1856, 1597),  # fits by less than the finer sums of squares would take
+    (1, 128, 512, 8, 0, 5115, 639),     # takes the coarse sums to fit
+])
+def test_noalloc_serves_calls_that_just_fit(H, d, D, n, F, N, t):
+    wl = synth.tiny_workload(H=H, d=d, D=D, n=n, F=F, N=N, heavy=2, ts=(t,))
+    r = Runner(wl, t)
+    try:
+        K, V = synth.gen_kv(wl, 0, device=DEV)
+        Ck, Cv = r.out(t)
+        still.still_compact_layer_noalloc(r.ctx, 0, K, V, t, Ck, Cv)
+        r.check_status()
+        rk, rv, _, _ = oracle_layer(wl, r.W[0], K, V, t)
+        assert_parity(rk, synth.bf16_to_f64(Ck), "C_k")
+        assert_parity(rv, synth.bf16_to_f64(Cv), "C_v")
+    finally:
+        r.close()
+
+
 def test_noalloc_rejects_sizes_beyond_the_scratch():
     wl = dict(synth.WORKLOADS["tiny_1k"])
     t = wl["ts"][0]
