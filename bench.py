@@ -19,6 +19,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -60,8 +61,8 @@ def describe(name, wl, t):
             f"({round(wl['N'] / t)}x)")
 
 # DRAM traffic (read + write) per launch of the dominant kernel at a workload, from an ncu
-# capture; valid only for the kernel sources it was taken on, or later ones that load and store
-# the same (hash of the listed sources).
+# capture; valid only for the kernel code it was taken on (hash of the listed sources without
+# their comments and layout).
 # The fused cross-attention kernel (the scores GEMM entry is kept for the record: no workload
 # takes it any more).
 TRAFFIC = {
@@ -70,27 +71,34 @@ TRAFFIC = {
     "ca_fused": [
         # 1.325 GB read + 0.125 GB written per launch (profiles/ca_fused_qwen7b_8k_t1024.md,
         # the CTA-pair kernel, whose source is ca_flash.cuh)
-        {"files": ["ca_flash.cuh"], "kernel_hash": "8bcaa4bfd11a12d5",
+        {"files": ["ca_flash.cuh"], "kernel_hash": "beeaf9187b20f38b",
          "bytes_per_launch": 1.4500e9, "workload": ("qwen7b_8k", 1024),
          "profile": "profiles/ca_fused_qwen7b_8k_t1024.md"},
         # the head-dim-256 kernel (source ca_pair.cu) captured on one KV-head of a 16k-token
         # cache (1.234 GB read + 0.091 GB written, profiles/ca_pair_gemma_n16k_t655.md), scaled
         # by the units of a full-size launch (2 KV-heads x 131072 tokens: x16); its traffic (k
         # read once, X^T, partials) grows in proportion
-        {"files": ["ca_pair.cu"], "kernel_hash": "92e60bc557ded1a8",
+        {"files": ["ca_pair.cu"], "kernel_hash": "2dddaaf20878659d",
          "bytes_per_launch": 16 * 1.3253e9, "workload": ("gemma_128k", 655),
          "profile": "profiles/ca_pair_gemma_n16k_t655.md"},
     ],
 }
 
 
+def _code_only(src):
+    """C++ source without comments and with every run of blanks as one space."""
+    src = re.sub(r'"(?:\\.|[^"\\\n])*"|//[^\n]*|/\*.*?\*/',
+                 lambda m: m.group() if m.group()[0] == '"' else " ", src, flags=re.S)
+    return " ".join(src.split())
+
+
 def _kernel_hash(files):
     h = hashlib.sha256()
     d = os.path.join(ROOT, "paper_2606_07878_gb300", "csrc")
     for f in files:
-        with open(os.path.join(d, f), "rb") as fh:
+        with open(os.path.join(d, f), encoding="utf-8") as fh:
             h.update(f.encode())
-            h.update(fh.read())
+            h.update(_code_only(fh.read()).encode())
     return h.hexdigest()[:16]
 
 

@@ -73,6 +73,14 @@ def test_describe_names_the_shape():
     assert math.isclose(65536 / 1311, 49.99, rel_tol=1e-3)
 
 
+def test_kernel_hash_covers_the_code_and_not_its_comments():
+    src = 'x = a / b;  // ratio\n/* of\n two */ y("//no comment");'
+    assert bench._code_only(src) == 'x = a / b; y("//no comment");'
+    assert bench._code_only(src.replace("ratio", "share")) == bench._code_only(src)
+    assert bench._code_only(src.replace("a / b", "b / a")) != bench._code_only(src)
+    assert bench._code_only('y("a")') != bench._code_only('y("b")')
+
+
 def test_traffic_records_name_existing_profiles_and_current_kernels():
     """Every DRAM-traffic record of the bench line points at a committed ncu summary and was
     taken on the kernel source as it is now (otherwise the bench would silently report null)."""
