@@ -671,8 +671,9 @@ inline int flash_split(int64_t base_units, int tiles_k, int num_sms, int max_spl
 // The kernel runs on CTA pairs (clusters of two): f.nunits counts (query-tile pair, key split,
 // batch) units.
 template <int D2, bool EX = false>
-inline cudaError_t launch_ca_flash(const Operand2D& Q, const Operand2D& K, const Operand2D& XT,
-                                   const FlashParams& f, int num_sms, cudaStream_t stream) {
+inline cudaError_t launch_ca_flash(const KernelTable& dev, const Operand2D& Q, const Operand2D& K,
+                                   const Operand2D& XT, const FlashParams& f,
+                                   cudaStream_t stream) {
   using S = FlashSmem<D2, EX>;
   if (f.D <= 0 || f.D % kBK != 0 || f.t <= 0 || f.N <= 0 || f.Np % kBK != 0 || f.Np < f.N ||
       f.nunits <= 0)
@@ -682,28 +683,24 @@ inline cudaError_t launch_ca_flash(const Operand2D& Q, const Operand2D& K, const
   if (!make_tmap(&tq, Q, kBM) || !make_tmap(&tk, K, S::kKeys / 2) ||
       !make_tmap(&thi, XT, D2 / 2) || !make_tmap(&tlo, XT, D2 / 4))
     return cudaErrorInvalidValue;
-  auto kern = ca_flash_kernel<D2, EX>;
-  static thread_local int clusters = 0;  // resident CTA pairs (per instantiation)
-  if (clusters == 0) {
-    const cudaError_t e = resident_pairs(kern, kFlashThreads, S::kBytes, num_sms, &clusters);
-    if (e != cudaSuccess) return e;
-  }
-  return launch_chained(kern, 2 * std::min(f.nunits, clusters), kFlashThreads, S::kBytes, stream, 2,
-                        tq, tk, thi, tlo, f);
+  using Id = KernelId<ca_flash_kernel<D2, EX>, kFlashThreads, S::kBytes, 2>;
+  if (dev.of<Id>().status != cudaSuccess) return dev.of<Id>().status;
+  return launch_chained(ca_flash_kernel<D2, EX>,
+                        2 * std::min(f.nunits, dev.persistent_clusters<Id>(2)), kFlashThreads,
+                        S::kBytes, stream, 2, tq, tk, thi, tlo, f);
 }
 
 // 2d = 512 (head dim 256): the same computation on clusters of four CTAs, two query tiles x
 // two column halves; the CTAs of a query tile split the O columns and take turns computing S,
 // the two CTAs of a half run their MMAs as one 2-SM MMA over both query tiles (ca_pair.cu). Q, K as for launch_ca_flash;
 // XT: [H*512][2*Np] fp16 (hi | lo). f.nunits counts (query-tile pair, key split, batch) units.
-// num_sms: SMs of the device (four per cluster).
 // one_pass: q, k as fp16 hi | lo with S from the hi parts only (one MMA pass) and repair
 // candidates in f.cand_key / f.cand_c for ca_topk_repair; else 3-pass split-bf16 scores.
-cudaError_t launch_ca_pair(const Operand2D& Q, const Operand2D& K, const Operand2D& XT,
-                           const FlashParams& f, int num_sms, cudaStream_t stream,
+cudaError_t launch_ca_pair(const KernelTable& dev, const Operand2D& Q, const Operand2D& K,
+                           const Operand2D& XT, const FlashParams& f, cudaStream_t stream,
                            bool one_pass = false);
 // Four-CTA clusters of that kernel that can be resident at once (its persistent grid size).
-int ca_pair_clusters(int num_sms);
+int ca_pair_clusters(const KernelTable& dev);
 
 // Top-k repair of one-pass scores: for each (b, row), over the splits whose running max is within
 // `cut` (log2 units) of the row's largest, each candidate's exact logit

@@ -912,41 +912,20 @@ cudaError_t launch_ca_topk_repair(const TopkRepairParams& f, int d2, cudaStream_
   return cudaGetLastError();
 }
 
-// The persistent grid holds no more clusters than can be resident at once (a cluster needs two
+namespace {
+template <bool kOnePass>
+using PairKernel = KernelId<ca_pair_kernel<kOnePass>, kFlashThreads, PairSmem::kBytes, kPairCluster>;
+}  // namespace
+
+// The persistent grid holds no more clusters than can be resident at once (a cluster needs four
 // free SMs of one GPC): a cluster that waited for another to exit would start its whole share
 // of the units late.
-int ca_pair_clusters(int num_sms) {
-  static thread_local int resident = 0;
-  const int most = std::max(1, num_sms / kPairCluster);
-  if (resident == 0) {
-    if (cudaFuncSetAttribute(ca_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             PairSmem::kBytes) != cudaSuccess) {
-      cudaGetLastError();
-      return most;
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kPairCluster * most, 1, 1);
-    cfg.blockDim = dim3(kFlashThreads, 1, 1);
-    cfg.dynamicSmemBytes = PairSmem::kBytes;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kPairCluster;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, ca_pair_kernel<false>, &cfg) != cudaSuccess || n < 1) {
-      cudaGetLastError();
-      n = most;
-    }
-    resident = std::max(1, std::min(n, most));
-  }
-  return resident;
+int ca_pair_clusters(const KernelTable& dev) {
+  return dev.persistent_clusters<PairKernel<false>>(kPairCluster);
 }
 
-cudaError_t launch_ca_pair(const Operand2D& Q, const Operand2D& K, const Operand2D& XT,
-                           const FlashParams& f, int num_sms, cudaStream_t stream,
+cudaError_t launch_ca_pair(const KernelTable& dev, const Operand2D& Q, const Operand2D& K,
+                           const Operand2D& XT, const FlashParams& f, cudaStream_t stream,
                            bool one_pass) {
   using S = PairSmem;
   if (f.D <= 0 || f.D % kBK != 0 || f.t <= 0 || f.N <= 0 || f.Np % kBK != 0 || f.Np < f.N ||
@@ -957,14 +936,10 @@ cudaError_t launch_ca_pair(const Operand2D& Q, const Operand2D& K, const Operand
   if (!make_tmap(&tq, Q, kBM) || !make_tmap(&tk, K, kPairKeys / 2) || !make_tmap(&tx, XT, 64))
     return cudaErrorInvalidValue;
   auto kern = one_pass ? ca_pair_kernel<true> : ca_pair_kernel<false>;
-  static thread_local bool attr_set[2] = {false, false};
-  if (!attr_set[one_pass]) {
-    cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kBytes);
-    if (e != cudaSuccess) return e;
-    attr_set[one_pass] = true;
-  }
-  const int clusters = std::max(1, std::min(f.nunits, ca_pair_clusters(num_sms)));
+  const cudaError_t ready = one_pass ? dev.of<PairKernel<true>>().status
+                                     : dev.of<PairKernel<false>>().status;
+  if (ready != cudaSuccess) return ready;
+  const int clusters = std::min(f.nunits, ca_pair_clusters(dev));
   return launch_chained(kern, kPairCluster * clusters, kFlashThreads, S::kBytes, stream,
                         kPairCluster, tq, tk, tx, f);
 }

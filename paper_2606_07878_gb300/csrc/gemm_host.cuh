@@ -10,6 +10,7 @@
 #include <utility>
 
 #include "epilogues.cuh"
+#include "kernel_table.cuh"
 #include "launch.cuh"
 
 namespace still {
@@ -102,73 +103,17 @@ inline bool finalize_gemm(GemmParams& p, int ab_fmt) {
   return true;
 }
 
-// Sets the kernel's shared-memory size and finds how many clusters of two CTAs can be resident.
-template <class Kern>
-inline cudaError_t resident_pairs(Kern kern, int threads, int smem, int num_sms, int* clusters) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t q = {};
-  q.gridDim = dim3(2 * std::max(1, num_sms / 2), 1, 1);
-  q.blockDim = dim3(threads, 1, 1);
-  q.dynamicSmemBytes = smem;
-  cudaLaunchAttribute qa[1];
-  qa[0].id = cudaLaunchAttributeClusterDimension;
-  qa[0].val.clusterDim.x = 2;
-  qa[0].val.clusterDim.y = 1;
-  qa[0].val.clusterDim.z = 1;
-  q.attrs = qa;
-  q.numAttrs = 1;
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, kern, &q) != cudaSuccess || n < 1) {
-    cudaGetLastError();
-    n = num_sms / 2;
-  }
-  *clusters = std::max(1, std::min(n, num_sms / 2));
-  return cudaSuccess;
-}
-
-// Clusters of `size` CTAs of a kernel that can be resident at once (its shared-memory size set).
-template <class Kern>
-inline int resident_clusters(Kern kern, int size, int threads, int smem, int num_sms) {
-  cudaLaunchConfig_t q = {};
-  q.gridDim = dim3(size * std::max(1, num_sms / size), 1, 1);
-  q.blockDim = dim3(threads, 1, 1);
-  q.dynamicSmemBytes = smem;
-  cudaLaunchAttribute qa[1];
-  qa[0].id = cudaLaunchAttributeClusterDimension;
-  qa[0].val.clusterDim.x = size;
-  qa[0].val.clusterDim.y = 1;
-  qa[0].val.clusterDim.z = 1;
-  q.attrs = qa;
-  q.numAttrs = 1;
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, kern, &q) != cudaSuccess || n < 1) {
-    cudaGetLastError();
-    return 0;
-  }
-  return std::min(n, num_sms / size);
-}
-
-constexpr int kMaxSplit = 8;
-
-// Clusters of each size of tc_gemm_split_kernel<BN, Epi> that can be resident at once (0: none).
+// The kernels' places in the context's table.
+template <int BN, class Epi, int kRole>
+using SingleId =
+    KernelId<tc_gemm_kernel<BN, Epi, kRole>, gemm_threads<Epi>(), GemmSmem<BN, Epi>::kBytes>;
 template <int BN, class Epi>
-inline const int* split_resident(int num_sms) {
-  using S = GemmSmem<BN, Epi>;
-  auto kern = tc_gemm_split_kernel<BN, Epi>;
-  static thread_local int resident[kMaxSplit + 1] = {0};  // [0]: asked
-  if (resident[0] == 0) {
-    resident[0] = 1;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kBytes) !=
-        cudaSuccess) {
-      cudaGetLastError();
-      return resident;
-    }
-    for (int s = 2; s <= kMaxSplit; ++s)
-      resident[s] = resident_clusters(kern, s, gemm_threads<Epi>(), S::kBytes, num_sms);
-  }
-  return resident;
-}
+using PairId =
+    KernelId<tc_gemm2_kernel<BN, Epi>, gemm_threads<Epi>(), Gemm2Smem<BN, Epi>::kBytes, 2>;
+constexpr int kMaxSplit = 8;
+template <int BN, class Epi>
+using SplitId = KernelId<tc_gemm_split_kernel<BN, Epi>, gemm_threads<Epi>(),
+                         GemmSmem<BN, Epi>::kBytes, 2, kMaxSplit>;
 
 // CTAs per tile of the split kernel at tile width BN for a GEMM of `ntiles` such tiles: the count
 // that is fastest by the clocks of its parts (measured on 128-row tiles at about 1.9 GHz: 384 /
@@ -176,10 +121,10 @@ inline const int* split_resident(int num_sms) {
 // all but one of the partials of 256 columns through DSMEM, 1400 to write one; 2500 per 32
 // columns in the epilogue; 4000 to start), with all clusters resident at once. *cost: its clocks.
 template <int BN, class Epi>
-inline int split_ranks(int64_t ntiles, int iters, int num_sms, double* cost) {
+inline int split_ranks(const KernelTable& dev, int64_t ntiles, int iters, double* cost) {
   *cost = 1e30;
-  if (ntiles > num_sms / 2) return 1;
-  const int* resident = split_resident<BN, Epi>(num_sms);
+  if (ntiles > dev.num_sms / 2) return 1;
+  const int* resident = dev.of<SplitId<BN, Epi>>().clusters;
   int best = 1;
   for (int s = 2; s <= std::min(kMaxSplit, iters); ++s) {
     if (ntiles > resident[s]) continue;
@@ -208,37 +153,25 @@ inline cudaError_t launch_split(const CUtensorMap& ta, const CUtensorMap& tb,
 // that at 160; taken as that at 192 too, the width that 192 columns take.
 inline int gemm2_clocks(int bn) { return bn < 256 ? 650 : 720; }
 
-// Resident pairs of tc_gemm2_kernel<BN, Epi> (0: none).
-template <int BN, class Epi>
-inline int gemm2_resident(int num_sms) {
-  static thread_local int clusters = 0;
-  if (clusters == 0 && resident_pairs(tc_gemm2_kernel<BN, Epi>, gemm_threads<Epi>(),
-                                      Gemm2Smem<BN, Epi>::kBytes, num_sms, &clusters) !=
-                           cudaSuccess) {
-    cudaGetLastError();
-    clusters = 0;
-  }
-  return clusters;
-}
-
 // Time of a GEMM on pairs in clocks per K iteration: waves of its tiles.
 template <int BN, class Epi>
-inline int64_t gemm2_cost(const GemmParams& p, int num_sms) {
-  const int clusters = gemm2_resident<BN, Epi>(num_sms);
-  if (clusters == 0) return INT64_MAX;
+inline int64_t gemm2_cost(const KernelTable& dev, const GemmParams& p) {
+  if (dev.of<PairId<BN, Epi>>().status != cudaSuccess) return INT64_MAX;
+  const int clusters = dev.persistent_clusters<PairId<BN, Epi>>(2);
   const int64_t pairs = (int64_t)((p.tiles_m + 1) / 2) * ((p.N + BN - 1) / BN) * p.batch;
   return (pairs + clusters - 1) / clusters * gemm2_clocks(BN);
 }
 
 template <int BN, class Epi>
-inline cudaError_t launch_pairs(const CUtensorMap& ta, const Operand2D& B, const CUtensorMap& tc,
-                                GemmParams p, Epi epi, int ab_fmt, int num_sms,
+inline cudaError_t launch_pairs(const KernelTable& dev, const CUtensorMap& ta, const Operand2D& B,
+                                const CUtensorMap& tc, GemmParams p, Epi epi, int ab_fmt,
                                 cudaStream_t stream) {
   CUtensorMap tb;
   if (!finalize_gemm<BN>(p, ab_fmt) || !make_tmap(&tb, B, BN / 2)) return cudaErrorInvalidValue;
   epi.tile_cols_ = BN;
   const int64_t pairs = (int64_t)((p.tiles_m + 1) / 2) * p.tiles_n * p.batch;
-  const int clusters = (int)std::min<int64_t>(pairs, gemm2_resident<BN, Epi>(num_sms));
+  const int clusters =
+      (int)std::min<int64_t>(pairs, dev.persistent_clusters<PairId<BN, Epi>>(2));
   return launch_chained(tc_gemm2_kernel<BN, Epi>, 2 * clusters, gemm_threads<Epi>(),
                         Gemm2Smem<BN, Epi>::kBytes, stream, 2, ta, tb, tc, p, epi);
 }
@@ -251,30 +184,30 @@ inline cudaError_t launch_pairs(const CUtensorMap& ta, const Operand2D& B, const
 // 192. For the latent GEMMs widths of 192 and 224 gave the call 0.4% at t = 617 (better last
 // waves) and nothing elsewhere, and are not offered.
 template <class Epi, int... W>
-inline cudaError_t try_pairs(std::integer_sequence<int, W...>, const CUtensorMap& ta,
-                             const Operand2D& B, const CUtensorMap& tc, const GemmParams& p,
-                             const Epi& epi, int ab_fmt, int num_sms, cudaStream_t stream,
-                             bool* launched) {
+inline cudaError_t try_pairs(const KernelTable& dev, std::integer_sequence<int, W...>,
+                             const CUtensorMap& ta, const Operand2D& B, const CUtensorMap& tc,
+                             const GemmParams& p, const Epi& epi, int ab_fmt,
+                             cudaStream_t stream, bool* launched) {
   int width = 0;
-  int64_t best = ((int64_t)p.ntiles + num_sms - 1) / num_sms * 860;
+  int64_t best = ((int64_t)p.ntiles + dev.num_sms - 1) / dev.num_sms * 860;
   auto consider = [&](int64_t cost, int bn) {
     if (cost < best) {
       best = cost;
       width = bn;
     }
   };
-  (consider(gemm2_cost<W, Epi>(p, num_sms), W), ...);
+  (consider(gemm2_cost<W, Epi>(dev, p), W), ...);
   *launched = width != 0;
   cudaError_t e = cudaSuccess;
-  ((width == W ? (void)(e = launch_pairs<W, Epi>(ta, B, tc, p, epi, ab_fmt, num_sms, stream))
+  ((width == W ? (void)(e = launch_pairs<W, Epi>(dev, ta, B, tc, p, epi, ab_fmt, stream))
                : (void)0),
    ...);
   return e;
 }
 
 template <int BN, int kRole, class Epi>
-inline cudaError_t launch_gemm(const Operand2D& A, const Operand2D& B, GemmParams p, Epi epi,
-                               int ab_fmt, int num_sms, cudaStream_t stream,
+inline cudaError_t launch_gemm(const KernelTable& dev, const Operand2D& A, const Operand2D& B,
+                               GemmParams p, Epi epi, int ab_fmt, cudaStream_t stream,
                                const StoreView3D* out_view = nullptr) {
   using S = GemmSmem<BN, Epi>;
   if (!finalize_gemm<BN>(p, ab_fmt)) return cudaErrorInvalidValue;
@@ -285,11 +218,11 @@ inline cudaError_t launch_gemm(const Operand2D& A, const Operand2D& B, GemmParam
   epi.tile_cols_ = BN;
   if (epi.can_split() && p.ksplit == 1) {
     double cost = 0, cost64 = 1e30;
-    const int ranks = split_ranks<BN, Epi>(p.ntiles, p.iters_total, num_sms, &cost);
+    const int ranks = split_ranks<BN, Epi>(dev, p.ntiles, p.iters_total, &cost);
     if constexpr (Epi::kAnyTile && BN != 64) {  // narrower tiles: less to reduce per CTA
       GemmParams q = p;
       if (!finalize_gemm<64>(q, ab_fmt)) return cudaErrorInvalidValue;
-      const int ranks64 = split_ranks<64, Epi>(q.ntiles, q.iters_total, num_sms, &cost64);
+      const int ranks64 = split_ranks<64, Epi>(dev, q.ntiles, q.iters_total, &cost64);
       if (ranks64 > 1 && cost64 < cost) {
         if (!make_tmap(&tb, B, 64)) return cudaErrorInvalidValue;
         epi.tile_cols_ = 64;
@@ -301,21 +234,16 @@ inline cudaError_t launch_gemm(const Operand2D& A, const Operand2D& B, GemmParam
   if constexpr (BN == 256 && Epi::kPairs) {
     if (p.ksplit == 1) {
       bool launched = false;
-      const cudaError_t e = try_pairs(typename Epi::Widths(), ta, B, tc, p, epi, ab_fmt, num_sms,
+      const cudaError_t e = try_pairs(dev, typename Epi::Widths(), ta, B, tc, p, epi, ab_fmt,
                                       stream, &launched);
       if (launched) return e;
     }
   }
-  auto kern = tc_gemm_kernel<BN, Epi, kRole>;
-  static thread_local bool attr_set = false;  // per instantiation
-  if (!attr_set) {
-    cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kBytes);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  const int grid = p.ntiles < num_sms ? p.ntiles : num_sms;
-  return launch_chained(kern, grid, gemm_threads<Epi>(), S::kBytes, stream, 1, ta, tb, tc, p, epi);
+  const cudaError_t ready = dev.of<SingleId<BN, Epi, kRole>>().status;
+  if (ready != cudaSuccess) return ready;
+  const int grid = p.ntiles < dev.num_sms ? p.ntiles : dev.num_sms;
+  return launch_chained(tc_gemm_kernel<BN, Epi, kRole>, grid, gemm_threads<Epi>(), S::kBytes, stream,
+                        1, ta, tb, tc, p, epi);
 }
 
 }  // namespace still

@@ -1120,17 +1120,14 @@ template <int HD>
 static cudaError_t launch_strip_d(const KVSource& src, int64_t N, int H, const PosSegs& segs,
                                   const double* omega, int rope_fix, int vec, int x16, int Kp,
                                   __nv_bfloat16* X, __half* XT, int64_t Np, float2* gd,
-                                  double origin, int G, int num_sms, cudaStream_t s) {
+                                  double origin, int G, const KernelTable& dev, cudaStream_t s) {
   constexpr int smem = kStripTok * (2 * HD + 2 + HD + 2) * 2;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(strip_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    attr = true;
-  }
+  const cudaError_t ready = dev.of<KernelId<strip_kernel<HD>, 256, smem>>().status;
+  if (ready != cudaSuccess) return ready;
   // Shares of the heads only while the token tiles leave SMs without two CTAs: each share forms
   // the tile's angles again, at the fp64 rate.
   const int64_t tiles = Np / kStripTok;
-  const int shares = (int)std::max<int64_t>(1, std::min<int64_t>(H, 2 * num_sms / tiles));
+  const int shares = (int)std::max<int64_t>(1, std::min<int64_t>(H, 2 * dev.num_sms / tiles));
   strip_kernel<HD><<<dim3((unsigned)tiles, shares), 256, smem, s>>>(
       src, N, H, segs, omega, rope_fix, vec, x16, Kp, X, XT, Np, gd, origin, G);
   return cudaGetLastError();
@@ -1139,7 +1136,7 @@ static cudaError_t launch_strip_d(const KVSource& src, int64_t N, int H, const P
 cudaError_t launch_strip(const KVSource& src, int64_t N, int H, int d, const PosSegs& segs,
                          const double* omega, int rope_fix, __nv_bfloat16* X, __half* XT,
                          int64_t Np, float2* gd, double origin, int G, int x16, int Kp,
-                         int num_sms, cudaStream_t s) {
+                         const KernelTable& dev, cudaStream_t s) {
   if (Np < kStripTok || Np % kStripTok != 0 || (Kp != 0 && (Kp % 64 != 0 || Kp < 2 * d + 1)))
     return cudaErrorInvalidValue;
   auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
@@ -1149,7 +1146,7 @@ cudaError_t launch_strip(const KVSource& src, int64_t N, int H, int d, const Pos
                                src.sH2 % 8 == 0));
   auto launch = [&](auto hd) {
     return launch_strip_d<decltype(hd)::value>(src, N, H, segs, omega, rope_fix, vec, x16, Kp, X,
-                                               XT, Np, gd, origin, G, num_sms, s);
+                                               XT, Np, gd, origin, G, dev, s);
   };
   switch (d) {
     case 64: return launch(std::integral_constant<int, 64>{});

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "epilogues.cuh"
+#include "kernel_table.cuh"
 
 namespace still {
 
@@ -32,7 +33,7 @@ struct KVSource {
 cudaError_t launch_strip(const KVSource& src, int64_t N, int H, int d, const PosSegs& segs,
                          const double* omega, int rope_fix, __nv_bfloat16* X, __half* XT,
                          int64_t Np, float2* gd, double origin, int G, int x16, int Kp,
-                         int num_sms, cudaStream_t s);
+                         const KernelTable& dev, cudaStream_t s);
 
 // Folded key projection (no compactor RoPE): Wt [n][Kp][D] bf16, rows of W~_i = [W_K,i; b_K,i]
 // padded with zero rows to Kp, columns in pair-chunk order (from WkT [nD][2d] and bk [nD]).

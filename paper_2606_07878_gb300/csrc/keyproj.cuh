@@ -551,8 +551,9 @@ __global__ void __launch_bounds__(kKeyThreads, 1)
 // X: [H * N][3d] (hi | key lo), W: [n D][2d] rows in key_row_source order, both ab_fmt (1 bf16, 0
 // fp16); d of 64, 128 or 256, D a multiple of 256.
 template <int NB, bool kFrac, bool kF16>
-inline cudaError_t launch_key_proj_as(const Operand2D& X, const Operand2D& W, KeyProjParams p,
-                                      int ab_fmt, int num_sms, cudaStream_t stream) {
+inline cudaError_t launch_key_proj_as(const KernelTable& dev, const Operand2D& X,
+                                      const Operand2D& W, KeyProjParams p, int ab_fmt,
+                                      cudaStream_t stream) {
   using S = KeyProjSmem<NB>;
   if (p.N <= 0 || p.D <= 0 || p.D % 256 != 0 || p.nh <= 0 || p.heads <= 0 || X.cols != 96 * NB ||
       W.cols != 64 * NB || p.ncoarse < 1)
@@ -560,12 +561,9 @@ inline cudaError_t launch_key_proj_as(const Operand2D& X, const Operand2D& W, Ke
   CUtensorMap ta, tb;
   if (!make_tmap(&ta, X, kBM) || !make_tmap(&tb, W, kBM)) return cudaErrorInvalidValue;
   p.idesc = idesc_f16(2 * kBM, 256, ab_fmt);
-  auto kern = key_proj_kernel<NB, kFrac, kF16>;
-  static thread_local int clusters = 0;  // per instantiation: resident clusters of two
-  if (clusters == 0) {
-    const cudaError_t e = resident_pairs(kern, kKeyThreads, S::kBytes, num_sms, &clusters);
-    if (e != cudaSuccess) return e;
-  }
+  using Id = KernelId<key_proj_kernel<NB, kFrac, kF16>, kKeyThreads, S::kBytes, 2>;
+  if (dev.of<Id>().status != cudaSuccess) return dev.of<Id>().status;
+  const int clusters = dev.persistent_clusters<Id>(2);
   const int mp = (p.N + 2 * kBM - 1) / (2 * kBM);
   const int64_t total = (int64_t)mp * (p.nh * (p.D / 256)) * p.heads;
   if (total > 0x7fffffff) return cudaErrorInvalidValue;
@@ -574,20 +572,21 @@ inline cudaError_t launch_key_proj_as(const Operand2D& X, const Operand2D& W, Ke
   // and a phase gives every pair several tiles
   const int64_t band_tiles = (int64_t)kBand * (p.nh * (p.D / 256));
   p.pbands = (int)std::max<int64_t>({1, kPhaseBytes / band_bytes, 4 * clusters / band_tiles});
-  return launch_chained(kern, 2 * (int)std::min<int64_t>(total, clusters), kKeyThreads, S::kBytes,
-                        stream, 2, ta, tb, p);
+  return launch_chained(key_proj_kernel<NB, kFrac, kF16>,
+                        2 * (int)std::min<int64_t>(total, clusters), kKeyThreads, S::kBytes, stream,
+                        2, ta, tb, p);
 }
 
-inline cudaError_t launch_key_proj(const Operand2D& X, const Operand2D& W, const KeyProjParams& p,
-                                   int d, bool frac, bool f16, int ab_fmt, int num_sms,
+inline cudaError_t launch_key_proj(const KernelTable& dev, const Operand2D& X, const Operand2D& W,
+                                   const KeyProjParams& p, int d, bool frac, bool f16, int ab_fmt,
                                    cudaStream_t s) {
   auto pick = [&](auto nb) -> cudaError_t {
     constexpr int NB = decltype(nb)::value;
     if (frac)
-      return f16 ? launch_key_proj_as<NB, true, true>(X, W, p, ab_fmt, num_sms, s)
-                 : launch_key_proj_as<NB, true, false>(X, W, p, ab_fmt, num_sms, s);
-    return f16 ? launch_key_proj_as<NB, false, true>(X, W, p, ab_fmt, num_sms, s)
-               : launch_key_proj_as<NB, false, false>(X, W, p, ab_fmt, num_sms, s);
+      return f16 ? launch_key_proj_as<NB, true, true>(dev, X, W, p, ab_fmt, s)
+                 : launch_key_proj_as<NB, true, false>(dev, X, W, p, ab_fmt, s);
+    return f16 ? launch_key_proj_as<NB, false, true>(dev, X, W, p, ab_fmt, s)
+               : launch_key_proj_as<NB, false, false>(dev, X, W, p, ab_fmt, s);
   };
   switch (d) {
     case 64: return pick(std::integral_constant<int, 2>{});

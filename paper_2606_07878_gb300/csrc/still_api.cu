@@ -167,7 +167,7 @@ struct Profiler {
 
 struct still_ctx {
   int device = 0;
-  int nsm = 0;
+  KernelTable kernels;  // of this device
   int* err = nullptr;  // device error record [4]
   std::vector<LayerW> layers;
   void* ws = nullptr;
@@ -256,7 +256,7 @@ still_status run_gemm_bn(still_ctx* ctx, const Operand2D& A, const Operand2D& B,
                          const StoreView3D* view = nullptr) {
   p.err = ctx->err;
   ctx->prof.begin(CLS, s);
-  cudaError_t r = launch_gemm<BN, CLS>(A, B, p, e, ab_fmt, ctx->nsm, s, view);
+  cudaError_t r = launch_gemm<BN, CLS>(ctx->kernels, A, B, p, e, ab_fmt, s, view);
   ctx->prof.end(CLS, s);
   if (r == cudaErrorInvalidValue) return STILL_ERR_INVALID_ARG;
   return r == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
@@ -627,8 +627,8 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
   void* Z3 = ws + P.oZ3;
 
   KLAUNCH(STILL_K_STRIP, launch_strip(src, N, H, d, pos.segs, L.omega_b, c.rope_fix, X, XT, Np,
-                                      gd, pos.origin, P.G, L.f16 ? 1 : 0, fold_kp(L), ctx->nsm,
-                                      s));
+                                      gd, pos.origin, P.G, L.f16 ? 1 : 0, fold_kp(L),
+                                      ctx->kernels, s));
   RopeTables tables;
   tables.coarse = coarse;
   tables.omega = omega;
@@ -783,9 +783,9 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
       kp.err = ctx->err;
       ctx->prof.begin(STILL_K_KEYPROJ, s);
       // k as fp16 hi | lo for a block feeding another and for one-pass scores
-      const cudaError_t r = launch_key_proj(op(X, (int64_t)H * N, 3 * d),
+      const cudaError_t r = launch_key_proj(ctx->kernels, op(X, (int64_t)H * N, 3 * d),
                                             op(Bw.WkT, (int64_t)n * D, 2 * d), kp, d, pos.frac,
-                                            exact || tk, w_fmt, ctx->nsm, s);
+                                            exact || tk, w_fmt, s);
       ctx->prof.end(STILL_K_KEYPROJ, s);
       if (r == cudaErrorInvalidValue) return STILL_ERR_INVALID_ARG;
       if (r != cudaSuccess) return STILL_ERR_CUDA;
@@ -801,7 +801,7 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
     if (!L.fold)
       KLAUNCH(STILL_K_QROPE, launch_q_rope(qsrc, qscale_rows, q_tmax, q_b0, nbl, t, D, qstart,
                                            qstep, L.omega_c, c.compactor_rope, qhl,
-                                           exact || tk ? 1 : 0, qscale, ctx->nsm, s));
+                                           exact || tk ? 1 : 0, qscale, ctx->kernels.num_sms, s));
     {
       // S, the online softmax and P X in one kernel; per-split partials merged in order.
       FlashParams fp;
@@ -816,7 +816,7 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
       const int fkeys = exact ? FlashSmem<256, true>::kKeys : kFlashKeys;
       fp.tiles_k = (int)((N + fkeys - 1) / fkeys);
       // a unit holds two query tiles: a CTA pair (2d <= 256) or a cluster of four (2d = 512)
-      const int slots = d == 256 ? ca_pair_clusters(ctx->nsm) : ctx->nsm / 2;
+      const int slots = d == 256 ? ca_pair_clusters(ctx->kernels) : ctx->kernels.num_sms / 2;
       const int mt = (fp.tiles_m + 1) / 2;
       fp.nsplit = flash_split((int64_t)mt * nbl, fp.tiles_k, slots, kMaxFlashSplit);
       const int64_t nunits = (int64_t)mt * nbl * fp.nsplit;
@@ -846,11 +846,11 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
       ctx->prof.begin(STILL_K_CA_FUSED, s);
       cudaError_t r =
           d == 256 ? (exact ? cudaErrorInvalidValue  // two-block layers at d = 256 are refused
-                            : launch_ca_pair(qop, kop, xop, fp, ctx->nsm, s, tk))
-          : exact  ? (d == 64 ? launch_ca_flash<128, true>(qop, kop, xop, fp, ctx->nsm, s)
-                              : launch_ca_flash<256, true>(qop, kop, xop, fp, ctx->nsm, s))
-                   : (d == 64 ? launch_ca_flash<128>(qop, kop, xop, fp, ctx->nsm, s)
-                              : launch_ca_flash<256>(qop, kop, xop, fp, ctx->nsm, s));
+                            : launch_ca_pair(ctx->kernels, qop, kop, xop, fp, s, tk))
+          : exact  ? (d == 64 ? launch_ca_flash<128, true>(ctx->kernels, qop, kop, xop, fp, s)
+                              : launch_ca_flash<256, true>(ctx->kernels, qop, kop, xop, fp, s))
+                   : (d == 64 ? launch_ca_flash<128>(ctx->kernels, qop, kop, xop, fp, s)
+                              : launch_ca_flash<256>(ctx->kernels, qop, kop, xop, fp, s));
       ctx->prof.end(STILL_K_CA_FUSED, s);
       if (r == cudaErrorInvalidValue) return STILL_ERR_INVALID_ARG;
       if (r != cudaSuccess) return STILL_ERR_CUDA;
@@ -1466,12 +1466,14 @@ still_status still_create(int device, still_ctx** out) {
   if (major != 10 || minor != 3) return STILL_ERR_UNSUPPORTED;  // built for sm_103a only
   still_ctx* c = new still_ctx();
   c->device = device;
-  if (cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
       cudaMalloc(&c->err, 4 * sizeof(int)) != cudaSuccess ||
       cudaMemset(c->err, 0, 4 * sizeof(int)) != cudaSuccess) {
     delete c;
     return STILL_ERR_CUDA;
   }
+  c->kernels.fill(sms);
   *out = c;
   return STILL_OK;
 }
@@ -1666,12 +1668,13 @@ still_status attend_biased_impl(still_ctx* ctx, int32_t n_layers, const void* co
     a.scale = scale > 0.f ? scale : 1.f / std::sqrt((float)d);
   }
   CK(cudaSetDevice(ctx->device));
-  TRY(ensure_ws(ctx, decode_workspace_bytes((int64_t)nq * Hq, decode_slots(t + S, H, ctx->nsm), d,
+  const int nsm = ctx->kernels.num_sms;
+  TRY(ensure_ws(ctx, decode_workspace_bytes((int64_t)nq * Hq, decode_slots(t + S, H, nsm), d,
                                             n_layers)));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   ctx->prof.begin(STILL_K_DECODE, s);
   int launches = 0;
-  cudaError_t r = launch_decode_biased(st, ctx->ws, ctx->nsm, s, &launches);
+  cudaError_t r = launch_decode_biased(st, ctx->ws, nsm, s, &launches);
   ctx->prof.end(STILL_K_DECODE, s);
   ctx->prof.launches[STILL_K_DECODE] += launches - 1;  // begin counted the first
   if (r != cudaSuccess) return STILL_ERR_CUDA;
@@ -2108,6 +2111,31 @@ size_t still_internal_reserve(const still_layer_config* cfg, int32_t lazy_q, int
                               int32_t t, size_t limit) {
   size_t bytes = 0;
   return plan_reserve(*cfg, lazy_q != 0, Kp, N, t, limit, &bytes) ? bytes : 0;
+}
+
+// Fills a context's kernel table with the caller's answers in place of the driver's; returns the
+// number of kernels. out: per kernel the status, then the resident clusters of 1 .. 8 CTAs.
+int still_internal_kernel_table(int32_t sms, int (*set_smem)(const void* fn, int bytes),
+                                int (*clusters)(int* n, const void* fn, int size), int32_t* out,
+                                int32_t room) {
+  static thread_local decltype(set_smem) set;
+  static thread_local decltype(clusters) ask;
+  set = set_smem;
+  ask = clusters;
+  KernelQuery q;
+  q.set_smem = [](const void* fn, int bytes) { return (cudaError_t)set(fn, bytes); };
+  q.clusters = [](int* n, const KernelEntry& e, int size, int) {
+    return (cudaError_t)ask(n, e.fn, size);
+  };
+  KernelTable t;
+  t.fill(sms, q);
+  const int n = (int)t.kernels.size();
+  for (int i = 0; i < std::min(n, room); ++i) {
+    out[i * (kMaxCluster + 1)] = (int32_t)t.kernels[i].status;
+    for (int c = 1; c <= kMaxCluster; ++c)
+      out[i * (kMaxCluster + 1) + c] = t.kernels[i].clusters[c];
+  }
+  return n;
 }
 
 }  // extern "C"
