@@ -115,6 +115,13 @@ template <int BN, class Epi>
 using SplitId = KernelId<tc_gemm_split_kernel<BN, Epi>, gemm_threads<Epi>(),
                          GemmSmem<BN, Epi>::kBytes, 2, kMaxSplit>;
 
+// Most tiles that the split kernel takes at tile width BN: half of the SMs hold a cluster of two
+// per tile, or fewer where the device's GPCs leave single SMs over.
+template <int BN, class Epi>
+inline int most_split_tiles(const KernelTable& dev) {
+  return std::min(dev.num_sms / 2, dev.of<SplitId<BN, Epi>>().clusters[2]);
+}
+
 // CTAs per tile of the split kernel at tile width BN for a GEMM of `ntiles` such tiles: the count
 // that is fastest by the clocks of its parts (measured on 128-row tiles at about 1.9 GHz: 384 /
 // 512 / 768 per K iteration at BN = 64 / 128 / 256, where a stage's bytes bound it; 16000 to read
@@ -123,7 +130,7 @@ using SplitId = KernelId<tc_gemm_split_kernel<BN, Epi>, gemm_threads<Epi>(),
 template <int BN, class Epi>
 inline int split_ranks(const KernelTable& dev, int64_t ntiles, int iters, double* cost) {
   *cost = 1e30;
-  if (ntiles > dev.num_sms / 2) return 1;
+  if (ntiles > most_split_tiles<BN, Epi>(dev)) return 1;
   const int* resident = dev.of<SplitId<BN, Epi>>().clusters;
   int best = 1;
   for (int s = 2; s <= std::min(kMaxSplit, iters); ++s) {

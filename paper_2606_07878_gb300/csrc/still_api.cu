@@ -342,10 +342,13 @@ size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 bool value_hilo(const still_layer_config&) { return true; }
 
 // Largest latent count whose q/k projection has so few tiles (of 128 rows x 256 columns, for all H
-// banks) that it can be split over CTAs. Up to it the projection writes one sum-of-squares partial
-// per 32 columns (256 rows at d_l = 256, 4 heads: 20.4 -> 12.4 us); above, one per 128 columns,
-// which is less to write and read.
-int64_t split_latents(int64_t H, int64_t n, int64_t D) { return 76 / (2 * n * D / 256) * 128 / H; }
+// banks) that it is split over CTAs: split_tiles, the most that the device splits. Up to it the
+// projection writes one sum-of-squares partial per 32 columns (256 rows at d_l = 256, 4 heads:
+// 20.4 -> 12.4 us); above, one per 128 columns, which is less to write and read, and which the
+// 2-SM kernel has.
+int64_t split_latents(int64_t split_tiles, int64_t H, int64_t n, int64_t D) {
+  return split_tiles / (2 * n * D / 256) * 128 / H;
+}
 
 // Sum-of-squares partials per self-attention q~ / k~ vector, and the bytes that T vectors' partials
 // and inverse norms take.
@@ -367,8 +370,8 @@ bool one_pass_scores(const still_layer_config& c) {
   return c.n_blocks == 1 && c.head_dim == 256 && c.d_latent >= 512 && c.d_latent <= 2048;
 }
 
-bool make_plan(const still_layer_config& c, bool lazy_q, int Kp, int64_t N, int t, double pmin,
-               double pmax, size_t limit, Plan& P) {
+bool make_plan(const still_layer_config& c, int split_tiles, bool lazy_q, int Kp, int64_t N, int t,
+               double pmin, double pmax, size_t limit, Plan& P) {
   P.H = c.n_kv_heads;
   P.d = c.head_dim;
   P.D = c.d_latent;
@@ -464,7 +467,7 @@ bool make_plan(const still_layer_config& c, bool lazy_q, int Kp, int64_t N, int 
   // The finer sums only where their bytes cost no group: a limit that holds the call with one
   // partial per 128 columns holds it with the same groups here.
   if (!plan_sa(narrow_parts(D))) return false;
-  if (T <= split_latents(H, n, D)) {
+  if (T <= split_latents(split_tiles, H, n, D)) {
     const int heads = P.sa_heads, sub = P.sa_sub;
     if (!plan_sa(wide_parts(D)) || P.sa_heads != heads || P.sa_sub != sub)
       plan_sa(narrow_parts(D));
@@ -477,15 +480,22 @@ bool make_plan(const still_layer_config& c, bool lazy_q, int Kp, int64_t N, int 
 
 // Workspace of every call of up to N tokens and up to t latents. A call's need grows with both but
 // for the finer sums of squares, which end at split_latents: the larger of the two sides.
-bool plan_reserve(const still_layer_config& c, bool lazy_q, int Kp, int64_t N, int t, size_t limit,
-                  size_t* bytes) {
+bool plan_reserve(const still_layer_config& c, int split_tiles, bool lazy_q, int Kp, int64_t N,
+                  int t, size_t limit, size_t* bytes) {
   Plan P;
-  if (!make_plan(c, lazy_q, Kp, N, t, 0.0, (double)(N - 1), limit, P)) return false;
+  const double last = (double)(N - 1);
+  if (!make_plan(c, split_tiles, lazy_q, Kp, N, t, 0.0, last, limit, P)) return false;
   *bytes = P.total;
-  const int64_t ts = split_latents(c.n_kv_heads, c.n_cross_heads, c.d_latent);
-  if (ts >= 1 && ts < t && make_plan(c, lazy_q, Kp, N, (int)ts, 0.0, (double)(N - 1), limit, P))
+  const int64_t ts = split_latents(split_tiles, c.n_kv_heads, c.n_cross_heads, c.d_latent);
+  if (ts >= 1 && ts < t &&
+      make_plan(c, split_tiles, lazy_q, Kp, N, (int)ts, 0.0, last, limit, P))
     *bytes = std::max(*bytes, P.total);
   return true;
+}
+
+// Tiles up to which the context's device splits the q/k projection.
+int split_tiles(const still_ctx* ctx) {
+  return most_split_tiles<256, EpiAffineT<true>>(ctx->kernels);
 }
 
 still_status ensure_ws(still_ctx* ctx, size_t bytes) {
@@ -601,7 +611,8 @@ still_status compact_one(still_ctx* ctx, const LayerW& L, const KVSource& src,
   const still_layer_config& c = L.cfg;
   Plan P;
   const size_t limit = ws_fixed != nullptr ? ws_fixed_bytes : ctx->ws_limit;
-  if (!make_plan(c, queries_per_call(L), fold_kp(L), N, t, pos.pmin, pos.pmax, limit, P))
+  if (!make_plan(c, split_tiles(ctx), queries_per_call(L), fold_kp(L), N, t, pos.pmin, pos.pmax,
+                 limit, P))
     return STILL_ERR_OOM;
   if (ws_fixed == nullptr) TRY(ensure_ws(ctx, P.total));
   uint8_t* ws = ws_fixed != nullptr ? ws_fixed : static_cast<uint8_t*>(ctx->ws);
@@ -2000,7 +2011,8 @@ still_status still_workspace_size(const still_ctx* ctx, int64_t max_tokens, int3
     return ctx == nullptr || bytes == nullptr ? STILL_ERR_INVALID_ARG : STILL_ERR_NOT_LOADED;
   if (max_tokens < 1 || max_t < 1 || max_t > max_tokens) return STILL_ERR_SHAPE;
   const LayerW& L = ctx->layers[0];
-  return plan_reserve(L.cfg, queries_per_call(L), fold_kp(L), max_tokens, max_t, ctx->ws_limit, bytes)
+  return plan_reserve(L.cfg, split_tiles(ctx), queries_per_call(L), fold_kp(L), max_tokens, max_t,
+                      ctx->ws_limit, bytes)
              ? STILL_OK
              : STILL_ERR_OOM;
 }
@@ -2094,10 +2106,11 @@ int64_t still_param_count(const still_layer_config* cfg, int32_t t) {
 
 // The plan of a call: bytes, (h, i) pairs per cross-attention group, KV-heads and self heads per
 // self-attention group, sum-of-squares partials per vector. 0 when the limit is too small.
-int still_internal_plan(const still_layer_config* cfg, int32_t lazy_q, int32_t Kp, int64_t N,
-                        int32_t t, double pmin, double pmax, size_t limit, int64_t out[5]) {
+int still_internal_plan(const still_layer_config* cfg, int32_t split_tiles, int32_t lazy_q,
+                        int32_t Kp, int64_t N, int32_t t, double pmin, double pmax, size_t limit,
+                        int64_t out[5]) {
   Plan P;
-  if (!make_plan(*cfg, lazy_q != 0, Kp, N, t, pmin, pmax, limit, P)) return 0;
+  if (!make_plan(*cfg, split_tiles, lazy_q != 0, Kp, N, t, pmin, pmax, limit, P)) return 0;
   out[0] = (int64_t)P.total;
   out[1] = P.ca_units;
   out[2] = P.sa_heads;
@@ -2107,10 +2120,10 @@ int still_internal_plan(const still_layer_config* cfg, int32_t lazy_q, int32_t K
 }
 
 // Bytes that still_reserve_workspace takes; 0 when the limit is too small.
-size_t still_internal_reserve(const still_layer_config* cfg, int32_t lazy_q, int32_t Kp, int64_t N,
-                              int32_t t, size_t limit) {
+size_t still_internal_reserve(const still_layer_config* cfg, int32_t split_tiles, int32_t lazy_q,
+                              int32_t Kp, int64_t N, int32_t t, size_t limit) {
   size_t bytes = 0;
-  return plan_reserve(*cfg, lazy_q != 0, Kp, N, t, limit, &bytes) ? bytes : 0;
+  return plan_reserve(*cfg, split_tiles, lazy_q != 0, Kp, N, t, limit, &bytes) ? bytes : 0;
 }
 
 // Fills a context's kernel table with the caller's answers in place of the driver's; returns the

@@ -21,13 +21,15 @@ def _cfg(H, d, D, n, F, t_max):
     return still.make_config(H, d, D, n, F, t_max, 1e6)
 
 
-def plan(lib, cfg, N, t, limit, pmin=0.0, pmax=None):
+SPLIT = 75  # tiles that the device splits
+
+
+def plan(lib, cfg, N, t, limit, split=SPLIT):
     """(bytes, pairs per cross-attention group, KV-heads and self heads per self-attention group,
     partials per vector), or None when the limit is too small."""
     out = OUT()
-    ok = lib.still_internal_plan(ctypes.byref(cfg), 0, 0, ctypes.c_int64(N), t,
-                                 ctypes.c_double(pmin),
-                                 ctypes.c_double(N - 1 if pmax is None else pmax),
+    ok = lib.still_internal_plan(ctypes.byref(cfg), split, 0, 0, ctypes.c_int64(N), t,
+                                 ctypes.c_double(0), ctypes.c_double(N - 1),
                                  ctypes.c_size_t(limit), out)
     return tuple(out) if ok else None
 
@@ -110,8 +112,21 @@ def test_reservation_serves_every_smaller_call(lib, H, d, D, n, F):
     for t_max in (1, 40, 650, 1300, 4000, 5500):
         N = max(6000, t_max)
         cfg = _cfg(H, d, D, n, F, t_max)
-        bytes_ = lib.still_internal_reserve(ctypes.byref(cfg), 0, 0, ctypes.c_int64(N), t_max,
+        bytes_ = lib.still_internal_reserve(ctypes.byref(cfg), SPLIT, 0, 0, ctypes.c_int64(N), t_max,
                                             ctypes.c_size_t(limit))
         assert bytes_ > 0
         for t in range(1, t_max + 1, max(1, t_max // 200)):
             assert plan(lib, cfg, N, t, limit)[0] <= bytes_, (t_max, t)
+
+
+def test_finer_sums_end_where_the_device_stops_splitting(lib):
+    """2 n d_l / 256 = 4 column tiles: the last latent count whose row tiles times 4 still split,
+    for whole and for cut-down devices."""
+    H, d, D, n = 2, 64, 256, 2
+    for split in (76, 75, 74, 33, 8, 4, 3, 0):
+        rows = split // 4 * 128
+        for t in {1, max(1, rows // H), rows // H + 1, 700}:
+            tiles = -(-H * t // 128) * 4
+            cfg = _cfg(H, d, D, n, 512, t)
+            parts = plan(lib, cfg, 3000, t, 48 << 30, split)[4]
+            assert parts == (D // 32 if tiles <= split else 2 * (D // 256)), (split, t, tiles)
