@@ -115,6 +115,22 @@ template <int BN, class Epi>
 using SplitId = KernelId<tc_gemm_split_kernel<BN, Epi>, gemm_threads<Epi>(),
                          GemmSmem<BN, Epi>::kBytes, 2, kMaxSplit>;
 
+// ------------------------------------------------------------------------------ which form
+//
+// A GEMM takes one of three kernels (tc_gemm.cuh): tiles of 128 x BN on single SMs, 256 x W on CTA
+// pairs, or tiles shared by a cluster that splits K. choose_gemm decides by the shape and the
+// device's table alone.
+enum GemmForm : int32_t { GEMM_SINGLE = 1, GEMM_PAIRS = 2, GEMM_SPLIT = 3 };
+struct GemmChoice {
+  int32_t form = GEMM_SINGLE;
+  int32_t width = 0;  // tile columns
+  int32_t ranks = 1;  // CTAs per tile (GEMM_SPLIT)
+};
+
+inline int64_t gemm_tiles(const GemmParams& p, int width) {
+  return (int64_t)p.tiles_m * ((p.N + width - 1) / width) * p.batch;
+}
+
 // Most tiles that the split kernel takes at tile width BN: half of the SMs hold a cluster of two
 // per tile, or fewer where the device's GPCs leave single SMs over.
 template <int BN, class Epi>
@@ -122,11 +138,12 @@ inline int most_split_tiles(const KernelTable& dev) {
   return std::min(dev.num_sms / 2, dev.of<SplitId<BN, Epi>>().clusters[2]);
 }
 
-// CTAs per tile of the split kernel at tile width BN for a GEMM of `ntiles` such tiles: the count
-// that is fastest by the clocks of its parts (measured on 128-row tiles at about 1.9 GHz: 384 /
-// 512 / 768 per K iteration at BN = 64 / 128 / 256, where a stage's bytes bound it; 16000 to read
-// all but one of the partials of 256 columns through DSMEM, 1400 to write one; 2500 per 32
-// columns in the epilogue; 4000 to start), with all clusters resident at once. *cost: its clocks.
+// CTAs per tile of the split kernel at tile width BN: the count, two or more, that is fastest by the
+// clocks of its parts (measured on 128-row tiles at about 1.9 GHz: 384 / 512 / 768 per K iteration
+// at BN = 64 / 128 / 256, where a stage's bytes bound it; 16000 to read all but one of the partials
+// of 256 columns through DSMEM, 1400 to write one; 2500 per 32 columns in the epilogue; 4000 to
+// start), with all clusters resident at once. 1: too many tiles, or a single K iteration. *cost:
+// its clocks, which order the counts and the two widths but not the forms (see choose_gemm).
 template <int BN, class Epi>
 inline int split_ranks(const KernelTable& dev, int64_t ntiles, int iters, double* cost) {
   *cost = 1e30;
@@ -146,15 +163,6 @@ inline int split_ranks(const KernelTable& dev, int64_t ntiles, int iters, double
   return best;
 }
 
-template <int BN, class Epi>
-inline cudaError_t launch_split(const CUtensorMap& ta, const CUtensorMap& tb,
-                                const CUtensorMap& tc, GemmParams p, const Epi& epi, int ranks,
-                                cudaStream_t stream) {
-  p.ksplit = ranks;
-  return launch_chained(tc_gemm_split_kernel<BN, Epi>, ranks * p.ntiles, gemm_threads<Epi>(),
-                        GemmSmem<BN, Epi>::kBytes, stream, ranks, ta, tb, tc, p, epi);
-}
-
 // Clocks of tc_gemm2_kernel per K iteration of a 256 x bn tile on two SMs, epilogue included:
 // measured 720 at 256 columns (t = 1024, d_l = 1024) and, with the key norms' epilogue, 0.90 of
 // that at 160; taken as that at 192 too, the width that 192 columns take.
@@ -167,6 +175,68 @@ inline int64_t gemm2_cost(const KernelTable& dev, const GemmParams& p) {
   const int clusters = dev.persistent_clusters<PairId<BN, Epi>>(2);
   const int64_t pairs = (int64_t)((p.tiles_m + 1) / 2) * ((p.N + BN - 1) / BN) * p.batch;
   return (pairs + clusters - 1) / clusters * gemm2_clocks(BN);
+}
+
+// The width of Epi::Widths at which the 2-SM kernel is fastest, if its waves are shorter than the
+// 1-SM kernel's (860 clocks per K iteration of a 128 x 256 tile), else 0.
+// An odd number of m-tiles or a bad last wave can make the pairs slower: t = 617, d_l = 2048, P v
+// 488 us on single SMs, 584 on pairs. The key norms of the folded path have 320 columns, two tiles
+// of 160 or two of 256 with 192 columns of padding (170 -> 152 us at 8,192 tokens of 4 heads), or
+// 192. For the latent GEMMs widths of 192 and 224 gave the call 0.4% at t = 617 (better last
+// waves) and nothing elsewhere, and are not offered.
+template <class Epi, int... W>
+inline int pair_width(const KernelTable& dev, std::integer_sequence<int, W...>,
+                      const GemmParams& p) {
+  int width = 0;
+  int64_t best = ((int64_t)p.ntiles + dev.num_sms - 1) / dev.num_sms * 860;
+  auto consider = [&](int64_t cost, int bn) {
+    if (cost < best) {
+      best = cost;
+      width = bn;
+    }
+  };
+  (consider(gemm2_cost<W, Epi>(dev, p), W), ...);
+  return width;
+}
+
+// p: finalized at BN. Few tiles split first: up to most_split_tiles the other two forms leave half
+// of the SMs idle. Measured in calls replayed from a graph, forms forced one GEMM at a time, against
+// the split count that is taken. One SM per 128 x 256 tile: the GEMMs of a layer of t = 128,
+// d_l = 256, H = 2 cost the call 2 to 18 us more (of 123), also where the clocks above say about
+// even (8 K iterations: 2 to 8 us); those of t = 251, d_l = 1024, H = 4 up to 65 us (of 954). Pairs:
+// within 2 us of that at t = 128, up to 9 us less at t = 251. One CTA per 128 x 64 tile is within 2 us
+// of the split at t = 128; at t = 300, H = 2 it gains 4 us (of 180) in each of two GEMMs whose
+// 64-column tiles outnumber most_split_tiles but not the SMs, and is not offered.
+template <int BN, class Epi>
+inline GemmChoice choose_gemm(const KernelTable& dev, const GemmParams& p, bool can_split) {
+  if (can_split) {
+    double cost = 0, cost64 = 1e30;
+    const int ranks = split_ranks<BN, Epi>(dev, p.ntiles, p.iters_total, &cost);
+    if constexpr (Epi::kAnyTile && BN != 64) {  // narrower tiles: less to reduce per CTA
+      const int ranks64 = split_ranks<64, Epi>(dev, gemm_tiles(p, 64), p.iters_total, &cost64);
+      if (ranks64 > 1 && cost64 < cost) return {GEMM_SPLIT, 64, ranks64};
+    }
+    if (ranks > 1) return {GEMM_SPLIT, BN, ranks};
+  }
+  if constexpr (BN == 256 && Epi::kPairs) {
+    const int width = pair_width<Epi>(dev, typename Epi::Widths(), p);
+    if (width != 0) return {GEMM_PAIRS, width, 1};
+  }
+  return {GEMM_SINGLE, BN, 1};
+}
+
+// ------------------------------------------------------------------------------ launches
+
+template <int BN, class Epi>
+inline cudaError_t launch_split(const CUtensorMap& ta, const Operand2D& B, const CUtensorMap& tc,
+                                GemmParams p, Epi epi, int ab_fmt, int ranks,
+                                cudaStream_t stream) {
+  CUtensorMap tb;
+  if (!finalize_gemm<BN>(p, ab_fmt) || !make_tmap(&tb, B, BN)) return cudaErrorInvalidValue;
+  epi.tile_cols_ = BN;
+  p.ksplit = ranks;
+  return launch_chained(tc_gemm_split_kernel<BN, Epi>, ranks * p.ntiles, gemm_threads<Epi>(),
+                        GemmSmem<BN, Epi>::kBytes, stream, ranks, ta, tb, tc, p, epi);
 }
 
 template <int BN, class Epi>
@@ -182,75 +252,46 @@ inline cudaError_t launch_pairs(const KernelTable& dev, const CUtensorMap& ta, c
   return launch_chained(tc_gemm2_kernel<BN, Epi>, 2 * clusters, gemm_threads<Epi>(),
                         Gemm2Smem<BN, Epi>::kBytes, stream, 2, ta, tb, tc, p, epi);
 }
-
-// Launches the 2-SM kernel at the width of Epi::Widths that is fastest, if its waves are shorter
-// than the 1-SM kernel's (860 clocks per K iteration of a 128 x 256 tile). *launched says whether.
-// An odd number of m-tiles or a bad last wave can make the pairs slower: t = 617, d_l = 2048, P v
-// 488 us on single SMs, 584 on pairs. The key norms of the folded path have 320 columns, two tiles
-// of 160 or two of 256 with 192 columns of padding (170 -> 152 us at 8,192 tokens of 4 heads), or
-// 192. For the latent GEMMs widths of 192 and 224 gave the call 0.4% at t = 617 (better last
-// waves) and nothing elsewhere, and are not offered.
 template <class Epi, int... W>
-inline cudaError_t try_pairs(const KernelTable& dev, std::integer_sequence<int, W...>,
-                             const CUtensorMap& ta, const Operand2D& B, const CUtensorMap& tc,
-                             const GemmParams& p, const Epi& epi, int ab_fmt,
-                             cudaStream_t stream, bool* launched) {
-  int width = 0;
-  int64_t best = ((int64_t)p.ntiles + dev.num_sms - 1) / dev.num_sms * 860;
-  auto consider = [&](int64_t cost, int bn) {
-    if (cost < best) {
-      best = cost;
-      width = bn;
-    }
-  };
-  (consider(gemm2_cost<W, Epi>(dev, p), W), ...);
-  *launched = width != 0;
-  cudaError_t e = cudaSuccess;
+inline cudaError_t launch_pairs_at(const KernelTable& dev, int width,
+                                   std::integer_sequence<int, W...>, const CUtensorMap& ta,
+                                   const Operand2D& B, const CUtensorMap& tc, const GemmParams& p,
+                                   const Epi& epi, int ab_fmt, cudaStream_t stream) {
+  cudaError_t e = cudaErrorInvalidValue;
   ((width == W ? (void)(e = launch_pairs<W, Epi>(dev, ta, B, tc, p, epi, ab_fmt, stream))
                : (void)0),
    ...);
   return e;
 }
 
+// taken: the form that is launched.
 template <int BN, int kRole, class Epi>
 inline cudaError_t launch_gemm(const KernelTable& dev, const Operand2D& A, const Operand2D& B,
                                GemmParams p, Epi epi, int ab_fmt, cudaStream_t stream,
-                               const StoreView3D* out_view = nullptr) {
-  using S = GemmSmem<BN, Epi>;
+                               const StoreView3D* out_view, GemmChoice* taken) {
   if (!finalize_gemm<BN>(p, ab_fmt)) return cudaErrorInvalidValue;
   CUtensorMap ta, tb, tc;
-  if (!make_tmap(&ta, A, kBM) || !make_tmap(&tb, B, BN)) return cudaErrorInvalidValue;
+  if (!make_tmap(&ta, A, kBM)) return cudaErrorInvalidValue;
   std::memset(&tc, 0, sizeof(tc));
   if (out_view != nullptr && !make_store_tmap(&tc, *out_view)) return cudaErrorInvalidValue;
+  const GemmChoice c = choose_gemm<BN, Epi>(dev, p, epi.can_split());
+  *taken = c;
+  if (c.form == GEMM_SPLIT) {
+    if constexpr (Epi::kAnyTile && BN != 64)
+      if (c.width == 64) return launch_split<64, Epi>(ta, B, tc, p, epi, ab_fmt, c.ranks, stream);
+    return launch_split<BN, Epi>(ta, B, tc, p, epi, ab_fmt, c.ranks, stream);
+  }
+  if constexpr (BN == 256 && Epi::kPairs)
+    if (c.form == GEMM_PAIRS)
+      return launch_pairs_at<Epi>(dev, c.width, typename Epi::Widths(), ta, B, tc, p, epi, ab_fmt,
+                                  stream);
+  if (!make_tmap(&tb, B, BN)) return cudaErrorInvalidValue;
   epi.tile_cols_ = BN;
-  if (epi.can_split() && p.ksplit == 1) {
-    double cost = 0, cost64 = 1e30;
-    const int ranks = split_ranks<BN, Epi>(dev, p.ntiles, p.iters_total, &cost);
-    if constexpr (Epi::kAnyTile && BN != 64) {  // narrower tiles: less to reduce per CTA
-      GemmParams q = p;
-      if (!finalize_gemm<64>(q, ab_fmt)) return cudaErrorInvalidValue;
-      const int ranks64 = split_ranks<64, Epi>(dev, q.ntiles, q.iters_total, &cost64);
-      if (ranks64 > 1 && cost64 < cost) {
-        if (!make_tmap(&tb, B, 64)) return cudaErrorInvalidValue;
-        epi.tile_cols_ = 64;
-        return launch_split<64, Epi>(ta, tb, tc, q, epi, ranks64, stream);
-      }
-    }
-    if (ranks > 1) return launch_split<BN, Epi>(ta, tb, tc, p, epi, ranks, stream);
-  }
-  if constexpr (BN == 256 && Epi::kPairs) {
-    if (p.ksplit == 1) {
-      bool launched = false;
-      const cudaError_t e = try_pairs(dev, typename Epi::Widths(), ta, B, tc, p, epi, ab_fmt,
-                                      stream, &launched);
-      if (launched) return e;
-    }
-  }
   const cudaError_t ready = dev.of<SingleId<BN, Epi, kRole>>().status;
   if (ready != cudaSuccess) return ready;
   const int grid = p.ntiles < dev.num_sms ? p.ntiles : dev.num_sms;
-  return launch_chained(tc_gemm_kernel<BN, Epi, kRole>, grid, gemm_threads<Epi>(), S::kBytes, stream,
-                        1, ta, tb, tc, p, epi);
+  return launch_chained(tc_gemm_kernel<BN, Epi, kRole>, grid, gemm_threads<Epi>(),
+                        GemmSmem<BN, Epi>::kBytes, stream, 1, ta, tb, tc, p, epi);
 }
 
 }  // namespace still

@@ -176,6 +176,7 @@ struct still_ctx {
   size_t qhat_eager_limit = size_t(2) << 30;
   bool key_fold = true;  // fold W_K into the queries where the layer allows it
   Profiler prof;
+  GemmChoice gemms[STILL_K_COUNT];  // the form last launched per kernel class
 };
 
 namespace {
@@ -256,7 +257,8 @@ still_status run_gemm_bn(still_ctx* ctx, const Operand2D& A, const Operand2D& B,
                          const StoreView3D* view = nullptr) {
   p.err = ctx->err;
   ctx->prof.begin(CLS, s);
-  cudaError_t r = launch_gemm<BN, CLS>(ctx->kernels, A, B, p, e, ab_fmt, s, view);
+  cudaError_t r =
+      launch_gemm<BN, CLS>(ctx->kernels, A, B, p, e, ab_fmt, s, view, &ctx->gemms[CLS]);
   ctx->prof.end(CLS, s);
   if (r == cudaErrorInvalidValue) return STILL_ERR_INVALID_ARG;
   return r == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
@@ -2149,6 +2151,58 @@ int still_internal_kernel_table(int32_t sms, int (*set_smem)(const void* fn, int
       out[i * (kMaxCluster + 1) + c] = t.kernels[i].clusters[c];
   }
   return n;
+}
+
+// The form (1 one SM, 2 CTA pairs, 3 split along K), tile width and CTAs per tile that a GEMM of
+// M x N over `iters` K iterations of 64 takes on a device of `sms` SMs that holds resident[c]
+// clusters of c CTAs. kind: 0 the general epilogue, 1 with sums of squares per 32 columns, 2 with
+// one per tile half, 3 the folded key norms, 4 the output heads (tiles of 256), 5 (of 128).
+int still_internal_gemm_form(int32_t kind, int32_t M, int32_t N, int32_t batch, int32_t iters,
+                             int32_t sms, const int32_t resident[kMaxCluster + 1],
+                             int32_t out[3]) {
+  static thread_local const int32_t* answers;
+  answers = resident;
+  KernelQuery q;
+  q.set_smem = [](const void*, int) { return cudaSuccess; };
+  q.clusters = [](int* n, const KernelEntry&, int size, int) {
+    *n = answers[size];
+    return cudaSuccess;
+  };
+  KernelTable dev;
+  dev.fill(sms, q);
+  GemmParams p = gp(M, N, batch);
+  add_pass(p, 0, 0, 0, 0, iters * kBK);
+  float sums = 0;
+  EpiAffine plain, halves;
+  EpiAffineT<true> chunks;
+  halves.sumsq = chunks.sumsq = &sums;
+  if (!finalize_gemm<256>(p, 1)) return 0;
+  GemmChoice c;
+  switch (kind) {
+    case 0: c = choose_gemm<256, EpiAffine>(dev, p, plain.can_split()); break;
+    case 1: c = choose_gemm<256, EpiAffineT<true>>(dev, p, chunks.can_split()); break;
+    case 2: c = choose_gemm<256, EpiAffine>(dev, p, halves.can_split()); break;
+    case 3: c = choose_gemm<256, EpiQuad>(dev, p, EpiQuad().can_split()); break;
+    case 4: c = choose_gemm<256, EpiHeads>(dev, p, EpiHeads().can_split()); break;
+    case 5:
+      if (!finalize_gemm<128>(p, 1)) return 0;
+      c = choose_gemm<128, EpiHeads>(dev, p, EpiHeads().can_split());
+      break;
+    default: return 0;
+  }
+  out[0] = c.form;
+  out[1] = c.width;
+  out[2] = c.ranks;
+  return 1;
+}
+
+// The same of the last GEMM that the context launched in a kernel class (form 1, width 0: none).
+int still_internal_last_gemm(const still_ctx* ctx, int32_t cls, int32_t out[3]) {
+  if (ctx == nullptr || cls < 0 || cls >= STILL_K_COUNT) return 0;
+  out[0] = ctx->gemms[cls].form;
+  out[1] = ctx->gemms[cls].width;
+  out[2] = ctx->gemms[cls].ranks;
+  return 1;
 }
 
 }  // extern "C"

@@ -1,4 +1,5 @@
 """Shared helpers for the GPU parity tests: run the library, compare with the oracle."""
+import ctypes
 import json
 import os
 
@@ -63,8 +64,18 @@ class Runner:
         code, det = still.still_get_device_status(self.ctx)
         assert code == 0, f"device status {still.STATUS.get(code)} {det}"
 
+    def gemm(self, cls):
+        """(form, tile width, CTAs per tile) of the last GEMM launched in a kernel class."""
+        out = (ctypes.c_int32 * 3)()
+        assert still.lib().still_internal_last_gemm(self.ctx, still.KERNEL_CLASSES.index(cls), out)
+        return tuple(out)
+
     def close(self):
         still.still_destroy(self.ctx)
+
+
+# GEMM forms of Runner.gemm
+SINGLE, PAIRS, SPLIT = 1, 2, 3
 
 
 def oracle_layer(wl, W, K, V, t, kpos=None, heads=None, cfg_over=None):

@@ -3,7 +3,7 @@
 tile, and several waves."""
 import pytest
 
-from gpu_helpers import Runner, assert_parity, oracle_layer
+from gpu_helpers import PAIRS, Runner, assert_parity, oracle_layer
 from paper_2606_07878_gb300 import synth
 
 pytestmark = pytest.mark.gpu
@@ -11,17 +11,20 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-@pytest.mark.parametrize("H,d,D,n,F,t", [
-    (2, 64, 512, 4, 4096, 641),     # 11 row tiles (odd), FFN of 16 column tiles
-    (1, 128, 256, 16, 2880, 700),   # FFN width that ends inside a tile
-    (4, 64, 256, 8, 3072, 520),     # scores and P v over 32 batches
+@pytest.mark.parametrize("H,d,D,n,F,t,pairs", [
+    (2, 64, 512, 4, 4096, 641, ["ffn1"]),       # 11 row tiles (odd), FFN of 16 column tiles
+    (1, 128, 256, 16, 2880, 700, ["sa_proj"]),  # rows that end inside a tile, 32 column tiles
+    (4, 64, 256, 8, 3072, 520, ["sa_scores", "sa_pv", "ffn1"]),  # 32 batches
+    (2, 64, 256, 4, 2880, 1300, ["ffn1"]),      # FFN width that ends inside a tile
 ])
-def test_wide_latent_sublayers_match_oracle(H, d, D, n, F, t):
-    wl = synth.tiny_workload(H=H, d=d, D=D, n=n, F=F, N=768, heavy=2, ts=(t,))
+def test_wide_latent_sublayers_match_oracle(H, d, D, n, F, t, pairs):
+    wl = synth.tiny_workload(H=H, d=d, D=D, n=n, F=F, N=max(768, t), heavy=2, ts=(t,))
     r = Runner(wl, t)
     try:
         K, V = synth.gen_kv(wl, 0, device=DEV)
         Ck, Cv, _ = r.layer(0, K, V, t)
+        for cls in pairs:
+            assert r.gemm(cls) == (PAIRS, 256, 1), cls
         rk, rv, _, _ = oracle_layer(wl, r.W[0], K, V, t)
         for name, ref, got in (("C_k", rk, Ck), ("C_v", rv, Cv)):
             assert_parity(ref, synth.bf16_to_f64(got), name)
@@ -38,6 +41,7 @@ def test_folded_key_norms_match_oracle(d, D):
     try:
         K, V = synth.gen_kv(wl, 0, device=DEV)
         Ck, Cv, _ = r.layer(0, K, V, t)
+        assert r.gemm("keyproj")[0] == PAIRS
         rk, rv, _, _ = oracle_layer(wl, r.W[0], K, V, t, cfg_over=dict(compactor_rope=False))
         for name, ref, got in (("C_k", rk, Ck), ("C_v", rv, Cv)):
             assert_parity(ref, synth.bf16_to_f64(got), name)

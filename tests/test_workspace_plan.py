@@ -21,7 +21,7 @@ def _cfg(H, d, D, n, F, t_max):
     return still.make_config(H, d, D, n, F, t_max, 1e6)
 
 
-SPLIT = 75  # tiles that the device splits
+SPLIT = 76  # tiles that the device splits
 
 
 def plan(lib, cfg, N, t, limit, split=SPLIT):
