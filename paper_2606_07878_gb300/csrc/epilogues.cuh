@@ -163,6 +163,9 @@ struct EpiAffineT {
   static constexpr bool kAnyTile = true;  // its 32-column chunks are independent
   static constexpr bool kPairs = !kChunkSums;  // has a 2-SM form, of these tile widths:
   using Widths = std::integer_sequence<int, 256>;
+  // Clocks of the 2-SM form (see gemm2_cost): 720 measured at t = 1024, d_l = 1024.
+  static constexpr int pair_wave(int) { return 720; }
+  static constexpr int pair_start(int) { return 0; }
 
   // The residual rows of this warp's columns are pulled into L2 while the main loop runs.
   template <class Src>
@@ -446,7 +449,14 @@ struct EpiQuad {
   bool can_split() const { return true; }
   static constexpr bool kAnyTile = true;
   static constexpr bool kPairs = true;
-  using Widths = std::integer_sequence<int, 192, 160>;  // Kp is 192 or 320
+  // Kp is 320, two tiles of 160, or 192. Measured on both kernels (us, 1-SM then pairs; 4 KV-heads of
+  // 8 cross heads): Kp 320, 896 tokens 33.1, 32.6; 1,152 38.9, 37.8; 2,688 69.5, 63.5; 8,192 176.7,
+  // 151.8 (158.3 in two tiles of 192). Kp 192, 1,024 tokens 21.0, 22.5; 2,048 31.4, 31.4; 2,432
+  // 32.6, 35.9 (4 waves against 5); 4,864 52.8, 51.1; 8,192 81.3, 78.5. A line through each column
+  // over its waves gives the clocks.
+  using Widths = std::integer_sequence<int, 160, 192>;
+  static constexpr int pair_wave(int bn) { return bn == 160 ? 745 : 800; }
+  static constexpr int pair_start(int bn) { return bn == 160 ? -480 : 240; }
 
   template <class Src>
   __device__ void prefetch(const GemmParams&, const TileCoord&, int, const Src&, int) const {}

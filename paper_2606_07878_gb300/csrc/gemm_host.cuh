@@ -163,27 +163,21 @@ inline int split_ranks(const KernelTable& dev, int64_t ntiles, int iters, double
   return best;
 }
 
-// Clocks of tc_gemm2_kernel per K iteration of a 256 x bn tile on two SMs, epilogue included:
-// measured 720 at 256 columns (t = 1024, d_l = 1024) and, with the key norms' epilogue, 0.90 of
-// that at 160; taken as that at 192 too, the width that 192 columns take.
-inline int gemm2_clocks(int bn) { return bn < 256 ? 650 : 720; }
-
-// Time of a GEMM on pairs in clocks per K iteration: waves of its tiles.
+// Time of a GEMM on pairs, in clocks per K iteration beside 860 for a wave of the 1-SM kernel's
+// 128 x 256 tiles: waves of its tiles, and what its start adds or saves.
 template <int BN, class Epi>
 inline int64_t gemm2_cost(const KernelTable& dev, const GemmParams& p) {
   if (dev.of<PairId<BN, Epi>>().status != cudaSuccess) return INT64_MAX;
   const int clusters = dev.persistent_clusters<PairId<BN, Epi>>(2);
   const int64_t pairs = (int64_t)((p.tiles_m + 1) / 2) * ((p.N + BN - 1) / BN) * p.batch;
-  return (pairs + clusters - 1) / clusters * gemm2_clocks(BN);
+  return (pairs + clusters - 1) / clusters * Epi::pair_wave(BN) + Epi::pair_start(BN);
 }
 
-// The width of Epi::Widths at which the 2-SM kernel is fastest, if its waves are shorter than the
-// 1-SM kernel's (860 clocks per K iteration of a 128 x 256 tile), else 0.
+// The width of Epi::Widths at which the 2-SM kernel is fastest, if that is faster than the 1-SM
+// kernel, else 0.
 // An odd number of m-tiles or a bad last wave can make the pairs slower: t = 617, d_l = 2048, P v
-// 488 us on single SMs, 584 on pairs. The key norms of the folded path have 320 columns, two tiles
-// of 160 or two of 256 with 192 columns of padding (170 -> 152 us at 8,192 tokens of 4 heads), or
-// 192. For the latent GEMMs widths of 192 and 224 gave the call 0.4% at t = 617 (better last
-// waves) and nothing elsewhere, and are not offered.
+// 488 us on single SMs, 584 on pairs. For the latent GEMMs widths of 192 and 224 gave the call 0.4%
+// at t = 617 (better last waves) and nothing elsewhere, and are not offered.
 template <class Epi, int... W>
 inline int pair_width(const KernelTable& dev, std::integer_sequence<int, W...>,
                       const GemmParams& p) {

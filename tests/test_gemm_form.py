@@ -85,3 +85,21 @@ def test_pairs_where_their_waves_are_shorter():
     # sums of squares per tile half do not split
     assert form(HALF_SUMS, 600, 256, 8, 8)[0] == PAIRS
     assert form(HEADS, 4096, 512, 4, 64)[0] == SINGLE  # no 2-SM form
+
+
+def test_key_norms_take_the_faster_form():
+    """The folded key norms of 4 KV-heads of 8 cross heads: the faster of the two measured forms at
+    every measured token count (equal at 2,048 tokens of K_p = 192)."""
+    for tokens in (896, 1024, 1152, 1280, 2688, 8192):
+        assert form(NORMS, tokens, 320, 32, 15) == (PAIRS, 160, 1), tokens
+    for tokens, want in [(1024, SINGLE), (2048, SINGLE), (2432, SINGLE), (4864, PAIRS), (8192, PAIRS)]:
+        got = form(NORMS, tokens, 192, 32, 9)
+        assert got == ((PAIRS, 192, 1) if want == PAIRS else (SINGLE, 256, 1)), (tokens, got)
+
+
+@pytest.mark.parametrize("N,width", [(320, 160), (192, 192)])
+def test_key_norm_tiles_hold_no_padding(N, width):
+    for tokens in range(64, 20000, 97):
+        for batch in (1, 4, 16, 64):
+            f, w, _ = form(NORMS, tokens, N, batch, 3 * N // 64)
+            assert f != PAIRS or w == width, (tokens, batch)

@@ -1,9 +1,9 @@
-"""Latent sublayers and folded key norms wide enough for the GEMM on CTA pairs (tiles of 256 x 160 to
-256 columns) against the oracle: an odd number of row tiles, rows and columns that end inside a
+"""Latent sublayers and folded key norms wide enough for the GEMM on CTA pairs (tiles of 256 x 160,
+192 or 256) against the oracle: an odd number of row tiles, rows and columns that end inside a
 tile, and several waves."""
 import pytest
 
-from gpu_helpers import PAIRS, Runner, assert_parity, oracle_layer
+from gpu_helpers import PAIRS, SINGLE, Runner, assert_parity, oracle_layer
 from paper_2606_07878_gb300 import synth
 
 pytestmark = pytest.mark.gpu
@@ -32,16 +32,20 @@ def test_wide_latent_sublayers_match_oracle(H, d, D, n, F, t, pairs):
         r.close()
 
 
-@pytest.mark.parametrize("d,D", [(128, 512), (64, 256)])  # 320 and 192 columns of key norms
-def test_folded_key_norms_match_oracle(d, D):
+@pytest.mark.parametrize("d,D,N,want", [
+    (128, 512, 3001, (PAIRS, 160, 1)),   # 320 columns of key norms
+    (64, 256, 3001, (SINGLE, 256, 1)),   # 192 columns, three waves
+    (64, 256, 5501, (PAIRS, 192, 1)),    # five, an odd number of row tiles
+])
+def test_folded_key_norms_match_oracle(d, D, N, want):
     t = 48
-    wl = synth.tiny_workload(H=4, d=d, D=D, n=4, F=0, N=3001, heavy=2, ts=(t,))
+    wl = synth.tiny_workload(H=4, d=d, D=D, n=4, F=0, N=N, heavy=2, ts=(t,))
     over = dict(compactor_rope=0)
     r = Runner(wl, t, cfg_over=over)
     try:
         K, V = synth.gen_kv(wl, 0, device=DEV)
         Ck, Cv, _ = r.layer(0, K, V, t)
-        assert r.gemm("keyproj")[0] == PAIRS
+        assert r.gemm("keyproj") == want
         rk, rv, _, _ = oracle_layer(wl, r.W[0], K, V, t, cfg_over=dict(compactor_rope=False))
         for name, ref, got in (("C_k", rk, Ck), ("C_v", rv, Cv)):
             assert_parity(ref, synth.bf16_to_f64(got), name)
