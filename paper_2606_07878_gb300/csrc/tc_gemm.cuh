@@ -238,6 +238,18 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
           }
         }
       }
+      // every slot released by its MMAs (an issuer that gave up releases none) before the CTA may
+      // leave
+      for (int i = 0; i < kStages && !*abort_flag; ++i) {
+        if (!mbar_wait(&empty[stage], phase ^ 1)) {
+          dev_set_error(p.err, DEV_WAIT_TIMEOUT, 109);
+          *abort_flag = 1;
+        }
+        if (++stage == kStages) {
+          stage = 0;
+          phase ^= 1;
+        }
+      }
       if (*abort_flag) {
         // Let every copy this thread issued land before the CTA can exit.
         for (int s = 0; s < kStages; ++s)
@@ -738,6 +750,17 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
         tma_load_2d(sa + S::kABytes, &tmB, &full[stage], (int32_t)(bk + ps.b_koff + kk),
                     (int32_t)(br + ps.b_roff));
         ++sent;
+        if (++stage == kStages) {
+          stage = 0;
+          phase ^= 1;
+        }
+      }
+      // every slot released by its MMAs, as in tc_gemm_kernel
+      for (int i = 0; i < kStages && !*abort_flag; ++i) {
+        if (!mbar_wait(&empty[stage], phase ^ 1)) {
+          dev_set_error(p.err, DEV_WAIT_TIMEOUT, 113);
+          *abort_flag = 1;
+        }
         if (++stage == kStages) {
           stage = 0;
           phase ^= 1;
