@@ -89,7 +89,8 @@ STILL_DEV float max3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
 }
-// 2^x with results below 2^-126 flushed to 0 (exp2f's instruction without its scaling of those)
+// ex2.approx.ftz.f32: 2^x, subnormal inputs and results flushed to zero. For values that are rounded
+// to fp16, whose smallest positive one is 2^-24, next.
 STILL_DEV float ex2_ftz(float x) {
   float r;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
