@@ -238,18 +238,6 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
           }
         }
       }
-      // every slot released by its MMAs (an issuer that gave up releases none) before the CTA may
-      // leave
-      for (int i = 0; i < kStages && !*abort_flag; ++i) {
-        if (!mbar_wait(&empty[stage], phase ^ 1)) {
-          dev_set_error(p.err, DEV_WAIT_TIMEOUT, 109);
-          *abort_flag = 1;
-        }
-        if (++stage == kStages) {
-          stage = 0;
-          phase ^= 1;
-        }
-      }
       if (*abort_flag) {
         // Let every copy this thread issued land before the CTA can exit.
         for (int s = 0; s < kStages; ++s)
@@ -302,9 +290,21 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
           acc_phase ^= 1;
         }
       }
-      if (*abort_flag && issued) {
-        tc_commit(drain);
-        (void)mbar_wait(drain, 0);
+      if (*abort_flag) {
+        if (issued) {
+          tc_commit(drain);
+          (void)mbar_wait(drain, 0);
+        }
+        // The producer may have left with copies in flight into slots that no MMA releases any
+        // more: at most one round of the ring, which lands before the CTA exits (a wait for a
+        // copy that was not issued runs out).
+        for (int s = 0; s < kStages; ++s) {
+          (void)mbar_wait(&full[stage], phase);
+          if (++stage == kStages) {
+            stage = 0;
+            phase ^= 1;
+          }
+        }
       }
     }
   } else {
@@ -755,17 +755,6 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
           phase ^= 1;
         }
       }
-      // every slot released by its MMAs, as in tc_gemm_kernel
-      for (int i = 0; i < kStages && !*abort_flag; ++i) {
-        if (!mbar_wait(&empty[stage], phase ^ 1)) {
-          dev_set_error(p.err, DEV_WAIT_TIMEOUT, 113);
-          *abort_flag = 1;
-        }
-        if (++stage == kStages) {
-          stage = 0;
-          phase ^= 1;
-        }
-      }
       if (*abort_flag)  // let every copy this thread issued land before the CTA can exit
         for (int s = 0; s < min(sent, kStages); ++s) {
           const int i = sent - 1 - s;  // the i-th copy used stage i % kStages in round i / kStages
@@ -781,6 +770,14 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
         if (!mbar_wait(&full[stage], phase)) {
           dev_set_error(p.err, DEV_WAIT_TIMEOUT, 111);
           *abort_flag = 1;
+          // the copies that the producer may have left in flight (see tc_gemm_kernel)
+          for (int i = it; i < min(it + kStages, it1); ++i) {
+            (void)mbar_wait(&full[stage], phase);
+            if (++stage == kStages) {
+              stage = 0;
+              phase ^= 1;
+            }
+          }
           break;
         }
         tc_fence_after();
