@@ -69,17 +69,17 @@ TRAFFIC = {
     "scores": [],
     # one entry per captured workload
     "ca_fused": [
-        # 1.314 GB read + 0.127 GB written per launch (profiles/ca_fused_qwen7b_8k_t1024.md,
+        # 1.332 GB read + 0.127 GB written per launch (profiles/ca_fused_qwen7b_8k_t1024.md,
         # the CTA-pair kernel, whose source is ca_flash.cuh)
         {"files": ["ca_flash.cuh"], "kernel_hash": "066320b1977ebea0",
-         "bytes_per_launch": 1.4406e9, "workload": ("qwen7b_8k", 1024),
+         "bytes_per_launch": 1.4584e9, "workload": ("qwen7b_8k", 1024),
          "profile": "profiles/ca_fused_qwen7b_8k_t1024.md"},
         # the head-dim-256 kernel (source ca_pair.cu) captured on one KV-head of a 16k-token
-        # cache (1.233 GB read + 0.088 GB written, profiles/ca_pair_gemma_n16k_t655.md), scaled
+        # cache (1.237 GB read + 0.094 GB written, profiles/ca_pair_gemma_n16k_t655.md), scaled
         # by the units of a full-size launch (2 KV-heads x 131072 tokens: x16); its traffic (k
         # read once, X^T, partials) grows in proportion
-        {"files": ["ca_pair.cu"], "kernel_hash": "6eb62f16ac212d4e",
-         "bytes_per_launch": 16 * 1.3204e9, "workload": ("gemma_128k", 655),
+        {"files": ["ca_pair.cu"], "kernel_hash": "4eca71abd3f9e06a",
+         "bytes_per_launch": 16 * 1.3312e9, "workload": ("gemma_128k", 655),
          "profile": "profiles/ca_pair_gemma_n16k_t655.md"},
     ],
 }

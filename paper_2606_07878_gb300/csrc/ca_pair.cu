@@ -898,7 +898,7 @@ __global__ void __launch_bounds__(256, 3) ca_topk_repair_kernel(const TopkRepair
 }  // namespace
 
 cudaError_t launch_ca_topk_repair(const TopkRepairParams& f, int d2, cudaStream_t stream) {
-  if (f.D <= 0 || f.D % 8 != 0 || f.D > 2048 || f.d * 2 != d2 || f.t <= 0 || f.nb <= 0 ||
+  if (f.D <= 0 || f.D % 8 != 0 || f.d * 2 != d2 || f.t <= 0 || f.nb <= 0 ||
       f.N <= 0 || f.nsplit < 1 || f.nlists < 1 ||
       f.nlists * kTopK > 32 || f.tiles_k < f.nsplit || (int64_t)f.nb * f.t > 0x7fffffff ||
       (int64_t)f.tiles_k * f.keys_per_tile < f.N || f.q == nullptr || f.k == nullptr ||

@@ -112,12 +112,10 @@ __device__ __forceinline__ void pack_f32x16(const float* v, uint4 (&o)[4]) {
 }
 
 // General epilogue: v = acc * alpha [* colscale(c)] [* rowscale(r)] [+ bias(c)]
-//   -> [sum-of-squares partial] -> [GELU] -> [+ residual (split 0)] -> store (f32/bf16/hi-lo)
+//   -> [sum-of-squares partial] -> [GELU] -> [+ residual] -> store (f32/bf16/hi-lo)
 // colscale / rowscale are read from vectors of ready factors (see launch_inv_norms).
 // Sums of squares are written as partials, never accumulated atomically, so that results do
 // not depend on scheduling: per (vector, tile, half-warp) one slot, ss_parts slots per vector.
-// Split-K partial results go to out + split * split_stride and are reduced in a fixed order by
-// the consumer.
 // Host contract: csm, resm and (when vec_ok) om are contiguous in c (c0 == 1) with cdiv a
 // multiple of 32, so every 32-column chunk maps to 32 consecutive elements; ss_seg is a
 // multiple of the tile width.
@@ -149,7 +147,6 @@ struct EpiAffineT {
   // Vectors in blocks of ss_block consecutive indices, stored part-major (see launch_inv_norms),
   // so that a warp's 32 rows write 32 consecutive floats of one part.
   int64_t ss_block = 1;
-  int64_t split_stride = 0;
   int32_t vec_ok = 0;  // host: om.c0 == 1, cdiv % 32 == 0, 16-B aligned rows
   // OUT_F32 through TMA stores: the output is the 3-D view (col, row, batch) given to the
   // launcher (boxes of 32 x 32 fp32, 128-byte swizzled staging); rows / columns past the view
@@ -171,7 +168,7 @@ struct EpiAffineT {
   template <class Src>
   __device__ void prefetch(const GemmParams& p, const TileCoord& tc, int row, const Src& src,
                            int half) const {
-    if (res_kind == 0 || tc.split != 0) return;
+    if (res_kind == 0) return;
     const int r = tc.tm * kBM + row;
     if (r >= p.M) return;
     const int esz = res_kind == 1 ? 4 : 2;
@@ -211,7 +208,7 @@ struct EpiAffineT {
       }
       // Residual rows read coalesced by the whole warp. Not on the TMA-store path, whose
       // staging area may still be in use.
-      const bool res_vec = res_kind != 0 && tc.split == 0 && vec_ok && !tma_f32 && nv == 32;
+      const bool res_vec = res_kind != 0 && vec_ok && !tma_f32 && nv == 32;
       float resv[32];
       if (res_vec) {
         const int64_t o = resm.at(tc.b, r, c0);
@@ -268,7 +265,7 @@ struct EpiAffineT {
       if (res_vec) {
 #pragma unroll
         for (int e = 0; e < 32; ++e) v[e] += resv[e];
-      } else if (res_kind != 0 && tc.split == 0) {
+      } else if (res_kind != 0) {
         const int64_t o = resm.at(tc.b, r, c0);
         if (res_kind == 1) {
           const float* rp = static_cast<const float*>(res) + o;
@@ -285,7 +282,7 @@ struct EpiAffineT {
       if (tma_f32)
         store32_tma(tc, row, c0, v, stage, tmc);
       else
-        store32(p, tc.b, r, c0, v, tc.split, rvalid, stage);
+        store32(p, tc.b, r, c0, v, rvalid, stage);
     }
     if (!kChunkSums && sumsq != nullptr && rvalid) {
       const int c_tile = tc.tn * tile_cols_;
@@ -338,12 +335,11 @@ struct EpiAffineT {
 
   // Warp-collective on the vector path (every lane calls it; invalid rows store nothing).
   __device__ __forceinline__ void store32(const GemmParams& p, int b, int r, int c0,
-                                          const float (&v)[32], int split, bool rvalid,
+                                          const float (&v)[32], bool rvalid,
                                           uint4* stage) const {
     const bool full = vec_ok && (c0 + 32 <= max(p.N, pad_n));  // uniform across the warp
-    const int64_t so = (int64_t)split * split_stride;
     if (full) {
-      const int64_t o = om.at(b, r, c0) + so;
+      const int64_t o = om.at(b, r, c0);
       uint4 a4[4], b4[4];
       if (kind == OUT_F32) {
         float* dst = static_cast<float*>(out) + o;
@@ -370,7 +366,7 @@ struct EpiAffineT {
     for (int e = 0; e < 32; ++e) {
       const int c = c0 + e;
       if (c >= p.N) break;
-      const int64_t o = om.at(b, r, c) + so;
+      const int64_t o = om.at(b, r, c);
       if (kind == OUT_F32) {
         static_cast<float*>(out)[o] = v[e];
       } else if (kind == OUT_BF16) {

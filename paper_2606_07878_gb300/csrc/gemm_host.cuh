@@ -92,11 +92,9 @@ inline bool finalize_gemm(GemmParams& p, int ab_fmt) {
   }
   if ((p.a_k0 | p.a_k1 | p.b_k0 | p.b_k1) % 8 != 0) return false;
   p.iters_total = iters;
-  if (p.ksplit < 1) p.ksplit = 1;
-  if (p.ksplit > iters) p.ksplit = iters;
   p.tiles_m = (p.M + kBM - 1) / kBM;
   p.tiles_n = (p.N + BN - 1) / BN;
-  const int64_t nt = (int64_t)p.tiles_m * p.tiles_n * p.ksplit * p.batch;
+  const int64_t nt = (int64_t)p.tiles_m * p.tiles_n * p.batch;
   if (nt > 0x7fffffff) return false;
   p.ntiles = (int)nt;
   p.idesc = idesc_f16(kBM, BN, ab_fmt);
@@ -228,7 +226,7 @@ inline cudaError_t launch_split(const CUtensorMap& ta, const Operand2D& B, const
   CUtensorMap tb;
   if (!finalize_gemm<BN>(p, ab_fmt) || !make_tmap(&tb, B, BN)) return cudaErrorInvalidValue;
   epi.tile_cols_ = BN;
-  p.ksplit = ranks;
+  p.ranks = ranks;
   return launch_chained(tc_gemm_split_kernel<BN, Epi>, ranks * p.ntiles, gemm_threads<Epi>(),
                         GemmSmem<BN, Epi>::kBytes, stream, ranks, ta, tb, tc, p, epi);
 }

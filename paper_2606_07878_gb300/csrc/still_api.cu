@@ -238,7 +238,6 @@ GemmParams gp(int M, int N, int batch = 1, int bdiv = 1) {
   p.N = N;
   p.batch = batch;
   p.bdiv = bdiv;
-  p.ksplit = 1;
   return p;
 }
 

@@ -8,8 +8,9 @@
 // ~fp32 accuracy on bf16 tensor cores (a_hi b_hi + a_hi b_lo + a_lo b_hi).
 //
 // CTA = 2 + Epi::kWarps warps: warp 0 issues TMA, warp 1 owns TMEM and issues tcgen05.mma
-// (one thread), the rest run the epilogue from TMEM (Epi::kWarps / 4 per lane quarter). The accumulator is double-buffered in TMEM
-// (2 x BN fp32 columns), so a tile's epilogue overlaps the next tile's main loop.
+// (one thread), the rest run the epilogue from TMEM (Epi::kWarps / 4 per lane quarter). The
+// accumulator is double-buffered in TMEM (2 x BN fp32 columns), so a tile's epilogue overlaps the
+// next tile's main loop.
 // Tiles are 128 x BN; the grid is persistent (tile += gridDim.x), m-tiles fastest so that
 // CTAs running together share B tiles through L2.
 #pragma once
@@ -40,7 +41,7 @@ struct GemmParams {
   int64_t b_r1, b_r0, b_k1, b_k0;
   int32_t npass;
   GemmPass pass[3];
-  int32_t ksplit;  // split-K factor (each split = a contiguous range of K iterations)
+  int32_t ranks;   // CTAs per tile (tc_gemm_split_kernel)
   // Derived by the host launcher.
   int32_t tiles_m, tiles_n, iters_total, ntiles;
   uint32_t idesc;
@@ -48,24 +49,29 @@ struct GemmParams {
 };
 
 struct TileCoord {
-  int b, tm, tn, split;
+  int b, tm, tn;
 };
 
 __device__ __forceinline__ TileCoord decode_tile(const GemmParams& p, int tile) {
   TileCoord c;
   c.tm = tile % p.tiles_m;
   int r = tile / p.tiles_m;
-  c.split = r % p.ksplit;
-  r /= p.ksplit;
   c.tn = r % p.tiles_n;
   c.b = r / p.tiles_n;
   return c;
 }
 
-__device__ __forceinline__ void split_range(const GemmParams& p, int split, int& it0, int& it1) {
-  it0 = (int)(((int64_t)p.iters_total * split) / p.ksplit);
-  it1 = (int)(((int64_t)p.iters_total * (split + 1)) / p.ksplit);
-}
+// Walks the K iterations of a tile: pass and K offset inside it of iteration `it` (ascending).
+struct PassWalk {
+  int pass = 0, base = 0;
+  __device__ __forceinline__ int offset(const GemmParams& p, int it) {
+    while (pass < p.npass - 1 && it >= base + p.pass[pass].klen / kBK) {
+      base += p.pass[pass].klen / kBK;
+      ++pass;
+    }
+    return (it - base) * kBK;
+  }
+};
 
 // Per-epilogue-warp staging area (1024-byte aligned): 32 rows x 64 B for the LSU path (rows
 // 80 B apart), or one TMA-store box of up to 4 KB.
@@ -146,8 +152,9 @@ struct TmemTile {
 //                    is ready) and  operator()(p, tc, row_in_tile, src, half, warp_stage, out_map)
 // where src (TmemTile, or SplitTile below) holds the accumulator and names the chunks of this
 // warp; the functor loads them and stores its own results.
-// kRole only names the instantiation (one per GEMM of the launch sequence) so that profilers
-// can tell the GEMMs apart; it does not change the code.
+// kRole only names the instantiation, so that profilers can tell the GEMMs of the launch sequence
+// apart; it does not change the code. The split and pair forms below have one instantiation per
+// epilogue for all GEMMs: a profile tells those apart by their order in the sequence.
 template <int BN, class Epi, int kRole>
 __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
@@ -209,16 +216,10 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
         const int64_t ak = bo * p.a_k1 + bi * p.a_k0;
         const int64_t br = bo * p.b_r1 + bi * p.b_r0 + (int64_t)tc.tn * BN;
         const int64_t bk = bo * p.b_k1 + bi * p.b_k0;
-        int it0, it1;
-        split_range(p, tc.split, it0, it1);
-        int pass = 0, base = 0;
-        for (int it = it0; it < it1; ++it) {
-          while (pass < p.npass - 1 && it >= base + p.pass[pass].klen / kBK) {
-            base += p.pass[pass].klen / kBK;
-            ++pass;
-          }
-          const GemmPass& ps = p.pass[pass];
-          const int kk = (it - base) * kBK;
+        PassWalk walk;
+        for (int it = 0; it < p.iters_total; ++it) {
+          const int kk = walk.offset(p, it);
+          const GemmPass& ps = p.pass[walk.pass];
           if (!mbar_wait(&empty[stage], phase ^ 1)) {
             dev_set_error(p.err, DEV_WAIT_TIMEOUT, 100);
             *abort_flag = 1;
@@ -254,8 +255,6 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
       bool issued = false;
       for (int tile = blockIdx.x; tile < p.ntiles && !*abort_flag; tile += gridDim.x) {
         const TileCoord tc = decode_tile(p, tile);
-        int it0, it1;
-        split_range(p, tc.split, it0, it1);
         if (!mbar_wait(&tempty[acc], acc_phase ^ 1)) {
           dev_set_error(p.err, DEV_WAIT_TIMEOUT, 101);
           *abort_flag = 1;
@@ -263,7 +262,7 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
-        for (int it = it0; it < it1; ++it) {
+        for (int it = 0; it < p.iters_total; ++it) {
           if (!mbar_wait(&full[stage], phase)) {
             dev_set_error(p.err, DEV_WAIT_TIMEOUT, 102);
             *abort_flag = 1;
@@ -275,7 +274,7 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
           const uint64_t bd = sdesc_k_sw128(sa + S::kABytes);
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k)
-            tc_mma_f16(d_tmem, ad + 2 * k, bd + 2 * k, p.idesc, (it > it0 || k > 0) ? 1u : 0u);
+            tc_mma_f16(d_tmem, ad + 2 * k, bd + 2 * k, p.idesc, (it > 0 || k > 0) ? 1u : 0u);
           issued = true;
           tc_commit(&empty[stage]);
           if (++stage == kStages) {
@@ -413,7 +412,7 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
   const bool leader = x == 0;
   const uint16_t pair_mask = (uint16_t)((1u << rank) | (1u << (rank ^ 1u)));
   const int cid = (int)cluster_id_x(), ncl = (int)cluster_count_x();
-  const int npairs = ((p.tiles_m + 1) / 2) * p.tiles_n * p.ksplit * p.batch;
+  const int npairs = ((p.tiles_m + 1) / 2) * p.tiles_n * p.batch;
   // the 2-SM instruction descriptor: M = 256
   const uint32_t idesc2 = (p.idesc & ~(0x1Fu << 24)) | ((uint32_t)(2 * kBM >> 4) << 24);
 
@@ -458,16 +457,10 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
         const int64_t ak = bo * p.a_k1 + bi * p.a_k0;
         const int64_t br = bo * p.b_r1 + bi * p.b_r0 + (int64_t)tc.tn * BN + (BN / 2) * x;
         const int64_t bk = bo * p.b_k1 + bi * p.b_k0;
-        int it0, it1;
-        split_range(p, tc.split, it0, it1);
-        int pass = 0, base = 0;
-        for (int it = it0; it < it1; ++it) {
-          while (pass < p.npass - 1 && it >= base + p.pass[pass].klen / kBK) {
-            base += p.pass[pass].klen / kBK;
-            ++pass;
-          }
-          const GemmPass& ps = p.pass[pass];
-          const int kk = (it - base) * kBK;
+        PassWalk walk;
+        for (int it = 0; it < p.iters_total; ++it) {
+          const int kk = walk.offset(p, it);
+          const GemmPass& ps = p.pass[walk.pass];
           if (!mbar_wait(&empty[stage], phase ^ 1)) {
             dev_set_error(p.err, DEV_WAIT_TIMEOUT, 104);
             *abort_flag = 1;
@@ -517,8 +510,6 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
       bool issued = false;
       for (int tile = cid; tile < npairs && !*abort_flag; tile += ncl) {
         const TileCoord tc = decode_tile2(p, tile, x);
-        int it0, it1;
-        split_range(p, tc.split, it0, it1);
         if (!mbar_wait_cluster(&tempty[acc], acc_phase ^ 1)) {
           dev_set_error(p.err, DEV_WAIT_TIMEOUT, 106);
           *abort_flag = 1;
@@ -526,7 +517,7 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
-        for (int it = it0; it < it1; ++it) {
+        for (int it = 0; it < p.iters_total; ++it) {
           if (!mbar_wait_cluster(&full[stage], phase)) {
             dev_set_error(p.err, DEV_WAIT_TIMEOUT, 107);
             *abort_flag = 1;
@@ -538,7 +529,7 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
           const uint64_t bd = sdesc_k_sw128(sa + S::kABytes);
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k)
-            tc_mma_f16_2sm(d_tmem, ad + 2 * k, bd + 2 * k, idesc2, (it > it0 || k > 0) ? 1u : 0u);
+            tc_mma_f16_2sm(d_tmem, ad + 2 * k, bd + 2 * k, idesc2, (it > 0 || k > 0) ? 1u : 0u);
           issued = true;
           tc_commit_2sm_mc(&empty[stage], pair_mask);
           if (++stage == kStages) {
@@ -685,7 +676,7 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  const int rank = (int)cluster_ctarank(), ranks = p.ksplit;
+  const int rank = (int)cluster_ctarank(), ranks = p.ranks;
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&full[s], 1);
@@ -713,7 +704,6 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
     tc.tm = tile % p.tiles_m;
     tc.tn = (tile / p.tiles_m) % p.tiles_n;
     tc.b = tile / p.tiles_m / p.tiles_n;
-    tc.split = 0;  // the epilogue sees whole sums
   }
   const int it0 = p.iters_total * rank / ranks, it1 = p.iters_total * (rank + 1) / ranks;
   const int quarter = warp & 3;
@@ -728,16 +718,13 @@ __global__ void __launch_bounds__(gemm_threads<Epi>(), 1)
       const int64_t ak = bo * p.a_k1 + bi * p.a_k0;
       const int64_t br = bo * p.b_r1 + bi * p.b_r0 + (int64_t)tc.tn * BN;
       const int64_t bk = bo * p.b_k1 + bi * p.b_k0;
-      int stage = 0, pass = 0, base = 0;
+      int stage = 0;
       uint32_t phase = 0;
       int sent = 0;
+      PassWalk walk;
       for (int it = it0; it < it1; ++it) {
-        while (pass < p.npass - 1 && it >= base + p.pass[pass].klen / kBK) {
-          base += p.pass[pass].klen / kBK;
-          ++pass;
-        }
-        const GemmPass& ps = p.pass[pass];
-        const int kk = (it - base) * kBK;
+        const int kk = walk.offset(p, it);
+        const GemmPass& ps = p.pass[walk.pass];
         if (!mbar_wait(&empty[stage], phase ^ 1)) {
           dev_set_error(p.err, DEV_WAIT_TIMEOUT, 110);
           *abort_flag = 1;
