@@ -692,8 +692,9 @@ inline cudaError_t launch_ca_flash(const KernelTable& dev, const Operand2D& Q, c
 
 // 2d = 512 (head dim 256): the same computation on clusters of four CTAs, two query tiles x
 // two column halves; the CTAs of a query tile split the O columns and take turns computing S,
-// the two CTAs of a half run their MMAs as one 2-SM MMA over both query tiles (ca_pair.cu). Q, K as for launch_ca_flash;
-// XT: [H*512][2*Np] fp16 (hi | lo). f.nunits counts (query-tile pair, key split, batch) units.
+// the two CTAs of a half run their MMAs as one 2-SM MMA over both query tiles (ca_pair.cu). Q, K
+// as for launch_ca_flash; XT: [H*512][2*Np] fp16 (hi | lo). f.nunits counts (query-tile pair, key
+// split, batch) units.
 // one_pass: q, k as fp16 hi | lo with S from the hi parts only (one MMA pass) and repair
 // candidates in f.cand_key / f.cand_c for ca_topk_repair; else 3-pass split-bf16 scores.
 cudaError_t launch_ca_pair(const KernelTable& dev, const Operand2D& Q, const Operand2D& K,

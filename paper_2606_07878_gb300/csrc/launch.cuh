@@ -8,8 +8,9 @@ namespace still {
 // cluster > 1. It begins when the CTAs of the stream's previous kernel have exited, before that
 // kernel's completion has passed through the stream: its launch and its set-up (barriers, TMEM,
 // tensor map fetches) lie under the previous kernel's end. What bounds a call on a short sequence
-// is these gaps, 21 of them: 1,024 tokens of 2 heads of 64 channels 188 -> 144 us, three windows
-// of 1,024 in the lookahead call 1099 -> 858 us, 1,837 tokens with biases 1153 -> 1103 us. Letting
+// is these gaps, 20 launches of a one-block layer and 34 of two blocks without FFN: 1,024 tokens of
+// 2 heads of 64 channels 188 -> 144 us, three windows of 1,024 in the lookahead call 1099 -> 858 us,
+// 8,003 tokens with biases 1153 -> 1103 us. Letting
 // the next kernel begin earlier still (griddepcontrol.launch_dependents at a kernel's head) puts
 // its idle CTAs beside the working ones: 164, 921 and 1202 us, and the 32,768-token layer
 // slower than unchained (5389 against 5225 us); behind a kernel's last tile it changes nothing.

@@ -358,15 +358,16 @@ int wide_parts(int64_t D) { return (int)(D / 32); }
 size_t sumsq_bytes(int64_t vectors, int parts) { return a256(4 * vectors * (parts + 1)); }
 
 // The cross-attention scores of a one-block layer of head dim 256 (the kernel on clusters of
-// two CTAs) take one fp16 MMA pass (q_hi . k_hi) instead of three split-bf16 passes, and a
+// four CTAs) take one fp16 MMA pass (q_hi . k_hi) instead of three split-bf16 passes, and a
 // repair kernel then recomputes the logits of each row's heaviest keys from the fp16 hi | lo
 // operands (about 22 bits). At d_l >= 512 the rows put nearly all their weight on a few
 // keys: CPU emulation of the C_k error from the cross-attention logits alone, with the k
 // heaviest keys of every row repaired, gives 5.1e-4 (k = 8) and 1.5e-5 (k = 16) on the Gemma
 // shape at 16k tokens, against 3.7e-3 for the three-pass split. Head dims 64 and 128 keep the
-// split: there one CTA runs the softmax of every tile, a one-pass S tile takes no longer than
-// that softmax, and the kernel measured slower with one pass (the Qwen-7B-shaped stack went
-// from 76 to 109 ms, with 24 ms of repair).
+// split. One pass was measured slower there on an earlier form, one CTA per query tile whose
+// one-pass S tile took no longer than its softmax, with a repair three times slower than today's
+// (the Qwen-7B-shaped stack 76 -> 109 ms, 24 ms of it repair); on the CTA pairs it has not been
+// measured.
 bool one_pass_scores(const still_layer_config& c) {
   return c.n_blocks == 1 && c.head_dim == 256 && c.d_latent >= 512 && c.d_latent <= 2048;
 }

@@ -3,8 +3,12 @@
 Small enough for kernel captures (one layer's weights and workspace, a few GB; --N and --H shrink
 a large workload's cache while keeping its compactor shape), e.g.
 
-  ncu --set full --clock-control none --kernel-name-base mangled -k regex:EpiAffineELi4E \\
-      -s 1 -c 1 -o prof python -m paper_2606_07878_gb300.profile_layer --workload qwen7b_8k
+  ncu --set full --clock-control none -k regex:key_proj_kernel -s 1 -c 1 -o prof \\
+      python -m paper_2606_07878_gb300.profile_layer --workload qwen7b_8k
+
+The GEMMs that split K or run on CTA pairs have one kernel per epilogue and tile width for all
+sublayers: pick one by its place in the launch sequence (-s), after a run with
+--metrics gpu__time_duration.sum -k regex:gemm.
 
 Exits non-zero if the device reports an error.
 """
